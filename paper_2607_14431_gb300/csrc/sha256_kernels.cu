@@ -268,60 +268,187 @@ __device__ __forceinline__ void store_state(uint32_t *out, const uint32_t st[8])
 }
 
 // ---- two-warp form, for launches too small to fill the GPU ---------------
-// When there are few chains, each one's latency decides, and a thread that
-// both expands the message schedule and runs the rounds issues ~27
-// instructions a round from one warp.  Here a 64-thread CTA works on 32
-// chains (lane c of both warps on chain c): warp 1 loads each chain's next
-// 64-byte block, expands its schedule and leaves K[t] + W[t] in shared
-// memory; warp 0 runs the 64 rounds from there.  The rounds' warp then
-// issues ~18 instructions a round on its own scheduler: ~1,775 cycles per
-// block against ~2,480 (a probe over 256 blocks per chain, same digests).
-// Two buffers change hands through named barriers: 1 + b (buffer b full,
-// warp 1 arrives, warp 0 waits) and 3 + b (buffer b free again, warp 0
-// arrives, warp 1 waits).  Both warps run the same number of blocks, with
-// every lane taking part (lanes past the last chain hash zeros and store
-// nothing), so every arrival meets its wait.
-constexpr int kSplitChains = 32;
+// When there are few chains, each one's latency decides.  Two warps of a
+// 64-thread CTA share the work: one loads the message, expands the schedule
+// and leaves K[t] + W[t] in shared memory, the other runs the rounds.
+//
+// A compression's 64 rounds are one recurrence with two halves: e[t+1] needs
+// a[t-3], four rounds old, and a[t+1] = (e[t+1] - a[t-3]) + S0(a[t]) + maj.  So
+// a chain takes two lanes: lane c (c < 16) runs the e half at round t while
+// lane c + 16 runs the a half two rounds behind, and one shuffle per round
+// (each lane's new word to its partner, used two rounds later, so its latency
+// is hidden) carries both couplings.  Both halves are the same instructions
+// with per-lane rotation amounts: new = rotr(x, r1) ^ rotr(x, r2) ^ rotr(x, r3)
+// + choose + in, where maj(a, b, c) is b where a and b agree and c elsewhere,
+// i.e. a choose whose selector is ~(a ^ b).  What bounds it is the latency of
+// rotation, xor and addition, one after the other, once a round; a lane that
+// runs both halves adds twice their ALU work to it.  A lone chain takes 0.74
+// us per 64-byte block against 0.84 with both halves in one lane (and 1.46 in
+// one warp), the digests of 64 leaves 70 us against 77.  The loading warp's
+// half-warps take one block each, so a hand-over is a pair of blocks; the a
+// lanes read zeros for their K + W.
+//
+// The wide form runs both halves in one lane, 32 chains per CTA, a block per
+// hand-over: a leaf launch of 33 to 64 leaves per SM takes it, where four CTAs
+// of the other would put a loading warp beside every rounds' warp on its
+// scheduler (64 leaves per SM: 76 us wide, 92 with two lanes, 109 in one warp).
+//
+// Two buffers change hands through named barriers: 1 + b (buffer b full: the
+// loading warp arrives, the rounds' warp waits) and 3 + b (buffer b free
+// again: the rounds' warp arrives, the loading warp waits).  Both warps run
+// the same number of hand-overs, with every lane taking part (lanes past the
+// last chain hash zeros and store nothing), so every arrival meets its wait.
+constexpr int kSplitChains = 16;
+constexpr int kWideChains = 32;
+
+struct __align__(16) SplitShared {
+    // [buffer][block of the pair, or upper half of the wide form's chains]
+    // [t / 4][chain], 4 consecutive t each
+    uint4 kw[2][2][16][kSplitChains];
+    uint4 zero[16][kSplitChains];      // what the a lanes read
+    int consumer;                      // which of the two warps runs the rounds
+};
 
 __device__ __forceinline__ void bar_sync_pair(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 __device__ __forceinline__ void bar_arrive_pair(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
 
-// Warp 1: the message schedule of block w plus the round constants, into
-// column `lane` of kw[64][32] (plain ALU arithmetic: this warp's scheduler
-// has nothing else to issue).
-__device__ __forceinline__ void split_expand(uint32_t (*kw)[kSplitChains], uint32_t w[16], int lane) {
+// The loading warp: the message schedule of block w plus the round constants, into
+// column c of kw[16][kSplitChains].  Additions and plain shifts go to the FMA
+// pipe (fadd, fshr), which leaves the ALU pipe to a rounds' warp on the same
+// scheduler.
+__device__ __forceinline__ void split_expand(uint4 (*kw)[kSplitChains], uint32_t w[16], int c, uint32_t one) {
 #pragma unroll
-    for (int t = 0; t < 64; ++t) {
-        uint32_t wt;
-        if (t < 16) {
-            wt = w[t];
-        } else {
-            const uint32_t w15 = w[(t - 15) & 15], w2 = w[(t - 2) & 15];
-            const uint32_t s0 = rotr(w15, 7) ^ rotr(w15, 18) ^ (w15 >> 3);
-            const uint32_t s1 = rotr(w2, 17) ^ rotr(w2, 19) ^ (w2 >> 10);
-            wt = w[t & 15] = w[t & 15] + s0 + w[(t - 7) & 15] + s1;
+    for (int t4 = 0; t4 < 16; ++t4) {
+        uint32_t v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int t = 4 * t4 + i;
+            uint32_t wt;
+            if (t < 16) {
+                wt = w[t];
+            } else {
+                const uint32_t w15 = w[(t - 15) & 15], w2 = w[(t - 2) & 15];
+                const uint32_t s0 = rotr(w15, 7) ^ rotr(w15, 18) ^ fshr<3>(w15, one);
+                const uint32_t s1 = rotr(w2, 17) ^ rotr(w2, 19) ^ fshr<10>(w2, one);
+                wt = w[t & 15] = fadd(fadd(fadd(w[t & 15], w[(t - 7) & 15], one), s0, one), s1, one);
+            }
+            v[i] = fadd(wt, kK[t], one);
         }
-        kw[t][lane] = wt + kK[t];
+        kw[t4][c] = make_uint4(v[0], v[1], v[2], v[3]);
     }
 }
 
-// Warp 0: the 64 rounds of one block from kw (FIPS 180-4 sec. 6.2.2 step 3,
-// with h + K[t] + W[t] taken whole from shared memory) and the feed-forward.
-// The additions off the last step go to the FMA pipe (fadd), so the ALU pipe
-// carries the rotations and logic.
-__device__ __forceinline__ void split_rounds(uint32_t st[8], const uint32_t (*kw)[kSplitChains], int lane,
-                                             uint32_t one) {
+// The rounds' warp, per lane: which half of the recurrence it runs.
+struct SplitRole {
+    int r1, r2, r3;   // rotations of its sum function
+    uint32_t sign;    // 1 (e: + h) or -1 (a: - d), as a factor
+    uint32_t agree;   // 0 (choose by x) or ~0 (by ~(x ^ y))
+    bool a;
+};
+__device__ __forceinline__ SplitRole split_role(int lane) {
+    const bool a = lane >= kSplitChains;
+    return SplitRole{a ? 2 : 6, a ? 13 : 11, a ? 22 : 25, a ? 0xffffffffu : 1u, a ? 0xffffffffu : 0u, a};
+}
+
+// The rounds' warp: the 64 rounds of one block (FIPS 180-4 sec. 6.2.2 step 3) and the
+// feed-forward.  st is the lane's half of the state: e, f, g, h or a, b, c, d.
+// At step s the e lanes run round s and the a lanes round s - 2: in the
+// first two steps the a lanes only bring b and a into their window (which
+// starts as c, d), and after step 63 the e lanes' steps are ignored.
+__device__ __forceinline__ void split_rounds(uint32_t st[4], const uint4 *kw, const SplitRole &ro, uint32_t one) {
+    uint32_t p1 = ro.a ? st[2] : st[0], p2 = ro.a ? st[3] : st[1], p3 = st[2], p4 = st[3];
+    // the partner's words of two steps ago; before step 0: the e lanes get d, then c
+    uint32_t sh0 = __shfl_xor_sync(0xffffffffu, st[3], kSplitChains);
+    uint32_t sh1 = __shfl_xor_sync(0xffffffffu, st[2], kSplitChains);
+    uint32_t e1 = 0, e2 = 0, e3 = 0, e4 = 0;
+    uint4 k4 = make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int s = 0; s < 66; ++s) {
+        if (s < 64 && (s & 3) == 0) k4 = kw[(s >> 2) * kSplitChains];
+        const uint32_t k = s >= 64 ? 0u : (s & 3) == 0 ? k4.x : (s & 3) == 1 ? k4.y : (s & 3) == 2 ? k4.z : k4.w;
+        uint32_t q;  // h + K[t] + W[t], or -d
+        asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(q) : "r"(p4), "r"(ro.sign), "r"(k));
+        const uint32_t in = fadd(sh0, q, one);
+        const uint32_t S = __funnelshift_r(p1, p1, ro.r1) ^ __funnelshift_r(p1, p1, ro.r2) ^
+                           __funnelshift_r(p1, p1, ro.r3);
+        const uint32_t sel = p1 ^ (~p2 & ro.agree);
+        const uint32_t ch = (sel & p2) ^ (~sel & p3);
+        uint32_t n = S + ch + in;
+        if (s == 0) n = ro.a ? st[1] : n;
+        if (s == 1) n = ro.a ? st[0] : n;
+        sh0 = sh1;
+        if (s < 64) sh1 = __shfl_xor_sync(0xffffffffu, n, kSplitChains);
+        p4 = p3;
+        p3 = p2;
+        p2 = p1;
+        p1 = n;
+        if (s == 63) {
+            e1 = p1;
+            e2 = p2;
+            e3 = p3;
+            e4 = p4;
+        }
+    }
+    st[0] += ro.a ? p1 : e1;
+    st[1] += ro.a ? p2 : e2;
+    st[2] += ro.a ? p3 : e3;
+    st[3] += ro.a ? p4 : e4;
+}
+
+// Both warps, before their loops: the zeros of the a lanes, and which warp
+// does what (true: this one loads and expands).  A CTA's two warps sit on
+// neighbouring schedulers, so with warp 0 always running the rounds, four
+// CTAs on an SM would put their rounds on two of the four schedulers (105
+// instead of 90 us at 64 leaves per SM); every other pair of warp slots swaps
+// the roles instead.  The slot number is only read here, by one thread.
+__device__ __forceinline__ bool split_begin(SplitShared &sm) {
+    for (int i = threadIdx.x; i < 16 * kSplitChains; i += 64) (&sm.zero[0][0])[i] = make_uint4(0, 0, 0, 0);
+    if (threadIdx.x == 0) {
+        uint32_t slot;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
+        sm.consumer = (int)((slot >> 2) & 1);
+    }
+    __syncthreads();
+    return (int)(threadIdx.x >> 5) != sm.consumer;
+}
+
+// The rounds' warp over a chain of n_blocks blocks: its half of the state from H0
+// to the digest.
+__device__ __forceinline__ void split_consume(uint32_t st[4], const SplitShared &sm, int n_blocks, int lane,
+                                              uint32_t one) {
+    const SplitRole ro = split_role(lane);
+    const int c = lane & (kSplitChains - 1);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) st[i] = ro.a ? kH0[i] : kH0[4 + i];
+    const int n_pairs = (n_blocks + 1) >> 1;
+    for (int k = 0; k < n_pairs; ++k) {
+        const int buf = k & 1;
+        bar_sync_pair(1 + buf);
+#pragma unroll 1
+        for (int h = 0; h < 2 && 2 * k + h < n_blocks; ++h)
+            split_rounds(st, ro.a ? &sm.zero[0][c] : &sm.kw[buf][h][0][c], ro, one);
+        if (k + 2 < n_pairs) bar_arrive_pair(3 + buf);
+    }
+}
+
+// The wide form's rounds of one block: both halves of the state in one lane.
+// The additions off the last step go to the FMA pipe (fadd): e[t+1] is one
+// addition behind S1(e[t]) and a[t+1] = e[t+1] + S0 + (maj - d) one behind that.
+__device__ __forceinline__ void wide_rounds(uint32_t st[8], const uint4 *kw, uint32_t one) {
     uint32_t a = st[0], b = st[1], c = st[2], d = st[3], e = st[4], f = st[5], g = st[6], h = st[7];
+    uint4 k4 = make_uint4(0, 0, 0, 0);
 #pragma unroll
     for (int t = 0; t < 64; ++t) {
-        const uint32_t k = kw[t][lane];
+        if ((t & 3) == 0) k4 = kw[(t >> 2) * kSplitChains];
+        const uint32_t k = (t & 3) == 0 ? k4.x : (t & 3) == 1 ? k4.y : (t & 3) == 2 ? k4.z : k4.w;
         const uint32_t S1 = rotr(e, 6) ^ rotr(e, 11) ^ rotr(e, 25);
         const uint32_t ch = (e & f) ^ (~e & g);
         const uint32_t S0 = rotr(a, 2) ^ rotr(a, 13) ^ rotr(a, 22);
         const uint32_t maj = (a & b) ^ (a & c) ^ (b & c);
-        const uint32_t hkc = fadd(fadd(h, k, one), ch, one);  // h + K[t] + W[t] + Ch
-        const uint32_t T1 = fadd(hkc, S1, one);
-        const uint32_t ne = fadd(fadd(d, hkc, one), S1, one);  // d + T1
+        const uint32_t y = fadd(fadd(fadd(h, k, one), d, one), ch, one);
+        uint32_t md;  // maj - d
+        asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(md) : "r"(d), "r"(0u - one), "r"(maj));
+        const uint32_t ne = S1 + y;
         h = g;
         g = f;
         f = e;
@@ -329,7 +456,7 @@ __device__ __forceinline__ void split_rounds(uint32_t st[8], const uint32_t (*kw
         d = c;
         c = b;
         b = a;
-        a = T1 + S0 + maj;
+        a = ne + S0 + md;
     }
     st[0] += a;
     st[1] += b;
@@ -341,23 +468,24 @@ __device__ __forceinline__ void split_rounds(uint32_t st[8], const uint32_t (*kw
     st[7] += h;
 }
 
-// Warp 0's side of a chain of n_blocks blocks: state from H0 to the digest.
-__device__ __forceinline__ void split_consume(uint32_t st[8], uint32_t (*kw)[64][kSplitChains], int n_blocks,
-                                              int lane, uint32_t one) {
+// The rounds' warp of the wide form over a chain of n_blocks blocks.
+__device__ __forceinline__ void wide_consume(uint32_t st[8], const SplitShared &sm, int n_blocks, int lane,
+                                             uint32_t one) {
     init_state(st);
-    for (int blk = 0; blk < n_blocks; ++blk) {
-        const int buf = blk & 1;
+    for (int k = 0; k < n_blocks; ++k) {
+        const int buf = k & 1;
         bar_sync_pair(1 + buf);
-        split_rounds(st, kw[buf], lane, one);
-        if (blk + 2 < n_blocks) bar_arrive_pair(3 + buf);
+        wide_rounds(st, &sm.kw[buf][lane / kSplitChains][0][lane & (kSplitChains - 1)], one);
+        if (k + 2 < n_blocks) bar_arrive_pair(3 + buf);
     }
 }
 
-// Warp 1 hands over block blk (its 16 words in w) through buffer blk & 1.
-__device__ __forceinline__ void split_hand_over(uint32_t (*kw)[64][kSplitChains], uint32_t w[16], int blk, int lane) {
-    const int buf = blk & 1;
-    if (blk >= 2) bar_sync_pair(3 + buf);
-    split_expand(kw[buf], w, lane);
+// A lane of the loading warp hands over its block of pair (wide form: its
+// chain's block) k, 16 words in w, through buffer k & 1.
+__device__ __forceinline__ void split_hand_over(SplitShared &sm, uint32_t w[16], int k, int lane, uint32_t one) {
+    const int buf = k & 1;
+    if (k >= 2) bar_sync_pair(3 + buf);
+    split_expand(sm.kw[buf][lane / kSplitChains], w, lane & (kSplitChains - 1), one);
     __threadfence_block();
     bar_arrive_pair(1 + buf);
 }
@@ -372,33 +500,37 @@ __device__ __forceinline__ void padding_block(uint32_t w[16], uint64_t bytes) {
     w[15] = (uint32_t)bits;
 }
 
-// Warp 1's side of a whole 4 KiB leaf at v (nullptr: zeros), also written to
-// o when COPY (the bytes written are the bytes hashed): 64 data blocks, the
-// next two in flight, then the padding block.
-template <bool COPY>
-__device__ __forceinline__ void split_produce_leaf(uint32_t (*kw)[64][kSplitChains], const uint4 *v, uint4 *o,
-                                                   int lane) {
-    constexpr int kData = (int)(kLeafBytes / 64);
+// The loading warp over a whole 4 KiB leaf at v (nullptr: zeros), also written
+// to o when COPY (the bytes written are the bytes hashed): 32 pairs of data
+// blocks (wide form: 64 blocks), the next two in flight, then the padding
+// block.
+template <bool COPY, bool WIDE>
+__device__ __forceinline__ void split_produce_leaf(SplitShared &sm, const uint4 *v, uint4 *o, int lane,
+                                                   uint32_t one) {
+    constexpr int kStep = WIDE ? 4 : 8;  // vectors of the leaf per hand-over
+    constexpr int kHandOvers = (int)(kLeafBytes / 16) / kStep;
+    if (!WIDE && v) v += 4 * (lane / kSplitChains);
+    if (!WIDE && COPY && o) o += 4 * (lane / kSplitChains);
     uint4 n1[4], n2[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         n1[q] = v ? __ldg(v + q) : make_uint4(0, 0, 0, 0);
-        n2[q] = v ? __ldg(v + 4 + q) : make_uint4(0, 0, 0, 0);
+        n2[q] = v ? __ldg(v + kStep + q) : make_uint4(0, 0, 0, 0);
     }
-    for (int blk = 0; blk < kData; ++blk) {
+    for (int k = 0; k < kHandOvers; ++k) {
         uint4 x[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             x[q] = n1[q];
             n1[q] = n2[q];
         }
-        if (v && blk + 2 < kData) {
+        if (v && k + 2 < kHandOvers) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) n2[q] = __ldg(v + 4 * (blk + 2) + q);
+            for (int q = 0; q < 4; ++q) n2[q] = __ldg(v + kStep * (k + 2) + q);
         }
         if (COPY && o) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) __stcs(o + 4 * blk + q, x[q]);
+            for (int q = 0; q < 4; ++q) __stcs(o + kStep * k + q, x[q]);
         }
         uint32_t w[16];
 #pragma unroll
@@ -408,53 +540,91 @@ __device__ __forceinline__ void split_produce_leaf(uint32_t (*kw)[64][kSplitChai
             w[4 * q + 2] = bswap(x[q].z);
             w[4 * q + 3] = bswap(x[q].w);
         }
-        split_hand_over(kw, w, blk, lane);
+        split_hand_over(sm, w, k, lane, one);
     }
     uint32_t w[16];
     padding_block(w, kLeafBytes);
-    split_hand_over(kw, w, kData, lane);
+    split_hand_over(sm, w, kHandOvers, lane, one);
 }
 
 constexpr int kSplitLeafBlocks = (int)(kLeafBytes / 64) + 1;
 
+// The rounds' warp over whole 4 KiB leaves: the chain's digest to out (null:
+// nothing; zero: zeros instead).
+template <bool WIDE>
+__device__ __forceinline__ void split_consume_leaf(SplitShared &sm, uint32_t *out, bool zero, int lane, uint32_t one) {
+    if (WIDE) {
+        uint32_t st[8];
+        wide_consume(st, sm, kSplitLeafBlocks, lane, one);
+        if (!out) return;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) st[w] = zero ? 0u : st[w];
+        store_state(out, st);
+    } else {
+        uint32_t st[4];  // words 0-3 (a lanes) or 4-7
+        split_consume(st, sm, kSplitLeafBlocks, lane, one);
+        if (!out) return;
+        reinterpret_cast<uint4 *>(out)[lane >= kSplitChains ? 0 : 1] =
+            zero ? make_uint4(0, 0, 0, 0) : make_uint4(st[0], st[1], st[2], st[3]);
+    }
+}
+
+// The chain of a lane of either warp, within the CTA.
+template <bool WIDE>
+__device__ __forceinline__ int64_t split_chain(int lane) {
+    return WIDE ? (int64_t)blockIdx.x * kWideChains + lane
+                : (int64_t)blockIdx.x * kSplitChains + (lane & (kSplitChains - 1));
+}
+
+// The whole state in an e lane of the rounds' warp (all lanes take part).
+__device__ __forceinline__ void split_whole_state(uint32_t full[8], const uint32_t st[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        full[i] = __shfl_xor_sync(0xffffffffu, st[i], kSplitChains);
+        full[4 + i] = st[i];
+    }
+}
+
 // graft_verify_kernel's work in the two-warp form, for pages made of whole
-// 4 KiB leaves and launches of at most one such CTA per SM.
+// 4 KiB leaves and launches of a few such CTAs per SM.
+template <bool WIDE>
 __global__ void __launch_bounds__(64) graft_verify_split_kernel(const GraftParams p, int64_t leaves_per_page,
                                                                 uint32_t *__restrict__ out, uint32_t one) {
-    __shared__ __align__(16) uint32_t kw[2][64][kSplitChains];
+    __shared__ SplitShared sm;
+    const bool produce = split_begin(sm);
     graft_metadata(p);
     const int lane = threadIdx.x & 31;
     const uint64_t page_bytes = p.page_bytes;
     const int64_t n_leaves = (int64_t)p.n_layers * 2 * p.npb * leaves_per_page;
-    const int64_t idx = (int64_t)blockIdx.x * kSplitChains + lane;
+    const int64_t idx = split_chain<WIDE>(lane);
     const bool valid = idx < n_leaves;
     const int64_t page_u = idx / leaves_per_page;
     const int64_t i = idx - page_u * leaves_per_page;
     const int64_t lkv = page_u / p.npb;
     const int64_t jj = page_u - lkv * p.npb;
     const int64_t block_page = lkv * p.block_pages + p.page_base + jj;
-    if (threadIdx.x >= 32) {
+    if (produce) {
         const uint64_t off = (uint64_t)i * kLeafBytes;
         const uint4 *v = valid ? reinterpret_cast<const uint4 *>(p.src + (uint64_t)block_page * page_bytes + off)
                                : nullptr;
         uint4 *o = valid ? reinterpret_cast<uint4 *>(p.pool + ((uint64_t)lkv * p.pool_pages +
                                                                (uint64_t)p.pids.pid[jj]) * page_bytes + off)
                          : nullptr;
-        split_produce_leaf<true>(kw, v, o, lane);
+        split_produce_leaf<true, WIDE>(sm, v, o, lane, one);
     } else {
-        uint32_t st[8];
-        split_consume(st, kw, kSplitLeafBlocks, lane, one);
-        if (valid) store_state(out + (block_page * leaves_per_page + i) * 8, st);
+        split_consume_leaf<WIDE>(sm, valid ? out + (block_page * leaves_per_page + i) * 8 : nullptr, false, lane, one);
     }
 }
 
 // sha256_leaves_kernel's work in the two-warp form (whole 4 KiB leaves).
+template <bool WIDE>
 __global__ void __launch_bounds__(64) sha256_leaves_split_kernel(const PageSource src, int64_t n_pages,
                                                                  int64_t leaves_per_page,
                                                                  uint32_t *__restrict__ out, uint32_t one) {
-    __shared__ __align__(16) uint32_t kw[2][64][kSplitChains];
+    __shared__ SplitShared sm;
+    const bool produce = split_begin(sm);
     const int lane = threadIdx.x & 31;
-    const int64_t idx = (int64_t)blockIdx.x * kSplitChains + lane;
+    const int64_t idx = split_chain<WIDE>(lane);
     const bool valid = idx < n_pages * leaves_per_page;
     const int64_t p = idx / leaves_per_page;
     const int64_t i = idx - p * leaves_per_page;
@@ -463,24 +633,18 @@ __global__ void __launch_bounds__(64) sha256_leaves_split_kernel(const PageSourc
         const int32_t pid = src.pid[p - (p / src.npb) * src.npb];
         in_range = pid >= 0 && pid < src.plane_pages;
     }
-    if (threadIdx.x >= 32) {
+    if (produce) {
         const uint4 *v = in_range ? reinterpret_cast<const uint4 *>(page_addr(src, p) + (uint64_t)i * kLeafBytes)
                                   : nullptr;
-        split_produce_leaf<false>(kw, v, nullptr, lane);
+        split_produce_leaf<false, WIDE>(sm, v, nullptr, lane, one);
     } else {
-        uint32_t st[8];
-        split_consume(st, kw, kSplitLeafBlocks, lane, one);
-        if (!valid) return;
-        if (!in_range) {
-#pragma unroll
-            for (int w = 0; w < 8; ++w) st[w] = 0u;  // no digest of any page: reported as a mismatch
-        }
         int64_t po = p;
         if (src.pid && src.out_plane_stride) {
             const int64_t plane = p / src.npb;
             po = plane * src.out_plane_stride + src.out_j0 + (p - plane * src.npb);
         }
-        store_state(out + (po * leaves_per_page + i) * 8, st);
+        // a page id out of range has no digest: zeros, reported as a mismatch
+        split_consume_leaf<WIDE>(sm, valid ? out + (po * leaves_per_page + i) * 8 : nullptr, !in_range, lane, one);
     }
 }
 
@@ -650,57 +814,65 @@ __global__ void __launch_bounds__(128) sha256_pages_kernel(const uint32_t *__res
     page_verdict(p, st, out, expected, status, seq);
 }
 
-// sha256_pages_kernel in the two-warp form: warp 1 feeds each page's leaf
-// digests (already big-endian words) and the final block.
+// sha256_pages_kernel in the two-warp form: the loading warp feeds each page's
+// leaf digests (already big-endian words) and the final block.
 __global__ void __launch_bounds__(64) sha256_pages_split_kernel(const uint32_t *__restrict__ leaf_words,
                                                                 int64_t n_pages, int64_t m,
                                                                 uint8_t *__restrict__ out,
                                                                 const uint8_t *__restrict__ expected,
                                                                 DevStatus *status, int32_t seq, uint32_t one) {
-    __shared__ __align__(16) uint32_t kw[2][64][kSplitChains];
+    __shared__ SplitShared sm;
+    const bool produce = split_begin(sm);
     const int lane = threadIdx.x & 31;
-    const int64_t p = (int64_t)blockIdx.x * kSplitChains + lane;
+    const int64_t p = (int64_t)blockIdx.x * kSplitChains + (lane & (kSplitChains - 1));
     const bool valid = p < n_pages;
     const int64_t nwords = m * 8;
     const int nfull = (int)(nwords / 16);
     const int remw = (int)(nwords - (int64_t)nfull * 16);  // 0 or 8
-    if (threadIdx.x >= 32) {
+    if (produce) {
         const uint32_t *lw = leaf_words + (valid ? p : 0) * m * 8;
+        const int half = lane / kSplitChains;
+        // the lane's block of pair k: 16 whole words, the final block, or (past it) nothing
         uint4 nx[4];
+        auto load = [&](int blk) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            nx[q] = valid && nfull > 0 ? reinterpret_cast<const uint4 *>(lw)[q] : make_uint4(0, 0, 0, 0);
-        for (int blk = 0; blk < nfull; ++blk) {
-            uint4 x[4];
+            for (int q = 0; q < 4; ++q) nx[q] = make_uint4(0, 0, 0, 0);
+            if (!valid) return;
+            if (blk < nfull) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) x[q] = nx[q];
-            if (valid && blk + 1 < nfull) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) nx[q] = reinterpret_cast<const uint4 *>(lw + (blk + 1) * 16)[q];
+                for (int q = 0; q < 4; ++q) nx[q] = reinterpret_cast<const uint4 *>(lw + (int64_t)blk * 16)[q];
+            } else if (blk == nfull) {
+                const uint64_t bits = (uint64_t)m * 32ull * 8ull;
+                if (remw) {
+                    nx[0] = reinterpret_cast<const uint4 *>(lw + (int64_t)nfull * 16)[0];
+                    nx[1] = reinterpret_cast<const uint4 *>(lw + (int64_t)nfull * 16)[1];
+                    nx[2].x = 0x80000000u;
+                } else {
+                    nx[0].x = 0x80000000u;
+                }
+                nx[3].z = (uint32_t)(bits >> 32);
+                nx[3].w = (uint32_t)bits;
             }
+        };
+        const int n_pairs = (nfull + 2) >> 1;
+        load(half);
+        for (int k = 0; k < n_pairs; ++k) {
             uint32_t w[16];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                w[4 * q + 0] = x[q].x;
-                w[4 * q + 1] = x[q].y;
-                w[4 * q + 2] = x[q].z;
-                w[4 * q + 3] = x[q].w;
+                w[4 * q + 0] = nx[q].x;
+                w[4 * q + 1] = nx[q].y;
+                w[4 * q + 2] = nx[q].z;
+                w[4 * q + 3] = nx[q].w;
             }
-            split_hand_over(kw, w, blk, lane);
+            if (k + 1 < n_pairs) load(2 * (k + 1) + half);
+            split_hand_over(sm, w, k, lane, one);
         }
-        uint32_t w[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) w[q] = 0;
-        for (int q = 0; q < remw; ++q) w[q] = valid ? lw[nfull * 16 + q] : 0u;
-        w[remw] = 0x80000000u;
-        const uint64_t bits = (uint64_t)m * 32ull * 8ull;
-        w[14] = (uint32_t)(bits >> 32);
-        w[15] = (uint32_t)bits;
-        split_hand_over(kw, w, nfull, lane);
     } else {
-        uint32_t st[8];
-        split_consume(st, kw, nfull + 1, lane, one);
-        if (valid) page_verdict(p, st, out, expected, status, seq);
+        uint32_t st[4], full[8];
+        split_consume(st, sm, nfull + 1, lane, one);
+        split_whole_state(full, st);
+        if (valid && lane < kSplitChains) page_verdict(p, full, out, expected, status, seq);
     }
 }
 
@@ -833,54 +1005,78 @@ __global__ void __launch_bounds__(32) sha256_serial_kernel(const uint8_t *seg0, 
     }
 }
 
-// sha256_serial_kernel's whole 64-byte blocks in the two-warp form: every
-// lane of both warps runs the same chain (lane 0's result is kept), warp 1
-// reads the message two blocks ahead, warp 0 runs the rounds; lane 0 of
-// warp 0 then finishes the tail and the padding with the byte-wise hasher.
-// For 4-byte aligned segments with seg0's length a multiple of 4.
+// sha256_serial_kernel in the two-warp form: every pair of lanes of the
+// rounds' warp runs the same chain (lane 0's result is kept) and the other warp reads the message
+// two pairs of blocks ahead, the padding included.  For 4-byte aligned
+// segments with seg0's length a multiple of 4.
+// Word i of the padded message of n_blocks blocks, big-endian.
+__device__ __forceinline__ uint32_t padded_word(const uint8_t *seg0, uint64_t n0, const uint8_t *seg1, uint64_t n1,
+                                                uint64_t n_blocks, uint64_t i) {
+    const uint64_t total = n0 + n1, off = 4 * i;
+    if (off + 4 <= total) return bswap(msg_word(seg0, n0, seg1, i));
+    if (i + 2 >= 16 * n_blocks) {
+        const uint64_t bits = total * 8ull;
+        return i + 2 == 16 * n_blocks ? (uint32_t)(bits >> 32) : i + 1 == 16 * n_blocks ? (uint32_t)bits : 0u;
+    }
+    uint32_t v = 0;
+    for (int b = 0; b < 4; ++b) {
+        const uint64_t at = off + b;
+        const uint32_t x = at < total ? (at < n0 ? seg0[at] : seg1[at - n0]) : at == total ? 0x80u : 0u;
+        v |= x << (24 - 8 * b);
+    }
+    return v;
+}
+
 __global__ void __launch_bounds__(64) sha256_serial_split_kernel(const uint8_t *seg0, uint64_t n0, const uint8_t *seg1,
                                                                  uint64_t n1, int32_t n_blocks, uint8_t *out,
                                                                  const uint8_t *expected, DevStatus *status,
                                                                  uint32_t one) {
-    __shared__ __align__(16) uint32_t kw[2][64][kSplitChains];
+    __shared__ SplitShared sm;
+    const bool produce = split_begin(sm);
     const int lane = threadIdx.x & 31;
     if (blockIdx.x != 0) return;
-    if (threadIdx.x >= 32) {
+    if (produce) {
+        const uint64_t whole = (n0 + n1) / 64;  // blocks without padding
         uint32_t n1w[16], n2w[16];
+        // block blk as big-endian words (past the message: zeros)
+        auto load = [&](uint32_t w[16], int blk) {
+            if ((uint64_t)blk < whole) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            n1w[i] = n_blocks > 0 ? msg_word(seg0, n0, seg1, (uint64_t)i) : 0u;
-            n2w[i] = n_blocks > 1 ? msg_word(seg0, n0, seg1, 16ull + i) : 0u;
-        }
-        for (int blk = 0; blk < n_blocks; ++blk) {
+                for (int i = 0; i < 16; ++i) w[i] = bswap(msg_word(seg0, n0, seg1, 16ull * blk + i));
+            } else {
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    w[i] = blk < n_blocks ? padded_word(seg0, n0, seg1, n1, n_blocks, 16ull * blk + i) : 0u;
+            }
+        };
+        const int half = lane / kSplitChains;
+        const int n_pairs = (n_blocks + 1) >> 1;
+        load(n1w, half);
+        load(n2w, 2 + half);
+        for (int k = 0; k < n_pairs; ++k) {
             uint32_t w[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                w[i] = bswap(n1w[i]);
+                w[i] = n1w[i];
                 n1w[i] = n2w[i];
             }
-            if (blk + 2 < n_blocks) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) n2w[i] = msg_word(seg0, n0, seg1, 16ull * (blk + 2) + i);
-            }
-            split_hand_over(kw, w, blk, lane);
+            if (k + 2 < n_pairs) load(n2w, 2 * (k + 2) + half);
+            split_hand_over(sm, w, k, lane, one);
         }
         return;
     }
-    uint32_t st[8];
-    split_consume(st, kw, n_blocks, lane, one);
+    uint32_t st[4], full[8];
+    split_consume(st, sm, n_blocks, lane, one);
+    split_whole_state(full, st);
     if (lane != 0) return;
-    Stream s;
-    s.init(one);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) s.st[i] = st[i];
-    const uint64_t done = 64ull * (uint64_t)n_blocks;
-    s.total = done;
-    if (done < n0) s.feed(seg0 + done, n0 - done);
-    const uint64_t d1 = done > n0 ? done - n0 : 0;
-    if (d1 < n1) s.feed(seg1 + d1, n1 - d1);
     uint8_t dg[32];
-    s.final(dg);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        dg[4 * k + 0] = (uint8_t)(full[k] >> 24);
+        dg[4 * k + 1] = (uint8_t)(full[k] >> 16);
+        dg[4 * k + 2] = (uint8_t)(full[k] >> 8);
+        dg[4 * k + 3] = (uint8_t)full[k];
+    }
     if (out)
         for (int k = 0; k < 32; ++k) out[k] = dg[k];
     if (expected) {
@@ -895,26 +1091,32 @@ __global__ void __launch_bounds__(64) sha256_serial_split_kernel(const uint8_t *
 
 }  // namespace
 
-// The two-warp form is used for pages of whole 4 KiB leaves when a launch has
-// at most two of its 32-chain CTAs per SM (leaves) or four (page digests,
-// which read their input from L2); beyond that the one-warp forms keep more
-// chains going per SM.  KVG_SHA_NO_SPLIT=1 turns it off.
+// The two-warp form is used for pages of whole 4 KiB leaves (leaf launches
+// below) and for page digests, which read their input from L2, up to eight of
+// its CTAs per SM; beyond that the one-warp forms keep more chains going per
+// SM.  KVG_SHA_NO_SPLIT=1 turns it off.
 static bool split_off() {
     static const bool off = env_knob("KVG_SHA_NO_SPLIT", 0) > 0;
     return off;
 }
 
-// Leaves per SM up to which a leaf-hashing launch takes the two-warp form:
-// two of its CTAs per SM (four warps, one per scheduler).  A verified graft
-// of 16 to 64 leaves per SM took 0.082-0.083 ms in it against 0.117 in the
-// one-warp form; at 96 and 128 leaves per SM 0.130-0.137 against 0.118-0.121.
-// A verified graft from pinned host memory keeps the one-warp form: its leaf
-// loads outlast the rounds of a block in the two-warp form (the last chunk of
+// Leaves per SM up to which a leaf launch takes the two-warp form.  Up to two
+// CTAs of 16 chains per SM (four warps, one per scheduler) a chain has two
+// lanes; from there to two CTAs of 32 the wide form is faster: digests of 16,
+// 32, 48 and 64 leaves per SM take 71, 73, 87 and 92 us with two lanes, 73, 75,
+// 74 and 76 wide, and 104 to 109 in one warp; of 96 and 128, 138 and 176, 124
+// and 127, and 110.  A verified graft from pinned host memory keeps the one-warp
+// form: its leaf loads outlast the rounds of a block here (the last chunk of
 // the 12B block's host-store graft, 40 leaves per SM, made the e2e step
 // 15.73-15.83 ms instead of 15.63-15.71).
 static int split_leaves_per_sm() {
-    static const int v = env_knob("KVG_SHA_SPLIT_LEAVES_PER_SM", 2 * kSplitChains);
+    static const int v = env_knob("KVG_SHA_SPLIT_LEAVES_PER_SM", 2 * kWideChains);
     return v;
+}
+static bool split_wide(int64_t n, int n_sm) { return n > (int64_t)n_sm * 2 * kSplitChains; }
+static int split_grid(int64_t n, bool wide) {
+    const int per = wide ? kWideChains : kSplitChains;
+    return (int)((n + per - 1) / per);
 }
 
 static int current_sm_count() {
@@ -931,8 +1133,9 @@ cudaError_t launch_sha256_leaves(const PageSource &src, int64_t n_pages, uint32_
     const int64_t n = n_pages * m;
     if (n == 0) return cudaSuccess;
     if (!split_off() && src.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
-        sha256_leaves_split_kernel<<<(int)((n + kSplitChains - 1) / kSplitChains), 64, 0, s>>>(src, n_pages, m,
-                                                                                             leaf_words, 1u);
+        const bool wide = split_wide(n, n_sm);
+        auto *kernel = wide ? sha256_leaves_split_kernel<true> : sha256_leaves_split_kernel<false>;
+        kernel<<<split_grid(n, wide), 64, 0, s>>>(src, n_pages, m, leaf_words, 1u);
         count_launches(1);
         return cudaGetLastError();
     }
@@ -953,7 +1156,9 @@ cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int 
     const int64_t n = (int64_t)p.n_layers * 2 * p.npb * m;
     if (n == 0) return cudaSuccess;
     if (split_ok && !split_off() && p.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
-        graft_verify_split_kernel<<<(int)((n + kSplitChains - 1) / kSplitChains), 64, 0, s>>>(p, m, leaf_words, 1u);
+        const bool wide = split_wide(n, n_sm);
+        auto *kernel = wide ? graft_verify_split_kernel<true> : graft_verify_split_kernel<false>;
+        kernel<<<split_grid(n, wide), 64, 0, s>>>(p, m, leaf_words, 1u);
         count_launches(1);
         return cudaGetLastError();
     }
@@ -982,7 +1187,7 @@ cudaError_t launch_sha256_pages(const uint32_t *leaf_words, int64_t n_pages, int
                                 uint8_t *out, const uint8_t *expected, DevStatus *status,
                                 int32_t seq, cudaStream_t s) {
     if (n_pages == 0) return cudaSuccess;
-    if (!split_off() && n_pages <= (int64_t)current_sm_count() * 4 * kSplitChains) {
+    if (!split_off() && n_pages <= (int64_t)current_sm_count() * 8 * kSplitChains) {
         sha256_pages_split_kernel<<<(int)((n_pages + kSplitChains - 1) / kSplitChains), 64, 0, s>>>(
             leaf_words, n_pages, leaves_per_page, out, expected, status, seq, 1u);
         count_launches(1);
@@ -999,8 +1204,8 @@ cudaError_t launch_sha256_serial(const uint8_t *seg0, uint64_t n0, const uint8_t
                                  uint8_t *out, const uint8_t *expected, DevStatus *status,
                                  cudaStream_t s) {
     const bool aligned = !((reinterpret_cast<uintptr_t>(seg0) | reinterpret_cast<uintptr_t>(seg1) | n0) & 3);
-    const uint64_t n_blocks = (n0 + n1) / 64;
-    if (!split_off() && aligned && n_blocks >= 1 && n_blocks < (1ull << 30)) {
+    const uint64_t n_blocks = (n0 + n1 + 9 + 63) / 64;  // with the padding
+    if (!split_off() && aligned && n_blocks < (1ull << 30)) {
         sha256_serial_split_kernel<<<1, 64, 0, s>>>(seg0, n0, seg1, n1, (int32_t)n_blocks, out, expected, status, 1u);
     } else {
         sha256_serial_kernel<<<1, 32, 0, s>>>(seg0, n0, seg1, n1, out, expected, status, 1u);
