@@ -32,7 +32,10 @@ struct DevStatus {
     int32_t n_mismatch;
     int32_t n_checked;
     int32_t seq;
-    int32_t pad[3];
+    int32_t pad;
+    // a batch check's last failing graft: (call, graft, seq) from high to low
+    // bits, kept by maximum; 0 when a later check of one graft wrote seq
+    unsigned long long batch_fail;
     int32_t list[KVG_REPORT_MAX_PAGES];
 };
 
@@ -109,7 +112,8 @@ struct GraftMeta {
     int32_t npb;
     int32_t first_job;
     int32_t trig;      // -1: own position (byte copy)
-    int32_t pad_;
+    int32_t seq;
+    const uint8_t *digests;  // the block's page digests [n_layers][2][npb][32]
 };
 struct GraftBatchParams {
     const GraftJob *jobs;
@@ -124,7 +128,32 @@ struct GraftBatchParams {
     uint64_t page_bytes;
     int64_t pool_pages;
     uint8_t *pool;
+    int32_t write_meta;    // this launch writes the position tags, page tables and fills
+    int32_t rotated_only;  // copy kernel: only the key pages of re-based grafts
+    // verifying launches cover the jobs [job0, job0 + slice_jobs)
+    int64_t job0, slice_jobs;
+    int32_t hash_only;     // the pages are in the cache already: hash them there (re-based grafts: in the store)
 };
+
+// Position tags, page-table entries and fills of a batch's grafts: a graft's
+// are written by one CTA of the launch, or by up to 16 where it has that many
+// per graft.
+__device__ __forceinline__ void batch_metadata(const GraftBatchParams &p) {
+    const int64_t P = p.page_size;
+    const int per = (int)gridDim.x / p.n_grafts;
+    const int parts = per < 1 ? 1 : per > 16 ? 16 : per;
+    const int64_t step = (int64_t)parts * blockDim.x;
+    for (int64_t w = blockIdx.x; w < (int64_t)p.n_grafts * parts; w += gridDim.x) {
+        const GraftMeta m = p.metas[w / parts];
+        const int64_t t0 = (w % parts) * blockDim.x + threadIdx.x;
+        for (int64_t t = t0; t < m.n_tokens; t += step) m.dst_pos[t] = (int32_t)((int64_t)m.src_pos[t] + m.delta);
+        for (int64_t j = t0; j < m.npb; j += step) {
+            m.table_row[j] = p.jobs[m.first_job + j].pid;
+            const int64_t f = m.n_tokens - j * P;
+            m.fill_row[j] = (int32_t)(f < P ? f : P);
+        }
+    }
+}
 
 // ---------------------------------------------------------------- append --
 struct AppendParams {
@@ -287,6 +316,13 @@ cudaError_t launch_append_batch_e4m3(const AppendBatchParams &p, int n_sm, cudaS
 // from pinned host memory, whose loads are too slow for it).
 cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int n_sm, cudaStream_t s,
                                 bool ring_ok = true, bool split_ok = true);
+// A batch's jobs [job0, job0 + slice_jobs): copy and leaf hashes in one pass
+// (hash_only: hashes alone), leaf_words[(plane * slice_jobs + job - job0) *
+// leaves_per_page + leaf]; then the page digests, compared with each block's.
+cudaError_t launch_graft_batch_verify(const GraftBatchParams &p, uint32_t *leaf_words, int n_sm, cudaStream_t s,
+                                      bool ring_ok, bool split_ok);
+cudaError_t launch_graft_batch_pages(const GraftBatchParams &p, const uint32_t *leaf_words, DevStatus *status,
+                                     uint32_t call, cudaStream_t s);
 cudaError_t launch_append(const AppendParams &p, int n_sm, cudaStream_t s);
 cudaError_t launch_append_batch(const AppendBatchParams &p, int n_sm, cudaStream_t s);
 cudaError_t launch_gather(const GatherParams &p, int n_sm, cudaStream_t s);

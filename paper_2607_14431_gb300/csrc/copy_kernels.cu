@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(kCopyThreads) graft_batch_kernel(const GraftBa
         uint8_t *dst = p.pool + ((uint64_t)lkv * p.pool_pages + (uint64_t)job.pid) * page_bytes + off;
         const int32_t trig = ROT != 0 && !(lkv & 1) ? p.metas[job.meta].trig : -1;
         if (trig < 0) {
-            copy_chunk(dst, src, p.chunk_bytes);
+            if (!p.rotated_only) copy_chunk(dst, src, p.chunk_bytes);
         } else {
             const int half = p.head_dim >> 1;
             rotate_chunk<ROT>(dst, src, p.chunk_bytes, (int64_t)(off / row_bytes), (int64_t)job.page * p.page_size,
@@ -778,18 +778,7 @@ __global__ void __launch_bounds__(kCopyThreads) graft_batch_kernel(const GraftBa
         }
     }
     // metadata last: the copies start at once and this fills the tail wave
-    const int64_t P = p.page_size;
-    const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
-    for (int32_t g = 0; g < p.n_grafts; ++g) {
-        const GraftMeta m = p.metas[g];
-        for (int64_t t = gtid; t < m.n_tokens; t += gsz) m.dst_pos[t] = (int32_t)((int64_t)m.src_pos[t] + m.delta);
-        for (int64_t j = gtid; j < m.npb; j += gsz) {
-            m.table_row[j] = p.jobs[m.first_job + j].pid;
-            const int64_t f = m.n_tokens - j * P;
-            m.fill_row[j] = (int32_t)(f < P ? f : P);
-        }
-    }
+    if (p.write_meta) batch_metadata(p);
 }
 
 cudaError_t launch_graft_batch(const GraftBatchParams &p, int n_sm, cudaStream_t s, int max_ctas, int rotate) {

@@ -778,6 +778,7 @@ struct kvg_cache {
     // kvg_graft_batch's job table: staged in pinned host memory, copied to
     // batch_dev on the call's stream; batch_ev marks when the copy has read it
     Scratch batch_dev;
+    uint32_t batch_calls = 0;  // verified batches so far: orders their mismatches in the status word
     uint8_t *batch_host = nullptr;
     size_t batch_host_cap = 0;
     cudaEvent_t batch_ev = nullptr;
@@ -1381,6 +1382,7 @@ static kvg_status read_status(kvg_cache *c, kvg_graft_report *report) {
     DevStatus hs;
     KVG_CUDA(cudaMemcpy(&hs, c->status, sizeof hs, cudaMemcpyDeviceToHost));
     KVG_CUDA(cudaMemset(c->status, 0, sizeof(DevStatus)));
+    if (hs.batch_fail) hs.seq = (int32_t)(hs.batch_fail & 0xffffffffull);
     if (report) {
         report->seq = hs.seq;
         report->n_mismatch = hs.n_mismatch;
@@ -1734,6 +1736,27 @@ extern "C" kvg_status kvg_graft_chunked(kvg_store *s, uint64_t block_id, kvg_cac
     return graft_impl(s, block_id, c, seq, dst_slot, delta, flags, stream, report, ce);
 }
 
+// Leaf-digest scratch of a verified batch: one launch hashes *slice jobs (one
+// block page in every plane each), all of them where their leaf digests fit
+// 128 MiB (4 million leaves, some forty full waves of the hash kernel, so the
+// drained last wave of a slice costs little), and never fewer than the
+// longest block's, which one graft would need anyway.  Where the larger
+// scratch cannot be had, the smaller one serves.
+static cudaError_t batch_leaf_scratch(kvg_cache *c, int64_t pages, int64_t most_pages, int64_t *slice) {
+    const int64_t m = (int64_t)((c->page_bytes + kLeafBytes - 1) / kLeafBytes);
+    const uint64_t per_job = (uint64_t)c->dims.n_layers * 2 * m * 32;
+    static const int mib = env_knob("KVG_BATCH_LEAF_MB", 128);
+    const int64_t fit = std::max<int64_t>((int64_t)(((uint64_t)mib << 20) / per_job), most_pages);
+    *slice = std::min(pages, fit);
+    cudaError_t e = c->leaf.ensure((size_t)*slice * per_job);
+    if (e != cudaSuccess && *slice > most_pages) {
+        cudaGetLastError();
+        *slice = most_pages;
+        e = c->leaf.ensure((size_t)*slice * per_job);
+    }
+    return e;
+}
+
 extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, kvg_cache *c, const int32_t *seq_ids,
                                       const int64_t *deltas, int32_t n, uint32_t flags, void *stream,
                                       kvg_graft_report *report) {
@@ -1747,7 +1770,7 @@ extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, k
     const int64_t P = c->dims.page_size;
     // every check before any state changes: the batch happens whole or not at all
     std::unordered_map<int32_t, int64_t> slots;
-    int64_t pages = 0;
+    int64_t pages = 0, most_pages = 0;
     for (int32_t i = 0; i < n; ++i) {
         const int32_t seq = seq_ids[i];
         if (seq < 0 || seq >= c->max_seqs) return fail(KVG_ERR_ARG, "bad seq %d (graft %d)", seq, i);
@@ -1765,6 +1788,7 @@ extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, k
             return fail(KVG_ERR_ARG, "graft %d: relocation needs a bf16 cache", i);
         it->second = dst + blk.lay.n_tokens;
         pages += blk.lay.n_pages;
+        most_pages = std::max(most_pages, blk.lay.n_pages);
     }
     if (pages > (int64_t)c->free_list.size()) return fail(KVG_ERR_CAPACITY, "out of free pages");
     DeviceGuard g(c->device);
@@ -1796,9 +1820,14 @@ extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, k
         c->batch_host_cap = want;
     }
     KVG_CUDA(c->batch_dev.ensure(bytes));
+    const bool verify = flags & KVG_GRAFT_VERIFY;
+    int64_t slice = pages;  // jobs per verifying launch
+    if (verify) {
+        const cudaError_t e = batch_leaf_scratch(c, pages, most_pages, &slice);
+        if (e != cudaSuccess) return cuda_fail(e, "leaf digests of a batch");
+    }
     GraftMeta *metas = reinterpret_cast<GraftMeta *>(c->batch_host);
     GraftJob *jobs = reinterpret_cast<GraftJob *>(c->batch_host + meta_bytes);
-    std::vector<std::pair<int32_t, int64_t>> verify_at;  // (seq, first page index) per graft
     int32_t job = 0;
     for (int32_t i = 0; i < n; ++i) {
         const int32_t seq = seq_ids[i];
@@ -1821,11 +1850,11 @@ extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, k
         m.npb = (int32_t)npb;
         m.first_job = job;
         m.trig = trig_of[i];
-        m.pad_ = 0;
+        m.seq = seq;
+        m.digests = blk.dev + blk.lay.dig_off;
         for (int64_t j = 0; j < npb; ++j, ++job)
             jobs[job] = GraftJob{blk.dev + blk.lay.pages_off + (uint64_t)j * c->page_bytes, (int32_t)npb, pids[j], i,
                                  (int32_t)j};
-        verify_at.push_back({seq, jdst});
     }
     float *trig = reinterpret_cast<float *>(c->batch_host + trig_off);
     for (size_t t = 0; t < table_delta.size(); ++t)
@@ -1848,16 +1877,29 @@ extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, k
     p.pool = c->pool;
     // the store's RoPE pairing and base, as kvg_graft uses them
     const int rotate = table_delta.empty() ? 0 : s->dims.rope_style == KVG_ROPE_HALF ? 1 : 2;
-    KVG_CUDA(launch_graft_batch(p, c->n_sm, st, s->residency == KVG_RESIDENCY_PINNED_HOST ? host_copy_grid_cap() : 0,
-                                rotate));
-    // verification: own-position grafts hash their restored pages; re-based
-    // ones hash the stored pages (their key pages differ by design)
-    if (flags & KVG_GRAFT_VERIFY)
-        for (int32_t i = 0; i < n; ++i) {
-            kvg_status r = enqueue_verify(s, s->blocks[block_ids[i]], c, verify_at[i].first, verify_at[i].second,
-                                          trig_of[i] >= 0, st);
-            if (r != KVG_OK) return r;
+    if (!rotate) p.trig = nullptr;
+    const bool host_src = s->residency == KVG_RESIDENCY_PINNED_HOST;
+    // Verified, from an HBM store: every page is read once, its copy and its
+    // leaf hashes in one pass; only the re-based key pages are written by the
+    // rotating copy before.  From a pinned-host store the copy kernel, whose
+    // wide reads keep the host link at its limit, moves everything and the
+    // hashes follow in the cache (of re-based grafts: in the store).
+    p.write_meta = !verify || host_src;
+    p.rotated_only = verify && !host_src;
+    if (!p.rotated_only || rotate)
+        KVG_CUDA(launch_graft_batch(p, c->n_sm, st, host_src ? host_copy_grid_cap() : 0, rotate));
+    if (verify) {
+        const uint32_t call = ++c->batch_calls % (1u << 18) + 1;
+        p.hash_only = host_src;
+        for (p.job0 = 0; p.job0 < pages; p.job0 += slice) {
+            p.slice_jobs = std::min(slice, pages - p.job0);
+            p.write_meta = !host_src && p.job0 == 0;
+            // the two-warp form's loads are too slow for host memory (re-based grafts hash the store)
+            KVG_CUDA(launch_graft_batch_verify(p, static_cast<uint32_t *>(c->leaf.ptr), c->n_sm, st,
+                                               c->dims.kv_dtype == KVG_KV_BF16, !(host_src && rotate)));
+            KVG_CUDA(launch_graft_batch_pages(p, static_cast<const uint32_t *>(c->leaf.ptr), c->status, call, st));
         }
+    }
     return finish_verify(c, n == 1 ? seq_ids[0] : -1, flags,
                          (flags & KVG_GRAFT_VERIFY) ? (int32_t)(c->dims.n_layers * 2 * pages) : 0, st, report);
 }

@@ -146,7 +146,8 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // busy) hides behind the compressions without costing registers.  (A layout
 // with the 32 lanes' vectors side by side, free of bank conflicts, measured
 // slower in the 12b step: 6.05 against 5.94 ms.)
-template <int R>
+// SOME: only when copy_to is not null.
+template <int R, bool SOME = false>
 __device__ __forceinline__ void hash_leaf_ring(const uint8_t *leaf, uint64_t len, uint8_t *copy_to, uint32_t st[8],
                                                uint32_t one, uint4 *ring) {
     const uint4 *v = reinterpret_cast<const uint4 *>(leaf);
@@ -179,8 +180,10 @@ __device__ __forceinline__ void hash_leaf_ring(const uint8_t *leaf, uint64_t len
 #pragma unroll
             for (int q = 0; q < 4; ++q) cp_async16(ring + 4 * slot + q, v + 4 * (blk + R) + q);
         cp_async_commit();
+        if (!SOME || o) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) __stcs(o + 4 * blk + q, x[q]);
+            for (int q = 0; q < 4; ++q) __stcs(o + 4 * blk + q, x[q]);
+        }
         compress(st, w, one);
     }
     cp_async_wait<0>();
@@ -195,15 +198,17 @@ __device__ __forceinline__ void hash_leaf_ring(const uint8_t *leaf, uint64_t len
         w[15] = (uint32_t)bits;
         compress(st, w, one);
     } else {
-        for (int q = 0; q < rem / 16; ++q) o[4 * nfull + q] = v[4 * nfull + q];
+        if (!SOME || o)
+            for (int q = 0; q < rem / 16; ++q) o[4 * nfull + q] = v[4 * nfull + q];
         finish(st, leaf + (len & ~63ull), rem, len, one);
     }
 }
 
 // SHA-256 of one leaf of `len` bytes (16-byte aligned).  With COPY the leaf
 // is also written to `copy_to`, from the same registers that are hashed, so
-// the bytes written are exactly the bytes whose digest is checked.
-template <bool COPY>
+// the bytes written are exactly the bytes whose digest is checked (SOME: only
+// when copy_to is not null).
+template <bool COPY, bool SOME = false>
 __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uint8_t *copy_to, uint32_t st[8],
                                           uint32_t one) {
     const uint4 *v = reinterpret_cast<const uint4 *>(leaf);
@@ -231,7 +236,7 @@ __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uin
 #pragma unroll
             for (int q = 0; q < 4; ++q) n2[q] = __ldg(v + 4 * (blk + 2) + q);
         }
-        if (COPY) {
+        if (COPY && (!SOME || o)) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) __stcs(o + 4 * blk + q, x[q]);
         }
@@ -255,7 +260,7 @@ __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uin
         w[15] = (uint32_t)bits;
         compress(st, w, one);
     } else {
-        if (COPY)
+        if (COPY && (!SOME || o))
             for (int q = 0; q < rem / 16; ++q) o[4 * nfull + q] = v[4 * nfull + q];
         finish(st, leaf + (len & ~63ull), rem, len, one);
     }
@@ -743,42 +748,153 @@ __global__ void __launch_bounds__(128) graft_verify_kernel(const GraftParams p, 
     }
 }
 
-// Page p's digest (the state words, big-endian) written to out and/or
-// compared with expected; a mismatch is recorded in the status word.
-__device__ __forceinline__ void page_verdict(int64_t p, const uint32_t st[8], uint8_t *__restrict__ out,
-                                             const uint8_t *__restrict__ expected, DevStatus *status, int32_t seq) {
-    uint8_t dg[32];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        dg[4 * k + 0] = (uint8_t)(st[k] >> 24);
-        dg[4 * k + 1] = (uint8_t)(st[k] >> 16);
-        dg[4 * k + 2] = (uint8_t)(st[k] >> 8);
-        dg[4 * k + 3] = (uint8_t)st[k];
-    }
-    if (out) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) out[p * 32 + k] = dg[k];
-    }
-    if (expected) {
-        bool same = true;
-#pragma unroll
-        for (int k = 0; k < 32; ++k) same &= dg[k] == expected[p * 32 + k];
-        if (!same) {
-            const int slot = atomicAdd(&status->n_mismatch, 1);
-            if (slot < KVG_REPORT_MAX_PAGES) status->list[slot] = (int32_t)p;
-            status->seq = seq;
-            atomicCAS(&status->err, 0, (int32_t)KVG_ERR_DIGEST);
+// ---- a batch of grafts, verified ------------------------------------------
+// The leaves of a batch's jobs in one launch, so that a batch of short blocks
+// fills the GPU like one long block does: a leaf per thread, leaf fastest,
+// then job, then plane (a block's pages follow one another in a plane).  A graft at its own position is copied and hashed in
+// one pass; a re-based one's value pages too, while its key pages, which the
+// rotating copy has written, are hashed in the store.
+struct BatchLeaf {
+    const uint8_t *src;
+    uint8_t *dst;  // null: hash only
+    uint64_t len;
+};
+
+template <bool SOME>
+__device__ __forceinline__ BatchLeaf batch_leaf(const GraftBatchParams &p, int64_t idx, int64_t m) {
+    const int64_t page = idx / m;
+    const int64_t lkv = page / p.slice_jobs;
+    const int64_t jb = page - lkv * p.slice_jobs;
+    const uint64_t off = (uint64_t)(idx - page * m) * kLeafBytes;
+    const GraftJob job = p.jobs[p.job0 + jb];
+    BatchLeaf r;
+    r.len = p.page_bytes - off;
+    if (r.len > kLeafBytes) r.len = kLeafBytes;
+    r.src = job.src + (uint64_t)lkv * job.block_pages * p.page_bytes + off;
+    r.dst = p.pool + ((uint64_t)lkv * p.pool_pages + (uint64_t)job.pid) * p.page_bytes + off;
+    if (SOME) {
+        const bool rebased = p.metas[job.meta].trig >= 0;
+        if (p.hash_only) {
+            if (!rebased) r.src = r.dst;
+            r.dst = nullptr;
+        } else if (rebased && !(lkv & 1)) {
+            r.dst = nullptr;
         }
+    }
+    return r;
+}
+
+// graft_verify_ring_kernel for a batch (the same launch sizes).
+template <bool SOME>
+__global__ void __launch_bounds__(128, 5) graft_batch_verify_ring_kernel(const GraftBatchParams p,
+                                                                         int64_t leaves_per_page,
+                                                                         uint32_t *__restrict__ out, uint32_t one) {
+    constexpr int R = kGraftVerifyRing;
+    extern __shared__ __align__(16) uint4 ring_mem[];
+    if (p.write_meta) batch_metadata(p);
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= p.slice_jobs * p.n_layers * 2 * leaves_per_page) return;
+    const BatchLeaf l = batch_leaf<SOME>(p, idx, leaves_per_page);
+    uint32_t st[8];
+    hash_leaf_ring<R, SOME>(l.src, l.len, l.dst, st, one, ring_mem + threadIdx.x * 4 * R);
+    store_state(out + idx * 8, st);
+}
+
+// graft_verify_kernel for a batch.
+template <bool SOME>
+__global__ void __launch_bounds__(128) graft_batch_verify_kernel(const GraftBatchParams p, int64_t leaves_per_page,
+                                                                 uint32_t *__restrict__ out, uint32_t one) {
+    if (p.write_meta) batch_metadata(p);
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= p.slice_jobs * p.n_layers * 2 * leaves_per_page) return;
+    const BatchLeaf l = batch_leaf<SOME>(p, idx, leaves_per_page);
+    uint32_t st[8];
+    hash_leaf<true, SOME>(l.src, l.len, l.dst, st, one);
+    store_state(out + idx * 8, st);
+}
+
+// graft_verify_split_kernel for a batch.
+template <bool WIDE>
+__global__ void __launch_bounds__(64) graft_batch_verify_split_kernel(const GraftBatchParams p,
+                                                                      int64_t leaves_per_page,
+                                                                      uint32_t *__restrict__ out, uint32_t one) {
+    __shared__ SplitShared sm;
+    const bool produce = split_begin(sm);
+    if (p.write_meta) batch_metadata(p);
+    const int lane = threadIdx.x & 31;
+    const int64_t idx = split_chain<WIDE>(lane);
+    const bool valid = idx < p.slice_jobs * p.n_layers * 2 * leaves_per_page;
+    if (produce) {
+        BatchLeaf l{nullptr, nullptr, 0};
+        if (valid) l = batch_leaf<true>(p, idx, leaves_per_page);
+        split_produce_leaf<true, WIDE>(sm, reinterpret_cast<const uint4 *>(l.src), reinterpret_cast<uint4 *>(l.dst),
+                                       lane, one);
+    } else {
+        split_consume_leaf<WIDE>(sm, valid ? out + idx * 8 : nullptr, false, lane, one);
     }
 }
 
+// Whether the digest with state words st (written big-endian) differs from
+// the 32 bytes at expected.
+__device__ __forceinline__ bool digest_differs(const uint32_t st[8], const uint8_t *__restrict__ expected) {
+    bool same = true;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) same &= (uint8_t)(st[k >> 2] >> (24 - 8 * (k & 3))) == expected[k];
+    return !same;
+}
+
+__device__ __forceinline__ void record_mismatch(DevStatus *status, int32_t page) {
+    const int slot = atomicAdd(&status->n_mismatch, 1);
+    if (slot < KVG_REPORT_MAX_PAGES) status->list[slot] = page;
+    atomicCAS(&status->err, 0, (int32_t)KVG_ERR_DIGEST);
+}
+
+// What becomes of page p's digest.  PageOut: written to out and/or compared
+// with expected; a mismatch is recorded in the status word.
+struct PageOut {
+    uint8_t *out;
+    const uint8_t *expected;
+    DevStatus *status;
+    int32_t seq;
+    __device__ __forceinline__ void operator()(int64_t p, const uint32_t st[8]) const {
+        if (out) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) out[p * 32 + k] = (uint8_t)(st[k >> 2] >> (24 - 8 * (k & 3)));
+        }
+        if (expected && digest_differs(st, expected + p * 32)) {
+            record_mismatch(status, (int32_t)p);
+            status->seq = seq;
+            status->batch_fail = 0;
+        }
+    }
+};
+
+// BatchCheck: page p of a batch's slice compared with its block's digest; the
+// status keeps the last failing graft.
+struct BatchCheck {
+    const GraftJob *jobs;
+    const GraftMeta *metas;
+    int64_t job0, slice_jobs;
+    uint32_t call;
+    DevStatus *status;
+    __device__ __forceinline__ void operator()(int64_t p, const uint32_t st[8]) const {
+        const int64_t lkv = p / slice_jobs;
+        const GraftJob job = jobs[job0 + p - lkv * slice_jobs];
+        const GraftMeta &m = metas[job.meta];
+        const int64_t page = lkv * job.block_pages + job.page;
+        if (!digest_differs(st, m.digests + page * 32)) return;
+        record_mismatch(status, (int32_t)page);
+        atomicMax(&status->batch_fail, ((unsigned long long)call << 45) | ((unsigned long long)job.meta << 32) |
+                                           (unsigned long long)(uint32_t)m.seq);
+    }
+};
+
 // Page digest from its leaf digests: the message is the leaf digests' bytes,
 // i.e. (big-endian) exactly the 8 state words of each leaf in order.
+template <class Verdict>
 __global__ void __launch_bounds__(128) sha256_pages_kernel(const uint32_t *__restrict__ leaf_words,
-                                                           int64_t n_pages, int64_t m,
-                                                           uint8_t *__restrict__ out,
-                                                           const uint8_t *__restrict__ expected,
-                                                           DevStatus *status, int32_t seq, uint32_t one) {
+                                                           int64_t n_pages, int64_t m, const Verdict verdict,
+                                                           uint32_t one) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n_pages) return;
     const uint32_t *lw = leaf_words + p * m * 8;
@@ -811,16 +927,15 @@ __global__ void __launch_bounds__(128) sha256_pages_kernel(const uint32_t *__res
         w[15] = (uint32_t)bits;
         compress<false>(st, w, one);
     }
-    page_verdict(p, st, out, expected, status, seq);
+    verdict(p, st);
 }
 
 // sha256_pages_kernel in the two-warp form: the loading warp feeds each page's
 // leaf digests (already big-endian words) and the final block.
+template <class Verdict>
 __global__ void __launch_bounds__(64) sha256_pages_split_kernel(const uint32_t *__restrict__ leaf_words,
-                                                                int64_t n_pages, int64_t m,
-                                                                uint8_t *__restrict__ out,
-                                                                const uint8_t *__restrict__ expected,
-                                                                DevStatus *status, int32_t seq, uint32_t one) {
+                                                                int64_t n_pages, int64_t m, const Verdict verdict,
+                                                                uint32_t one) {
     __shared__ SplitShared sm;
     const bool produce = split_begin(sm);
     const int lane = threadIdx.x & 31;
@@ -872,7 +987,7 @@ __global__ void __launch_bounds__(64) sha256_pages_split_kernel(const uint32_t *
         uint32_t st[4], full[8];
         split_consume(st, sm, nfull + 1, lane, one);
         split_whole_state(full, st);
-        if (valid && lane < kSplitChains) page_verdict(p, full, out, expected, status, seq);
+        if (valid && lane < kSplitChains) verdict(p, full);
     }
 }
 
@@ -1127,6 +1242,11 @@ static int current_sm_count() {
     return cache[dev];
 }
 
+static bool regs_only() {
+    static const bool v = env_knob("KVG_SHA_REGISTER_FORM", 0) > 0;
+    return v;
+}
+
 cudaError_t launch_sha256_leaves(const PageSource &src, int64_t n_pages, uint32_t *leaf_words,
                                  int n_sm, cudaStream_t s) {
     const int64_t m = (int64_t)((src.page_bytes + kLeafBytes - 1) / kLeafBytes);
@@ -1172,8 +1292,7 @@ cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int 
     // caller allows it: the ring form; otherwise the register form (see
     // graft_verify_ring_kernel).  KVG_SHA_REGISTER_FORM=1 keeps the register
     // form for every size.
-    static const bool regs_only = env_knob("KVG_SHA_REGISTER_FORM", 0) > 0;
-    if (ring_ok && !regs_only && n >= (int64_t)n_sm * 5 * 128 && grid > (int64_t)n_sm * 4) {
+    if (ring_ok && !regs_only() && n >= (int64_t)n_sm * 5 * 128 && grid > (int64_t)n_sm * 4) {
         const size_t smem = (size_t)128 * kGraftVerifyRing * 64;  // 24 KiB of ring slots per CTA
         graft_verify_ring_kernel<<<(int)grid, 128, smem, s>>>(p, m, leaf_words, 1u);
     } else {
@@ -1183,21 +1302,57 @@ cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int 
     return cudaGetLastError();
 }
 
+cudaError_t launch_graft_batch_verify(const GraftBatchParams &p, uint32_t *leaf_words, int n_sm, cudaStream_t s,
+                                      bool ring_ok, bool split_ok) {
+    const int64_t m = (int64_t)((p.page_bytes + kLeafBytes - 1) / kLeafBytes);
+    const int64_t n = p.slice_jobs * p.n_layers * 2 * m;
+    if (n == 0) return cudaSuccess;
+    const int grid = (int)((n + 127) / 128);
+    // the forms and their launch sizes are those of launch_graft_verify
+    if (split_ok && !split_off() && p.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
+        const bool wide = split_wide(n, n_sm);
+        auto *kernel = wide ? graft_batch_verify_split_kernel<true> : graft_batch_verify_split_kernel<false>;
+        kernel<<<split_grid(n, wide), 64, 0, s>>>(p, m, leaf_words, 1u);
+    } else if (ring_ok && !regs_only() && n >= (int64_t)n_sm * 5 * 128) {
+        const size_t smem = (size_t)128 * kGraftVerifyRing * 64;
+        if (p.trig || p.hash_only)
+            graft_batch_verify_ring_kernel<true><<<grid, 128, smem, s>>>(p, m, leaf_words, 1u);
+        else
+            graft_batch_verify_ring_kernel<false><<<grid, 128, smem, s>>>(p, m, leaf_words, 1u);
+    } else if (p.trig || p.hash_only) {
+        graft_batch_verify_kernel<true><<<grid, 128, 0, s>>>(p, m, leaf_words, 1u);
+    } else {
+        graft_batch_verify_kernel<false><<<grid, 128, 0, s>>>(p, m, leaf_words, 1u);
+    }
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+template <class Verdict>
+static cudaError_t launch_pages(const uint32_t *leaf_words, int64_t n_pages, int64_t leaves_per_page,
+                                const Verdict &verdict, cudaStream_t s) {
+    if (n_pages == 0) return cudaSuccess;
+    if (!split_off() && n_pages <= (int64_t)current_sm_count() * 8 * kSplitChains)
+        sha256_pages_split_kernel<<<(int)((n_pages + kSplitChains - 1) / kSplitChains), 64, 0, s>>>(
+            leaf_words, n_pages, leaves_per_page, verdict, 1u);
+    else
+        sha256_pages_kernel<<<(int)((n_pages + 127) / 128), 128, 0, s>>>(leaf_words, n_pages, leaves_per_page,
+                                                                         verdict, 1u);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_sha256_pages(const uint32_t *leaf_words, int64_t n_pages, int64_t leaves_per_page,
                                 uint8_t *out, const uint8_t *expected, DevStatus *status,
                                 int32_t seq, cudaStream_t s) {
-    if (n_pages == 0) return cudaSuccess;
-    if (!split_off() && n_pages <= (int64_t)current_sm_count() * 8 * kSplitChains) {
-        sha256_pages_split_kernel<<<(int)((n_pages + kSplitChains - 1) / kSplitChains), 64, 0, s>>>(
-            leaf_words, n_pages, leaves_per_page, out, expected, status, seq, 1u);
-        count_launches(1);
-        return cudaGetLastError();
-    }
-    sha256_pages_kernel<<<(int)((n_pages + 127) / 128), 128, 0, s>>>(leaf_words, n_pages,
-                                                                     leaves_per_page, out,
-                                                                     expected, status, seq, 1u);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_pages(leaf_words, n_pages, leaves_per_page, PageOut{out, expected, status, seq}, s);
+}
+
+cudaError_t launch_graft_batch_pages(const GraftBatchParams &p, const uint32_t *leaf_words, DevStatus *status,
+                                     uint32_t call, cudaStream_t s) {
+    const int64_t m = (int64_t)((p.page_bytes + kLeafBytes - 1) / kLeafBytes);
+    return launch_pages(leaf_words, p.slice_jobs * p.n_layers * 2, m,
+                        BatchCheck{p.jobs, p.metas, p.job0, p.slice_jobs, call, status}, s);
 }
 
 cudaError_t launch_sha256_serial(const uint8_t *seg0, uint64_t n0, const uint8_t *seg1, uint64_t n1,
