@@ -56,7 +56,11 @@ __device__ __forceinline__ uint32_t bswap(uint32_t x) { return __byte_perm(x, 0,
 // message schedule kept as a rolling 16-word window.  Rotations and logic
 // stay on the ALU pipe; additions and the schedule's plain shifts go to the
 // FMA pipe (fadd/fshr), balancing the two.
-template <bool FMA = true>
+// LAT: the additions reassociated for launches of few warps per scheduler,
+// where the recurrence's latency decides: e[t+1] is one addition behind
+// S1(e[t]) (h + K + W + d and Ch are added up before it), and a[t+1] =
+// e[t+1] + (S0 + Maj - d) is one behind e[t+1].  One addition a round more.
+template <bool FMA = true, bool LAT = false>
 __device__ __forceinline__ void compress(uint32_t st[8], uint32_t w[16], uint32_t one) {
     uint32_t a = st[0], b = st[1], c = st[2], d = st[3], e = st[4], f = st[5], g = st[6], h = st[7];
 #pragma unroll
@@ -72,6 +76,23 @@ __device__ __forceinline__ void compress(uint32_t st[8], uint32_t w[16], uint32_
         }
         const uint32_t S1 = rotr(e, 6) ^ rotr(e, 11) ^ rotr(e, 25);
         const uint32_t ch = (e & f) ^ (~e & g);
+        if (LAT) {
+            const uint32_t y = fadd<FMA>(fadd<FMA>(fadd<FMA>(wt, kK[t], one), h, one), d, one);
+            const uint32_t ne = fadd<FMA>(fadd<FMA>(y, ch, one), S1, one);
+            const uint32_t S0 = rotr(a, 2) ^ rotr(a, 13) ^ rotr(a, 22);
+            const uint32_t maj = (a & b) ^ (a & c) ^ (b & c);
+            uint32_t md;  // Maj - d
+            asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(md) : "r"(d), "r"(0u - one), "r"(maj));
+            h = g;
+            g = f;
+            f = e;
+            e = ne;
+            d = c;
+            c = b;
+            b = a;
+            a = fadd<FMA>(ne, fadd<FMA>(S0, md, one), one);
+            continue;
+        }
         const uint32_t T1 = fadd<FMA>(fadd<FMA>(h, S1, one), fadd<FMA>(fadd<FMA>(ch, kK[t], one), wt, one), one);
         const uint32_t S0 = rotr(a, 2) ^ rotr(a, 13) ^ rotr(a, 22);
         const uint32_t maj = (a & b) ^ (a & c) ^ (b & c);
@@ -208,7 +229,7 @@ __device__ __forceinline__ void hash_leaf_ring(const uint8_t *leaf, uint64_t len
 // is also written to `copy_to`, from the same registers that are hashed, so
 // the bytes written are exactly the bytes whose digest is checked (SOME: only
 // when copy_to is not null).
-template <bool COPY, bool SOME = false>
+template <bool COPY, bool SOME = false, bool LAT = false>
 __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uint8_t *copy_to, uint32_t st[8],
                                           uint32_t one) {
     const uint4 *v = reinterpret_cast<const uint4 *>(leaf);
@@ -247,7 +268,7 @@ __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uin
             w[4 * q + 2] = bswap(x[q].z);
             w[4 * q + 3] = bswap(x[q].w);
         }
-        compress(st, w, one);
+        compress<true, LAT>(st, w, one);
     }
     const int rem = (int)(len & 63);
     if (rem == 0) {
@@ -258,7 +279,7 @@ __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uin
         const uint64_t bits = len * 8ull;
         w[14] = (uint32_t)(bits >> 32);
         w[15] = (uint32_t)bits;
-        compress(st, w, one);
+        compress<true, LAT>(st, w, one);
     } else {
         if (COPY && (!SOME || o))
             for (int q = 0; q < rem / 16; ++q) o[4 * nfull + q] = v[4 * nfull + q];
@@ -653,6 +674,7 @@ __global__ void __launch_bounds__(64) sha256_leaves_split_kernel(const PageSourc
     }
 }
 
+template <bool LAT>
 __global__ void __launch_bounds__(128) sha256_leaves_kernel(const PageSource src, int64_t n_pages,
                                                             int64_t leaves_per_page,
                                                             uint32_t *__restrict__ out, uint32_t one) {
@@ -670,7 +692,7 @@ __global__ void __launch_bounds__(128) sha256_leaves_kernel(const PageSource src
             in_range = pid >= 0 && pid < src.plane_pages;
         }
         if (in_range) {
-            hash_leaf<false>(page_addr(src, p) + (uint64_t)i * kLeafBytes, len, nullptr, st, one);
+            hash_leaf<false, false, LAT>(page_addr(src, p) + (uint64_t)i * kLeafBytes, len, nullptr, st, one);
         } else {
 #pragma unroll
             for (int w = 0; w < 8; ++w) st[w] = 0u;  // no digest of any page: reported as a mismatch
@@ -1234,6 +1256,16 @@ static int split_grid(int64_t n, bool wide) {
     return (int)((n + per - 1) / per);
 }
 
+// Whether a one-warp launch of sha256_leaves_kernel uses the latency order of
+// additions: checking a restored block of 107, 215, 323, 431 and 646 leaves per
+// SM takes 127, 201, 278, 350 and 499 us with it, 138, 217, 290, 364 and 507
+// without; of 1,024 and more the same either way.  (In the copying kernels it
+// costs more registers than it gains: 198 against 146 us at 107 leaves per SM.)
+static bool lat_order(int64_t n, int n_sm) {
+    static const int per_sm = env_knob("KVG_SHA_LAT_LEAVES_PER_SM", 512);
+    return n <= (int64_t)n_sm * per_sm;
+}
+
 static int current_sm_count() {
     static int cache[64] = {};
     int dev = 0;
@@ -1265,7 +1297,8 @@ cudaError_t launch_sha256_leaves(const PageSource &src, int64_t n_pages, uint32_
     // 2-3% faster than a capped, striding grid.
     static const int ctas_per_sm = env_knob("KVG_SHA_CTAS_PER_SM", 0);
     if (ctas_per_sm > 0 && grid > (int64_t)n_sm * ctas_per_sm) grid = (int64_t)n_sm * ctas_per_sm;
-    sha256_leaves_kernel<<<(int)grid, 128, 0, s>>>(src, n_pages, m, leaf_words, 1u);
+    auto *kernel = lat_order(n, n_sm) ? sha256_leaves_kernel<true> : sha256_leaves_kernel<false>;
+    kernel<<<(int)grid, 128, 0, s>>>(src, n_pages, m, leaf_words, 1u);
     count_launches(1);
     return cudaGetLastError();
 }
