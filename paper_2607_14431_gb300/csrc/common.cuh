@@ -132,7 +132,7 @@ struct GraftBatchParams {
     int32_t rotated_only;  // copy kernel: only the key pages of re-based grafts
     // verifying launches cover the jobs [job0, job0 + slice_jobs)
     int64_t job0, slice_jobs;
-    int32_t hash_only;     // the pages are in the cache already: hash them there (re-based grafts: in the store)
+    int32_t hash_only;     // the pages are in the cache already: hash them there (re-based grafts': in the store)
 };
 
 // Position tags, page-table entries and fills of a batch's grafts: a graft's

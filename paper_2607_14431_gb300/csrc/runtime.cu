@@ -1877,28 +1877,31 @@ extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, k
     p.pool = c->pool;
     // the store's RoPE pairing and base, as kvg_graft uses them
     const int rotate = table_delta.empty() ? 0 : s->dims.rope_style == KVG_ROPE_HALF ? 1 : 2;
-    if (!rotate) p.trig = nullptr;
     const bool host_src = s->residency == KVG_RESIDENCY_PINNED_HOST;
     // Verified, from an HBM store: every page is read once, its copy and its
-    // leaf hashes in one pass; only the re-based key pages are written by the
-    // rotating copy before.  From a pinned-host store the copy kernel, whose
-    // wide reads keep the host link at its limit, moves everything and the
-    // hashes follow in the cache (of re-based grafts: in the store).
-    p.write_meta = !verify || host_src;
-    p.rotated_only = verify && !host_src;
-    if (!p.rotated_only || rotate)
-        KVG_CUDA(launch_graft_batch(p, c->n_sm, st, host_src ? host_copy_grid_cap() : 0, rotate));
+    // leaf hashes in one pass, and the rotating copy then writes the key pages of
+    // re-based grafts.  From a pinned-host store the copy kernel, whose wide reads
+    // keep the host link at its limit, moves everything and the hashes follow in
+    // the cache (of re-based grafts: in the store).
+    const int ctas = host_src ? host_copy_grid_cap() : 0;
+    p.write_meta = 1;
+    if (!verify || host_src) {
+        KVG_CUDA(launch_graft_batch(p, c->n_sm, st, ctas, rotate));
+        p.write_meta = 0;
+    }
     if (verify) {
         const uint32_t call = ++c->batch_calls % (1u << 18) + 1;
         p.hash_only = host_src;
         for (p.job0 = 0; p.job0 < pages; p.job0 += slice) {
             p.slice_jobs = std::min(slice, pages - p.job0);
-            p.write_meta = !host_src && p.job0 == 0;
             // the two-warp form's loads are too slow for host memory (re-based grafts hash the store)
             KVG_CUDA(launch_graft_batch_verify(p, static_cast<uint32_t *>(c->leaf.ptr), c->n_sm, st,
                                                c->dims.kv_dtype == KVG_KV_BF16, !(host_src && rotate)));
             KVG_CUDA(launch_graft_batch_pages(p, static_cast<const uint32_t *>(c->leaf.ptr), c->status, call, st));
+            p.write_meta = 0;
         }
+        p.rotated_only = 1;
+        if (rotate && !host_src) KVG_CUDA(launch_graft_batch(p, c->n_sm, st, ctas, rotate));
     }
     return finish_verify(c, n == 1 ? seq_ids[0] : -1, flags,
                          (flags & KVG_GRAFT_VERIFY) ? (int32_t)(c->dims.n_layers * 2 * pages) : 0, st, report);

@@ -167,8 +167,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // busy) hides behind the compressions without costing registers.  (A layout
 // with the 32 lanes' vectors side by side, free of bank conflicts, measured
 // slower in the 12b step: 6.05 against 5.94 ms.)
-// SOME: only when copy_to is not null.
-template <int R, bool SOME = false>
+template <int R>
 __device__ __forceinline__ void hash_leaf_ring(const uint8_t *leaf, uint64_t len, uint8_t *copy_to, uint32_t st[8],
                                                uint32_t one, uint4 *ring) {
     const uint4 *v = reinterpret_cast<const uint4 *>(leaf);
@@ -201,10 +200,8 @@ __device__ __forceinline__ void hash_leaf_ring(const uint8_t *leaf, uint64_t len
 #pragma unroll
             for (int q = 0; q < 4; ++q) cp_async16(ring + 4 * slot + q, v + 4 * (blk + R) + q);
         cp_async_commit();
-        if (!SOME || o) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) __stcs(o + 4 * blk + q, x[q]);
-        }
+        for (int q = 0; q < 4; ++q) __stcs(o + 4 * blk + q, x[q]);
         compress(st, w, one);
     }
     cp_async_wait<0>();
@@ -219,17 +216,15 @@ __device__ __forceinline__ void hash_leaf_ring(const uint8_t *leaf, uint64_t len
         w[15] = (uint32_t)bits;
         compress(st, w, one);
     } else {
-        if (!SOME || o)
-            for (int q = 0; q < rem / 16; ++q) o[4 * nfull + q] = v[4 * nfull + q];
+        for (int q = 0; q < rem / 16; ++q) o[4 * nfull + q] = v[4 * nfull + q];
         finish(st, leaf + (len & ~63ull), rem, len, one);
     }
 }
 
 // SHA-256 of one leaf of `len` bytes (16-byte aligned).  With COPY the leaf
 // is also written to `copy_to`, from the same registers that are hashed, so
-// the bytes written are exactly the bytes whose digest is checked (SOME: only
-// when copy_to is not null).
-template <bool COPY, bool SOME = false, bool LAT = false>
+// the bytes written are exactly the bytes whose digest is checked.
+template <bool COPY, bool LAT = false>
 __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uint8_t *copy_to, uint32_t st[8],
                                           uint32_t one) {
     const uint4 *v = reinterpret_cast<const uint4 *>(leaf);
@@ -257,7 +252,7 @@ __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uin
 #pragma unroll
             for (int q = 0; q < 4; ++q) n2[q] = __ldg(v + 4 * (blk + 2) + q);
         }
-        if (COPY && (!SOME || o)) {
+        if (COPY) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) __stcs(o + 4 * blk + q, x[q]);
         }
@@ -281,7 +276,7 @@ __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uin
         w[15] = (uint32_t)bits;
         compress<true, LAT>(st, w, one);
     } else {
-        if (COPY && (!SOME || o))
+        if (COPY)
             for (int q = 0; q < rem / 16; ++q) o[4 * nfull + q] = v[4 * nfull + q];
         finish(st, leaf + (len & ~63ull), rem, len, one);
     }
@@ -692,7 +687,7 @@ __global__ void __launch_bounds__(128) sha256_leaves_kernel(const PageSource src
             in_range = pid >= 0 && pid < src.plane_pages;
         }
         if (in_range) {
-            hash_leaf<false, false, LAT>(page_addr(src, p) + (uint64_t)i * kLeafBytes, len, nullptr, st, one);
+            hash_leaf<false, LAT>(page_addr(src, p) + (uint64_t)i * kLeafBytes, len, nullptr, st, one);
         } else {
 #pragma unroll
             for (int w = 0; w < 8; ++w) st[w] = 0u;  // no digest of any page: reported as a mismatch
@@ -773,16 +768,19 @@ __global__ void __launch_bounds__(128) graft_verify_kernel(const GraftParams p, 
 // ---- a batch of grafts, verified ------------------------------------------
 // The leaves of a batch's jobs in one launch, so that a batch of short blocks
 // fills the GPU like one long block does: a leaf per thread, leaf fastest,
-// then job, then plane (a block's pages follow one another in a plane).  A graft at its own position is copied and hashed in
-// one pass; a re-based one's value pages too, while its key pages, which the
-// rotating copy has written, are hashed in the store.
+// then job, then plane (a block's pages follow one another in a plane).  COPY:
+// every page is copied and hashed in one pass (the key pages of re-based
+// grafts too: the rotating copy that follows overwrites them; the hashing is
+// what the launch waits for, so writing them twice costs nothing).  Otherwise
+// the pages are in the cache already and are hashed there, re-based grafts' in
+// the store.
 struct BatchLeaf {
     const uint8_t *src;
-    uint8_t *dst;  // null: hash only
+    uint8_t *dst;
     uint64_t len;
 };
 
-template <bool SOME>
+template <bool COPY>
 __device__ __forceinline__ BatchLeaf batch_leaf(const GraftBatchParams &p, int64_t idx, int64_t m) {
     const int64_t page = idx / m;
     const int64_t lkv = page / p.slice_jobs;
@@ -794,49 +792,48 @@ __device__ __forceinline__ BatchLeaf batch_leaf(const GraftBatchParams &p, int64
     if (r.len > kLeafBytes) r.len = kLeafBytes;
     r.src = job.src + (uint64_t)lkv * job.block_pages * p.page_bytes + off;
     r.dst = p.pool + ((uint64_t)lkv * p.pool_pages + (uint64_t)job.pid) * p.page_bytes + off;
-    if (SOME) {
-        const bool rebased = p.metas[job.meta].trig >= 0;
-        if (p.hash_only) {
-            if (!rebased) r.src = r.dst;
-            r.dst = nullptr;
-        } else if (rebased && !(lkv & 1)) {
-            r.dst = nullptr;
-        }
-    }
+    if (!COPY && p.metas[job.meta].trig < 0) r.src = r.dst;
     return r;
 }
 
 // graft_verify_ring_kernel for a batch (the same launch sizes).
-template <bool SOME>
 __global__ void __launch_bounds__(128, 5) graft_batch_verify_ring_kernel(const GraftBatchParams p,
                                                                          int64_t leaves_per_page,
                                                                          uint32_t *__restrict__ out, uint32_t one) {
     constexpr int R = kGraftVerifyRing;
     extern __shared__ __align__(16) uint4 ring_mem[];
     if (p.write_meta) batch_metadata(p);
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= p.slice_jobs * p.n_layers * 2 * leaves_per_page) return;
-    const BatchLeaf l = batch_leaf<SOME>(p, idx, leaves_per_page);
-    uint32_t st[8];
-    hash_leaf_ring<R, SOME>(l.src, l.len, l.dst, st, one, ring_mem + threadIdx.x * 4 * R);
-    store_state(out + idx * 8, st);
+    const int64_t n_leaves = p.slice_jobs * p.n_layers * 2 * leaves_per_page;
+    uint4 *ring = ring_mem + threadIdx.x * 4 * R;
+    // (a loop, though the grid has a thread for every leaf: straight-line, the
+    // compiler's schedule of the compressions ran 13% slower, 4.69 against 4.08 ms
+    // for 1.06 million leaves)
+    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n_leaves;
+         idx += (int64_t)gridDim.x * blockDim.x) {
+        const BatchLeaf l = batch_leaf<true>(p, idx, leaves_per_page);
+        uint32_t st[8];
+        hash_leaf_ring<R>(l.src, l.len, l.dst, st, one, ring);
+        store_state(out + idx * 8, st);
+    }
 }
 
 // graft_verify_kernel for a batch.
-template <bool SOME>
+template <bool COPY>
 __global__ void __launch_bounds__(128) graft_batch_verify_kernel(const GraftBatchParams p, int64_t leaves_per_page,
                                                                  uint32_t *__restrict__ out, uint32_t one) {
     if (p.write_meta) batch_metadata(p);
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= p.slice_jobs * p.n_layers * 2 * leaves_per_page) return;
-    const BatchLeaf l = batch_leaf<SOME>(p, idx, leaves_per_page);
-    uint32_t st[8];
-    hash_leaf<true, SOME>(l.src, l.len, l.dst, st, one);
-    store_state(out + idx * 8, st);
+    const int64_t n_leaves = p.slice_jobs * p.n_layers * 2 * leaves_per_page;
+    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n_leaves;
+         idx += (int64_t)gridDim.x * blockDim.x) {
+        const BatchLeaf l = batch_leaf<COPY>(p, idx, leaves_per_page);
+        uint32_t st[8];
+        hash_leaf<COPY>(l.src, l.len, l.dst, st, one);
+        store_state(out + idx * 8, st);
+    }
 }
 
 // graft_verify_split_kernel for a batch.
-template <bool WIDE>
+template <bool COPY, bool WIDE>
 __global__ void __launch_bounds__(64) graft_batch_verify_split_kernel(const GraftBatchParams p,
                                                                       int64_t leaves_per_page,
                                                                       uint32_t *__restrict__ out, uint32_t one) {
@@ -848,8 +845,8 @@ __global__ void __launch_bounds__(64) graft_batch_verify_split_kernel(const Graf
     const bool valid = idx < p.slice_jobs * p.n_layers * 2 * leaves_per_page;
     if (produce) {
         BatchLeaf l{nullptr, nullptr, 0};
-        if (valid) l = batch_leaf<true>(p, idx, leaves_per_page);
-        split_produce_leaf<true, WIDE>(sm, reinterpret_cast<const uint4 *>(l.src), reinterpret_cast<uint4 *>(l.dst),
+        if (valid) l = batch_leaf<COPY>(p, idx, leaves_per_page);
+        split_produce_leaf<COPY, WIDE>(sm, reinterpret_cast<const uint4 *>(l.src), reinterpret_cast<uint4 *>(l.dst),
                                        lane, one);
     } else {
         split_consume_leaf<WIDE>(sm, valid ? out + idx * 8 : nullptr, false, lane, one);
@@ -1344,18 +1341,17 @@ cudaError_t launch_graft_batch_verify(const GraftBatchParams &p, uint32_t *leaf_
     // the forms and their launch sizes are those of launch_graft_verify
     if (split_ok && !split_off() && p.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
         const bool wide = split_wide(n, n_sm);
-        auto *kernel = wide ? graft_batch_verify_split_kernel<true> : graft_batch_verify_split_kernel<false>;
+        auto *kernel = p.hash_only ? (wide ? graft_batch_verify_split_kernel<false, true>
+                                           : graft_batch_verify_split_kernel<false, false>)
+                                   : (wide ? graft_batch_verify_split_kernel<true, true>
+                                           : graft_batch_verify_split_kernel<true, false>);
         kernel<<<split_grid(n, wide), 64, 0, s>>>(p, m, leaf_words, 1u);
-    } else if (ring_ok && !regs_only() && n >= (int64_t)n_sm * 5 * 128) {
+    } else if (ring_ok && !p.hash_only && !regs_only() && n >= (int64_t)n_sm * 5 * 128) {
         const size_t smem = (size_t)128 * kGraftVerifyRing * 64;
-        if (p.trig || p.hash_only)
-            graft_batch_verify_ring_kernel<true><<<grid, 128, smem, s>>>(p, m, leaf_words, 1u);
-        else
-            graft_batch_verify_ring_kernel<false><<<grid, 128, smem, s>>>(p, m, leaf_words, 1u);
-    } else if (p.trig || p.hash_only) {
-        graft_batch_verify_kernel<true><<<grid, 128, 0, s>>>(p, m, leaf_words, 1u);
+        graft_batch_verify_ring_kernel<<<grid, 128, smem, s>>>(p, m, leaf_words, 1u);
     } else {
-        graft_batch_verify_kernel<false><<<grid, 128, 0, s>>>(p, m, leaf_words, 1u);
+        auto *kernel = p.hash_only ? graft_batch_verify_kernel<false> : graft_batch_verify_kernel<true>;
+        kernel<<<grid, 128, 0, s>>>(p, m, leaf_words, 1u);
     }
     count_launches(1);
     return cudaGetLastError();
