@@ -190,6 +190,16 @@ struct AppendBatchParams {
 };
 
 // --------------------------------------------------------------- deposit --
+// What surrounds a serialized block's rows: its header and the alignment gaps
+// after the position tags and after the page digests, which the layout
+// defines as zero (reused memory is not).
+struct BlockFrame {
+    uint8_t *base;         // start of the block (null: no frame to write)
+    uint64_t gap_off[2];   // from base, multiples of 4
+    uint32_t gap_bytes[2];
+    uint8_t header[256];
+};
+
 struct GatherParams {
     const uint8_t *pool;
     uint8_t *dst;              // block pages region (dst_pids.n == 0), or the pool (dst_pids given)
@@ -197,11 +207,13 @@ struct GatherParams {
     int64_t pool_pages;
     int32_t n_layers, npb, page_base, block_pages;
     int32_t n_kv_heads, page_size, head_dim;
+    int32_t chunk_bytes;       // unit of work: divides page_bytes, whole rows
     int64_t n_tokens;          // rows >= n_tokens are written as zero
     const int32_t *src_pos;    // positions row + slot0 (nullable: no position copy)
     int32_t *dst_pos;          // block positions
     PageList pids;             // source pool pages
     PageList dst_pids;         // destination pool pages (pool-resident blocks), n = 0 when unused
+    BlockFrame frame;
 };
 
 // Own-position graft by aliasing: page-table entries, fills and position
@@ -219,11 +231,6 @@ struct AliasParams {
 struct IntsParams {
     int32_t *dst;
     PageList vals;
-};
-
-struct HeaderParams {
-    uint8_t *dst;
-    uint8_t bytes[256];
 };
 
 // ---------------------------------------------------------------- digest --
@@ -326,7 +333,6 @@ cudaError_t launch_graft_batch_pages(const GraftBatchParams &p, const uint32_t *
 cudaError_t launch_append(const AppendParams &p, int n_sm, cudaStream_t s);
 cudaError_t launch_append_batch(const AppendBatchParams &p, int n_sm, cudaStream_t s);
 cudaError_t launch_gather(const GatherParams &p, int n_sm, cudaStream_t s);
-cudaError_t launch_write_header(const HeaderParams &p, cudaStream_t s);
 cudaError_t launch_alias(const AliasParams &p, int n_sm, cudaStream_t s);
 // One 4-byte load per `stride` bytes of [base, base + bytes) (base 4-byte
 // aligned, stride a multiple of 4): resolves the GPU's address translations
@@ -351,6 +357,18 @@ cudaError_t launch_sha256_pages(const uint32_t *leaf_words, int64_t n_pages, int
 cudaError_t launch_sha256_serial(const uint8_t *seg0, uint64_t n0, const uint8_t *seg1, uint64_t n1,
                                  uint8_t *out, const uint8_t *expected, DevStatus *status,
                                  cudaStream_t s);
+// The same digest in parts, for 4-byte aligned segments and n0 a multiple of
+// 4: the message's 64-byte blocks [b0, b1) of serial_blocks(n0 + n1) (the
+// padding included), from the state at `state` (b0 = 0: the initial one);
+// the part that ends the message writes the digest, the others the state.
+// state and out may be the same 32 bytes (16-byte aligned).
+int64_t serial_blocks(uint64_t bytes);
+cudaError_t launch_sha256_serial_part(const uint8_t *seg0, uint64_t n0, const uint8_t *seg1, uint64_t n1, int64_t b0,
+                                      int64_t b1, uint8_t *state, uint8_t *out, cudaStream_t s);
+// Whether the hashing in parts is there (the two-warp forms are not turned off).
+bool sha256_parts_ok();
+// Leaves in a launch that gives every scheduler of the device one warp of them.
+int64_t sha256_wave_leaves(int n_sm);
 
 // Persistent decode: p.n_warps one-warp CTAs over p.n_tiles tiles, then the
 // combine over every (layer, row, query head).  decode_tile_tokens() is the

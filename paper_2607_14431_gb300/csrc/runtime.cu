@@ -232,8 +232,9 @@ struct kvg_store {
     // deposits: the block digest (one serial SHA-256 chain) runs on its own
     // stream after the page digests; a pinned-host store's blocks are
     // assembled and hashed in an HBM staging buffer, then copied out
-    cudaStream_t digest_stream = nullptr;
-    cudaEvent_t pages_done = nullptr, stage_free = nullptr;
+    // (page_stream: the page digests of a block hashed in several chunks)
+    cudaStream_t digest_stream = nullptr, page_stream = nullptr;
+    cudaEvent_t pages_done = nullptr, stage_free = nullptr, chunk_done = nullptr;
     bool pages_recorded = false;  // a deposit's page hashing (which uses `leaf`) may still run
     bool stage_used = false;
     Scratch stage;
@@ -352,6 +353,8 @@ extern "C" void kvg_store_destroy(kvg_store *s) {
     for (cudaStream_t st : s->load_streams) cudaStreamDestroy(st);
     for (cudaEvent_t e : s->load_events) cudaEventDestroy(e);
     if (s->digest_stream) cudaStreamDestroy(s->digest_stream);
+    if (s->page_stream) cudaStreamDestroy(s->page_stream);
+    if (s->chunk_done) cudaEventDestroy(s->chunk_done);
     if (s->pages_done) cudaEventDestroy(s->pages_done);
     if (s->stage_free) cudaEventDestroy(s->stage_free);
     s->stage.release();
@@ -416,15 +419,16 @@ static kvg_status hash_block(kvg_store *s, uint8_t *blk_dev, const BlockLayout &
     return KVG_OK;
 }
 
-// Zeroes a serialized block's alignment gaps (after the position tags and
-// after the page digests): the layout defines them as zero, and reused
-// memory (a staging buffer, a slab freed and allocated again) is not.
-static kvg_status zero_block_gaps(uint8_t *base, const BlockLayout &lay, int32_t n_layers, cudaStream_t st) {
+// The frame of a serialized block at base, written by the deposit's gather.
+static void block_frame(BlockFrame *f, uint8_t *base, const kvg_dims &d, const BlockLayout &lay) {
     const uint64_t pos_end = lay.pos_off + 4ull * (uint64_t)lay.n_tokens;
-    const uint64_t dig_end = lay.dig_off + (uint64_t)n_layers * 2 * (uint64_t)lay.n_pages * 32;
-    if (lay.dig_off > pos_end) KVG_CUDA(cudaMemsetAsync(base + pos_end, 0, lay.dig_off - pos_end, st));
-    if (lay.pages_off > dig_end) KVG_CUDA(cudaMemsetAsync(base + dig_end, 0, lay.pages_off - dig_end, st));
-    return KVG_OK;
+    const uint64_t dig_end = lay.dig_off + (uint64_t)d.n_layers * 2 * (uint64_t)lay.n_pages * 32;
+    f->base = base;
+    f->gap_off[0] = pos_end;
+    f->gap_bytes[0] = (uint32_t)(lay.dig_off - pos_end);
+    f->gap_off[1] = dig_end;
+    f->gap_bytes[1] = (uint32_t)(lay.pages_off - dig_end);
+    build_header(f->header, d, lay);
 }
 
 static void minmax_positions(const int32_t *pos, int64_t n, int64_t *mn, int64_t *mx) {
@@ -1222,17 +1226,13 @@ static kvg_status pool_deposit(kvg_store *s, kvg_cache *c, int32_t seq, int32_t 
     if (stt != KVG_OK) return stt;
     auto pids = take_pages(c, lay.n_pages);
     for (int32_t pid : pids) c->pinned[pid] = 1;
-    HeaderParams hp;
-    hp.dst = meta;
-    build_header(hp.bytes, s->dims, lay);
-    KVG_CUDA(launch_write_header(hp, st));
-    stt = zero_block_gaps(meta, lay, s->dims.n_layers, st);
-    if (stt != KVG_OK) return stt;
     const int64_t P = c->dims.page_size;
     const auto &sp = c->seq_pages[seq];
     const int64_t j_first = slot0 / P;
     for (int64_t base = 0; base < lay.n_pages; base += kMaxPagesPerLaunch) {
         GatherParams p{};
+        if (base == 0) block_frame(&p.frame, meta, s->dims, lay);
+        p.chunk_bytes = copy_chunk_bytes(c->dims);
         p.pool = c->pool;
         p.dst = c->pool;
         p.page_bytes = c->page_bytes;
@@ -1289,6 +1289,8 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (!s->digest_stream) {
         KVG_CUDA(cudaStreamCreateWithFlags(&s->digest_stream, cudaStreamNonBlocking));
+        KVG_CUDA(cudaStreamCreateWithFlags(&s->page_stream, cudaStreamNonBlocking));
+        KVG_CUDA(cudaEventCreateWithFlags(&s->chunk_done, cudaEventDisableTiming));
         KVG_CUDA(cudaEventCreateWithFlags(&s->pages_done, cudaEventDisableTiming));
         KVG_CUDA(cudaEventCreateWithFlags(&s->stage_free, cudaEventDisableTiming));
     }
@@ -1308,16 +1310,12 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
         }
         tgt = static_cast<uint8_t *>(s->stage.ptr);
     }
-    HeaderParams hp;
-    hp.dst = tgt;
-    build_header(hp.bytes, s->dims, lay);
-    KVG_CUDA(launch_write_header(hp, st));
-    stt = zero_block_gaps(tgt, lay, s->dims.n_layers, st);
-    if (stt != KVG_OK) return stt;
     const auto &sp = c->seq_pages[seq];
     const int64_t j_first = slot0 / P;
     for (int64_t base = 0; base < lay.n_pages; base += kMaxPagesPerLaunch) {
         GatherParams p{};
+        if (base == 0) block_frame(&p.frame, tgt, s->dims, lay);
+        p.chunk_bytes = copy_chunk_bytes(c->dims);
         p.pool = c->pool;
         p.dst = tgt + lay.pages_off;
         p.page_bytes = c->page_bytes;
@@ -1336,36 +1334,79 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
         for (int32_t i = 0; i < p.npb; ++i) p.pids.pid[i] = sp[j_first + base + i];
         KVG_CUDA(launch_gather(p, s->n_sm, st));
     }
-    // the position tags bound later relocations (host-side checks): read once
-    std::vector<int32_t> pos(n);
-    KVG_CUDA(cudaMemcpyAsync(pos.data(), tgt + lay.pos_off, 4ull * n, cudaMemcpyDeviceToHost, st));
-    KVG_CUDA(cudaStreamSynchronize(st));
-    // page digests on the caller's stream; the block digest (one serial chain
-    // over the position tags and every page digest) on the store's digest
-    // stream, so the call does not wait for it and consecutive deposits
-    // overlap it.  Everything that reads a block digest (block info, export,
-    // save) synchronizes the device first.
+    // Digests.  The block digest is one serial chain over the position tags
+    // and the page digests in order, so a long block is hashed in chunks of
+    // pages: while one chunk's leaves are hashed on the caller's stream, the
+    // page digests of the one before follow on the store's page stream and
+    // the chain over those on its digest stream (its state waits in the
+    // header's digest field between chunks).  A chunk is at least a leaf for
+    // every thread of one warp per scheduler, which hashes as many leaves a
+    // second as fuller launches do; the chain is slower than the hashing, so
+    // later chunks grow.  The call waits for the rows (it reads the position
+    // tags back, which bound later relocations) but not for the digests, and
+    // everything that reads a block digest (block info, export, save)
+    // synchronizes the device first.
     const kvg_dims &d = s->dims;
     const uint64_t pb = page_bytes_of(d);
     const int64_t m = (int64_t)((pb + kLeafBytes - 1) / kLeafBytes);
     const int64_t n_pages = (int64_t)d.n_layers * 2 * lay.n_pages;
+    const uint64_t pos_bytes = 4ull * n;
+    KVG_CUDA(cudaEventRecord(s->chunk_done, st));
+    KVG_CUDA(cudaStreamWaitEvent(s->page_stream, s->chunk_done, 0));  // the rows are gathered
     KVG_CUDA(wait_for_leaf_scratch(s, st));
     KVG_CUDA(s->leaf.ensure((size_t)n_pages * m * 32));
-    PageSource src{tgt + lay.pages_off, pb, nullptr, 1, 0};
     uint32_t *leaf = static_cast<uint32_t *>(s->leaf.ptr);
-    KVG_CUDA(launch_sha256_leaves(src, n_pages, leaf, s->n_sm, st));
-    KVG_CUDA(launch_sha256_pages(leaf, n_pages, m, tgt + lay.dig_off, nullptr, s->status, -1, st));
-    KVG_CUDA(cudaEventRecord(s->pages_done, st));
-    s->pages_recorded = true;
-    KVG_CUDA(cudaStreamWaitEvent(s->digest_stream, s->pages_done, 0));
-    KVG_CUDA(launch_sha256_serial(tgt + lay.pos_off, 4ull * n, tgt + lay.dig_off, (uint64_t)n_pages * 32, tgt + 96,
-                                  nullptr, s->status, s->digest_stream));
+    const int64_t wave = std::max<int64_t>(1, sha256_wave_leaves(s->n_sm) / m);
+    const bool parts = sha256_parts_ok() && n_pages > wave + wave / 4 &&
+                       serial_blocks(pos_bytes + (uint64_t)n_pages * 32) < (1ll << 30);
+    std::vector<int32_t> pos(n);
+    double grow = 1.0;
+    int64_t chained = 0;  // blocks of the chain enqueued so far
+    for (int64_t p0 = 0; p0 < n_pages;) {
+        int64_t np = parts ? wave * std::max<int64_t>(1, (int64_t)grow) : n_pages;
+        if (n_pages - p0 - np < wave / 2) np = n_pages - p0;
+        grow *= 1.3;
+        const PageSource src{tgt + lay.pages_off + (uint64_t)p0 * pb, pb, nullptr, 1, 0};
+        KVG_CUDA(launch_sha256_leaves(src, np, leaf + p0 * m * 8, s->n_sm, st));
+        if (p0 == 0) {
+            KVG_CUDA(cudaMemcpyAsync(pos.data(), tgt + lay.pos_off, pos_bytes, cudaMemcpyDeviceToHost,
+                                     s->page_stream));
+            KVG_CUDA(cudaStreamSynchronize(s->page_stream));
+        }
+        cudaStream_t ps = parts ? s->page_stream : st;
+        if (parts) {
+            KVG_CUDA(cudaEventRecord(s->chunk_done, st));
+            KVG_CUDA(cudaStreamWaitEvent(ps, s->chunk_done, 0));
+        }
+        KVG_CUDA(launch_sha256_pages(leaf + p0 * m * 8, np, m, tgt + lay.dig_off + (uint64_t)p0 * 32, nullptr,
+                                     s->status, -1, ps));
+        KVG_CUDA(cudaEventRecord(s->pages_done, ps));
+        s->pages_recorded = true;
+        KVG_CUDA(cudaStreamWaitEvent(s->digest_stream, s->pages_done, 0));
+        p0 += np;
+        if (parts) {
+            const uint64_t total = pos_bytes + (uint64_t)n_pages * 32;
+            const int64_t b1 = p0 == n_pages ? serial_blocks(total) : (int64_t)((pos_bytes + (uint64_t)p0 * 32) / 64);
+            KVG_CUDA(launch_sha256_serial_part(tgt + lay.pos_off, pos_bytes, tgt + lay.dig_off,
+                                               (uint64_t)n_pages * 32, chained, b1, tgt + 96, tgt + 96,
+                                               s->digest_stream));
+            chained = b1;
+        } else {
+            KVG_CUDA(launch_sha256_serial(tgt + lay.pos_off, pos_bytes, tgt + lay.dig_off, (uint64_t)n_pages * 32,
+                                          tgt + 96, nullptr, s->status, s->digest_stream));
+        }
+    }
+    if (parts) KVG_CUDA(cudaStreamWaitEvent(st, s->pages_done, 0));  // later work on the caller's stream
     if (host) {
         // everything but the header follows the page digests on the caller's
         // stream; the header (with the block digest) follows the digest
         KVG_CUDA(cudaMemcpyAsync(host + lay.pos_off, tgt + lay.pos_off, lay.total - lay.pos_off,
                                  cudaMemcpyDeviceToHost, st));
         KVG_CUDA(cudaMemcpyAsync(host, tgt, lay.pos_off, cudaMemcpyDeviceToHost, s->digest_stream));
+        // both copies have read the staging buffer before the next deposit, on
+        // whatever stream, fills it
+        KVG_CUDA(cudaEventRecord(s->chunk_done, st));
+        KVG_CUDA(cudaStreamWaitEvent(s->digest_stream, s->chunk_done, 0));
         KVG_CUDA(cudaEventRecord(s->stage_free, s->digest_stream));
         s->stage_used = true;
     }
@@ -1487,6 +1528,7 @@ static kvg_status pool_graft(kvg_store *s, const kvg_store::Blk &blk, kvg_cache 
         p.n_kv_heads = c->dims.n_kv_heads;
         p.page_size = (int32_t)P;
         p.head_dim = c->dims.head_dim;
+        p.chunk_bytes = copy_chunk_bytes(c->dims);
         p.n_tokens = n;
         p.src_pos = nullptr;
         p.pids.n = 1;

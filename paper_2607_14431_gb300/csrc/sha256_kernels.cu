@@ -433,14 +433,14 @@ __device__ __forceinline__ bool split_begin(SplitShared &sm) {
     return (int)(threadIdx.x >> 5) != sm.consumer;
 }
 
-// The rounds' warp over a chain of n_blocks blocks: its half of the state from H0
-// to the digest.
+// The rounds' warp over a chain of n_blocks blocks: its half of the state from
+// H0 (from: a stored state's words) to the digest.
 __device__ __forceinline__ void split_consume(uint32_t st[4], const SplitShared &sm, int n_blocks, int lane,
-                                              uint32_t one) {
+                                              uint32_t one, const uint32_t *from = nullptr) {
     const SplitRole ro = split_role(lane);
     const int c = lane & (kSplitChains - 1);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) st[i] = ro.a ? kH0[i] : kH0[4 + i];
+    for (int i = 0; i < 4; ++i) st[i] = from ? from[i + (ro.a ? 0 : 4)] : kH0[i + (ro.a ? 0 : 4)];
     const int n_pairs = (n_blocks + 1) >> 1;
     for (int k = 0; k < n_pairs; ++k) {
         const int buf = k & 1;
@@ -1161,10 +1161,14 @@ __device__ __forceinline__ uint32_t padded_word(const uint8_t *seg0, uint64_t n0
     return v;
 }
 
+// Blocks [b0, b1) of the padded message's n_blocks, from the state `from`
+// (b0 > 0).  The part that ends the message writes the digest to out and/or
+// compares it with expected; the others write the state to `to`.
 __global__ void __launch_bounds__(64) sha256_serial_split_kernel(const uint8_t *seg0, uint64_t n0, const uint8_t *seg1,
-                                                                 uint64_t n1, int32_t n_blocks, uint8_t *out,
-                                                                 const uint8_t *expected, DevStatus *status,
-                                                                 uint32_t one) {
+                                                                 uint64_t n1, int32_t b0, int32_t b1,
+                                                                 int32_t n_blocks, const uint32_t *from, uint32_t *to,
+                                                                 uint8_t *out, const uint8_t *expected,
+                                                                 DevStatus *status, uint32_t one) {
     __shared__ SplitShared sm;
     const bool produce = split_begin(sm);
     const int lane = threadIdx.x & 31;
@@ -1172,21 +1176,23 @@ __global__ void __launch_bounds__(64) sha256_serial_split_kernel(const uint8_t *
     if (produce) {
         const uint64_t whole = (n0 + n1) / 64;  // blocks without padding
         uint32_t n1w[16], n2w[16];
-        // block blk as big-endian words (past the message: zeros)
+        // block blk as big-endian words (past the part: zeros)
         auto load = [&](uint32_t w[16], int blk) {
-            if ((uint64_t)blk < whole) {
+            if (blk >= b1) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) w[i] = 0u;
+            } else if ((uint64_t)blk < whole) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) w[i] = bswap(msg_word(seg0, n0, seg1, 16ull * blk + i));
             } else {
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    w[i] = blk < n_blocks ? padded_word(seg0, n0, seg1, n1, n_blocks, 16ull * blk + i) : 0u;
+                for (int i = 0; i < 16; ++i) w[i] = padded_word(seg0, n0, seg1, n1, n_blocks, 16ull * blk + i);
             }
         };
-        const int half = lane / kSplitChains;
-        const int n_pairs = (n_blocks + 1) >> 1;
-        load(n1w, half);
-        load(n2w, 2 + half);
+        const int first = b0 + lane / kSplitChains;
+        const int n_pairs = (b1 - b0 + 1) >> 1;
+        load(n1w, first);
+        load(n2w, first + 2);
         for (int k = 0; k < n_pairs; ++k) {
             uint32_t w[16];
 #pragma unroll
@@ -1194,32 +1200,26 @@ __global__ void __launch_bounds__(64) sha256_serial_split_kernel(const uint8_t *
                 w[i] = n1w[i];
                 n1w[i] = n2w[i];
             }
-            if (k + 2 < n_pairs) load(n2w, 2 * (k + 2) + half);
+            if (k + 2 < n_pairs) load(n2w, first + 2 * (k + 2));
             split_hand_over(sm, w, k, lane, one);
         }
         return;
     }
     uint32_t st[4], full[8];
-    split_consume(st, sm, n_blocks, lane, one);
+    split_consume(st, sm, b1 - b0, lane, one, b0 > 0 ? from : nullptr);
     split_whole_state(full, st);
     if (lane != 0) return;
-    uint8_t dg[32];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        dg[4 * k + 0] = (uint8_t)(full[k] >> 24);
-        dg[4 * k + 1] = (uint8_t)(full[k] >> 16);
-        dg[4 * k + 2] = (uint8_t)(full[k] >> 8);
-        dg[4 * k + 3] = (uint8_t)full[k];
+    if (b1 < n_blocks) {
+        store_state(to, full);
+        return;
     }
-    if (out)
-        for (int k = 0; k < 32; ++k) out[k] = dg[k];
-    if (expected) {
-        bool same = true;
-        for (int k = 0; k < 32; ++k) same &= dg[k] == expected[k];
-        if (!same) {
-            atomicAdd(&status->n_mismatch, 1);
-            atomicCAS(&status->err, 0, (int32_t)KVG_ERR_DIGEST);
-        }
+    if (out) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) reinterpret_cast<uint32_t *>(out)[k] = bswap(full[k]);
+    }
+    if (expected && digest_differs(full, expected)) {
+        atomicAdd(&status->n_mismatch, 1);
+        atomicCAS(&status->err, 0, (int32_t)KVG_ERR_DIGEST);
     }
 }
 
@@ -1384,16 +1384,33 @@ cudaError_t launch_graft_batch_pages(const GraftBatchParams &p, const uint32_t *
                         BatchCheck{p.jobs, p.metas, p.job0, p.slice_jobs, call, status}, s);
 }
 
+int64_t serial_blocks(uint64_t bytes) { return (int64_t)((bytes + 9 + 63) / 64); }
+bool sha256_parts_ok() { return !split_off(); }
+int64_t sha256_wave_leaves(int n_sm) { return (int64_t)n_sm * 128; }
+
 cudaError_t launch_sha256_serial(const uint8_t *seg0, uint64_t n0, const uint8_t *seg1, uint64_t n1,
                                  uint8_t *out, const uint8_t *expected, DevStatus *status,
                                  cudaStream_t s) {
-    const bool aligned = !((reinterpret_cast<uintptr_t>(seg0) | reinterpret_cast<uintptr_t>(seg1) | n0) & 3);
-    const uint64_t n_blocks = (n0 + n1 + 9 + 63) / 64;  // with the padding
-    if (!split_off() && aligned && n_blocks < (1ull << 30)) {
-        sha256_serial_split_kernel<<<1, 64, 0, s>>>(seg0, n0, seg1, n1, (int32_t)n_blocks, out, expected, status, 1u);
+    const bool aligned = !((reinterpret_cast<uintptr_t>(seg0) | reinterpret_cast<uintptr_t>(seg1) |
+                            reinterpret_cast<uintptr_t>(out) | n0) & 3);
+    const int64_t n_blocks = serial_blocks(n0 + n1);
+    if (!split_off() && aligned && n_blocks < (1ll << 30)) {
+        sha256_serial_split_kernel<<<1, 64, 0, s>>>(seg0, n0, seg1, n1, 0, (int32_t)n_blocks, (int32_t)n_blocks,
+                                                    nullptr, nullptr, out, expected, status, 1u);
     } else {
         sha256_serial_kernel<<<1, 32, 0, s>>>(seg0, n0, seg1, n1, out, expected, status, 1u);
     }
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sha256_serial_part(const uint8_t *seg0, uint64_t n0, const uint8_t *seg1, uint64_t n1, int64_t b0,
+                                      int64_t b1, uint8_t *state, uint8_t *out, cudaStream_t s) {
+    if (b1 <= b0) return cudaSuccess;
+    sha256_serial_split_kernel<<<1, 64, 0, s>>>(seg0, n0, seg1, n1, (int32_t)b0, (int32_t)b1,
+                                                (int32_t)serial_blocks(n0 + n1),
+                                                reinterpret_cast<const uint32_t *>(state),
+                                                reinterpret_cast<uint32_t *>(state), out, nullptr, nullptr, 1u);
     count_launches(1);
     return cudaGetLastError();
 }
