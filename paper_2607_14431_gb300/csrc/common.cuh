@@ -345,9 +345,12 @@ cudaError_t launch_write_ints(const IntsParams &p, cudaStream_t s);
 cudaError_t launch_reset_seq(int32_t *table_row, int32_t *fill_row, int32_t max_pages,
                              int32_t *pos_row, int32_t max_slots, cudaStream_t s);
 
-// leaf digests (8 uint32 words per leaf, host order of the hash state)
+// leaf digests (8 uint32 words per leaf, host order of the hash state);
+// split_ok: a small launch may take the two-warp form; max_ctas > 0 caps the
+// grid of the one-warp form (CTAs of kLeafCtaThreads leaves at a time).
+constexpr int kLeafCtaThreads = 128;
 cudaError_t launch_sha256_leaves(const PageSource &src, int64_t n_pages, uint32_t *leaf_words,
-                                 int n_sm, cudaStream_t s);
+                                 int n_sm, cudaStream_t s, bool split_ok = true, int max_ctas = 0);
 // page digests from leaf digests; writes out (nullable, 32 bytes per page) and
 // compares with expected (nullable), recording mismatches in status.
 cudaError_t launch_sha256_pages(const uint32_t *leaf_words, int64_t n_pages, int64_t leaves_per_page,
@@ -367,8 +370,6 @@ cudaError_t launch_sha256_serial_part(const uint8_t *seg0, uint64_t n0, const ui
                                       int64_t b1, uint8_t *state, uint8_t *out, cudaStream_t s);
 // Whether the hashing in parts is there (the two-warp forms are not turned off).
 bool sha256_parts_ok();
-// Leaves in a launch that gives every scheduler of the device one warp of them.
-int64_t sha256_wave_leaves(int n_sm);
 
 // Persistent decode: p.n_warps one-warp CTAs over p.n_tiles tiles, then the
 // combine over every (layer, row, query head).  decode_tile_tokens() is the

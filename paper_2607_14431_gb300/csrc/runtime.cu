@@ -1269,6 +1269,8 @@ static kvg_status pool_deposit(kvg_store *s, kvg_cache *c, int32_t seq, int32_t 
     return KVG_OK;
 }
 
+constexpr int kChainSms = 8;  // SMs a long deposit's leaf hashes leave free
+
 extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq, int32_t slot0, int32_t n,
                                   void *stream, uint64_t *block_id_out) {
     Trace trace_("kvg_deposit");
@@ -1339,10 +1341,13 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
     // pages: while one chunk's leaves are hashed on the caller's stream, the
     // page digests of the one before follow on the store's page stream and
     // the chain over those on its digest stream (its state waits in the
-    // header's digest field between chunks).  A chunk is at least a leaf for
-    // every thread of one warp per scheduler, which hashes as many leaves a
-    // second as fuller launches do; the chain is slower than the hashing, so
-    // later chunks grow.  The call waits for the rows (it reads the position
+    // header's digest field between chunks).  The chain is what the whole waits
+    // for, so the leaf hashes leave it alone: one CTA (a warp per scheduler) on
+    // all but kChainSms of the SMs, which still hashes 1.2 times what the chain
+    // takes in, and the page digests and the chain have the others to themselves
+    // (beside a leaf CTA a page chunk's digests took 92 us instead of 35, and a
+    // block of the chain 0.88 instead of 0.80).  A chunk is one round of those
+    // CTAs; later ones grow, since the hashing runs ahead.  The call waits for the rows (it reads the position
     // tags back, which bound later relocations) but not for the digests, and
     // everything that reads a block digest (block info, export, save)
     // synchronizes the device first.
@@ -1356,7 +1361,8 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
     KVG_CUDA(wait_for_leaf_scratch(s, st));
     KVG_CUDA(s->leaf.ensure((size_t)n_pages * m * 32));
     uint32_t *leaf = static_cast<uint32_t *>(s->leaf.ptr);
-    const int64_t wave = std::max<int64_t>(1, sha256_wave_leaves(s->n_sm) / m);
+    const int leaf_ctas = std::max(1, s->n_sm - kChainSms);
+    const int64_t wave = std::max<int64_t>(1, (int64_t)leaf_ctas * kLeafCtaThreads / m);
     const bool parts = sha256_parts_ok() && n_pages > wave + wave / 4 &&
                        serial_blocks(pos_bytes + (uint64_t)n_pages * 32) < (1ll << 30);
     std::vector<int32_t> pos(n);
@@ -1367,7 +1373,7 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
         if (n_pages - p0 - np < wave / 2) np = n_pages - p0;
         grow *= 1.3;
         const PageSource src{tgt + lay.pages_off + (uint64_t)p0 * pb, pb, nullptr, 1, 0};
-        KVG_CUDA(launch_sha256_leaves(src, np, leaf + p0 * m * 8, s->n_sm, st));
+        KVG_CUDA(launch_sha256_leaves(src, np, leaf + p0 * m * 8, s->n_sm, st, !parts, parts ? leaf_ctas : 0));
         if (p0 == 0) {
             KVG_CUDA(cudaMemcpyAsync(pos.data(), tgt + lay.pos_off, pos_bytes, cudaMemcpyDeviceToHost,
                                      s->page_stream));

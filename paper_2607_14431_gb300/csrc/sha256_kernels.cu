@@ -1277,11 +1277,11 @@ static bool regs_only() {
 }
 
 cudaError_t launch_sha256_leaves(const PageSource &src, int64_t n_pages, uint32_t *leaf_words,
-                                 int n_sm, cudaStream_t s) {
+                                 int n_sm, cudaStream_t s, bool split_ok, int max_ctas) {
     const int64_t m = (int64_t)((src.page_bytes + kLeafBytes - 1) / kLeafBytes);
     const int64_t n = n_pages * m;
     if (n == 0) return cudaSuccess;
-    if (!split_off() && src.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
+    if (split_ok && !split_off() && src.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
         const bool wide = split_wide(n, n_sm);
         auto *kernel = wide ? sha256_leaves_split_kernel<true> : sha256_leaves_split_kernel<false>;
         kernel<<<split_grid(n, wide), 64, 0, s>>>(src, n_pages, m, leaf_words, 1u);
@@ -1294,6 +1294,7 @@ cudaError_t launch_sha256_leaves(const PageSource &src, int64_t n_pages, uint32_
     // 2-3% faster than a capped, striding grid.
     static const int ctas_per_sm = env_knob("KVG_SHA_CTAS_PER_SM", 0);
     if (ctas_per_sm > 0 && grid > (int64_t)n_sm * ctas_per_sm) grid = (int64_t)n_sm * ctas_per_sm;
+    if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
     auto *kernel = lat_order(n, n_sm) ? sha256_leaves_kernel<true> : sha256_leaves_kernel<false>;
     kernel<<<(int)grid, 128, 0, s>>>(src, n_pages, m, leaf_words, 1u);
     count_launches(1);
@@ -1386,7 +1387,6 @@ cudaError_t launch_graft_batch_pages(const GraftBatchParams &p, const uint32_t *
 
 int64_t serial_blocks(uint64_t bytes) { return (int64_t)((bytes + 9 + 63) / 64); }
 bool sha256_parts_ok() { return !split_off(); }
-int64_t sha256_wave_leaves(int n_sm) { return (int64_t)n_sm * 128; }
 
 cudaError_t launch_sha256_serial(const uint8_t *seg0, uint64_t n0, const uint8_t *seg1, uint64_t n1,
                                  uint8_t *out, const uint8_t *expected, DevStatus *status,
