@@ -120,28 +120,33 @@ struct Cfg {
 struct TilePos {
     int lr, b, g;
     int64_t unit;
-    int tile;
+    int tile, n_tiles;  // index within the unit, tiles of the unit
+    int grp;            // the layer's group
 };
 
 __device__ __forceinline__ TilePos locate(const DecodeParams &p, int64_t t) {
-    const int64_t sumT = p.rows.pref_tiles[p.B];
-    const int64_t per_layer = (int64_t)p.n_kv_heads * sumT;
     TilePos r;
-    r.lr = (int)(t / per_layer);
-    const int64_t rem = t - (int64_t)r.lr * per_layer;
+    r.grp = t >= p.tile1;
+    if (r.grp) t -= p.tile1;
+    const GroupRows &rows = p.rows[r.grp];
+    const int64_t sumT = rows.pref_tiles[p.B];
+    const int64_t per_layer = (int64_t)p.n_kv_heads * sumT;
+    const int l = (int)(t / per_layer);
+    const int64_t rem = t - (int64_t)l * per_layer;
+    r.lr = l + (r.grp ? p.layer1 : 0);
     int lo = 0, hi = p.B - 1;  // largest b with Hkv * pref[b] <= rem
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if ((int64_t)p.n_kv_heads * p.rows.pref_tiles[mid] <= rem)
+        if ((int64_t)p.n_kv_heads * rows.pref_tiles[mid] <= rem)
             lo = mid;
         else
             hi = mid - 1;
     }
     r.b = lo;
-    const int64_t r2 = rem - (int64_t)p.n_kv_heads * p.rows.pref_tiles[lo];
-    const int Tb = p.rows.pref_tiles[lo + 1] - p.rows.pref_tiles[lo];
-    r.g = (int)(r2 / Tb);
-    r.tile = (int)(r2 - (int64_t)r.g * Tb);
+    const int64_t r2 = rem - (int64_t)p.n_kv_heads * rows.pref_tiles[lo];
+    r.n_tiles = rows.pref_tiles[lo + 1] - rows.pref_tiles[lo];
+    r.g = (int)(r2 / r.n_tiles);
+    r.tile = (int)(r2 - (int64_t)r.g * r.n_tiles);
     r.unit = ((int64_t)r.lr * p.B + r.b) * p.n_kv_heads + r.g;
     return r;
 }
@@ -260,12 +265,12 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
         cur.lr = tp.lr;
         cur.b = tp.b;
         cur.g = tp.g;
-        cur.seq = p.rows.seq[tp.b];
-        const int tile = tp.tile + p.rows.tile0[tp.b];
+        cur.seq = p.seq[tp.b];
+        const int tile = tp.tile + p.rows[tp.grp].tile0[tp.b];
         cur.jj = tile / tpp;
         cur.k = tile - cur.jj * tpp;
-        cur.lo = tp.tile == 0 ? p.rows.lo[tp.b] : 0;
-        cur.end = cur.t - tp.tile + (p.rows.pref_tiles[tp.b + 1] - p.rows.pref_tiles[tp.b]);
+        cur.lo = tp.tile == 0 ? p.rows[tp.grp].lo[tp.b] : 0;
+        cur.end = cur.t - tp.tile + tp.n_tiles;
     };
 
     // The page-table entry and fill of the next tile to issue are loaded one
@@ -417,7 +422,7 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
             if (cur_unit >= 0) flush(cur_unit);
             begin(tp);
             cur_unit = tp.unit;
-            unit_end = t - tp.tile + (p.rows.pref_tiles[tp.b + 1] - p.rows.pref_tiles[tp.b]);
+            unit_end = t - tp.tile + tp.n_tiles;
         }
         const bool ok = mbar_wait_bounded(&bars[stg], par);
         if (!__all_sync(0xffffffffu, ok)) {
@@ -627,12 +632,14 @@ __device__ __forceinline__ Merged<D> merge_partials(const DecodeParams &p, int h
     const int g = h / G, hh = h - g * G;
     const int d4 = threadIdx.x % LANES, r = threadIdx.x / LANES, R = blockDim.x / LANES;
     Merged<D> res{make_float4(0.f, 0.f, 0.f, 0.f), -INFINITY, 0.f};
-    const int64_t Tb = p.rows.pref_tiles[b + 1] - p.rows.pref_tiles[b];
+    const int grp = lr >= p.layer1;
+    const int32_t *pref = p.rows[grp].pref_tiles;
+    const int64_t Tb = pref[b + 1] - pref[b];
     if (Tb <= 0) return res;  // the whole block
     const int64_t T = p.n_tiles, W = p.n_warps;
     const int64_t unit = ((int64_t)lr * p.B + b) * p.n_kv_heads + g;
-    const int64_t first = (int64_t)p.n_kv_heads * ((int64_t)lr * p.rows.pref_tiles[p.B] + p.rows.pref_tiles[b]) +
-                          (int64_t)g * Tb;
+    const int64_t first = (grp ? p.tile1 : 0) + (int64_t)g * Tb +
+                          (int64_t)p.n_kv_heads * ((int64_t)(lr - (grp ? p.layer1 : 0)) * pref[p.B] + pref[b]);
     const int64_t wa = warp_of(first, T, W);
     const int n = (int)(warp_of(first + Tb - 1, T, W) - wa) + 1;
     const float2 *ml = p.part_ml + (unit + wa) * G + hh;
@@ -882,7 +889,9 @@ cudaError_t launch_decode(int head_dim, int group, bool fp8, const DecodeParams 
 // the row with the most of them (the loads one thread keeps in flight).
 static int combine_threads(int head_dim, const DecodeParams &p) {
     int64_t tb = 0;
-    for (int b = 0; b < p.B; ++b) tb = std::max<int64_t>(tb, p.rows.pref_tiles[b + 1] - p.rows.pref_tiles[b]);
+    for (int g = 0; g < (p.layer1 < p.n_layers_run ? 2 : 1); ++g)
+        for (int b = 0; b < p.B; ++b)
+            tb = std::max<int64_t>(tb, p.rows[g].pref_tiles[b + 1] - p.rows[g].pref_tiles[b]);
     const int64_t most = p.n_tiles > 0 ? tb * p.n_warps / p.n_tiles + 2 : 1;
     const int lanes = head_dim / 4;
     int threads = std::max(lanes, 32);

@@ -250,15 +250,18 @@ struct PageSource {
 
 // --------------------------------------------------------------- decode --
 // A launch covers Lrun layers x B batch rows x Hkv kv heads ("units").  Unit
-// (l, b, g) owns T_b = npages_b * tiles_per_page tiles, in page order; the
-// global tile list orders units (l, b, g) with g fastest.  Warp w of W takes
-// the contiguous range [w*T/W, (w+1)*T/W) and writes one partial per unit it
-// touches, at slot unit + w (unique because both ranges are contiguous).
-struct BatchRows {
-    int32_t seq[kMaxBatchPerLaunch];
+// (l, b, g) owns the T_b tiles its layer reads of row b (all of them, or a
+// window's), in page order; the global tile list orders units (l, b, g) with
+// g fastest.  Warp w of W takes the contiguous range [w*T/W, (w+1)*T/W) and
+// writes one partial per unit it touches, at slot unit + w (unique because
+// both ranges are contiguous).  The run layers are ordered in up to
+// kMaxWindowGroups groups that read the same tiles of a row: layers
+// [0, layer1) by rows[0], the others by rows[1].
+constexpr int kMaxWindowGroups = 2;
+struct GroupRows {
     int32_t tile0[kMaxBatchPerLaunch];  // first tile of the row's pages that is read (window start)
-    int32_t lo[kMaxBatchPerLaunch];     // rows of that first tile before the window start
     int32_t pref_tiles[kMaxBatchPerLaunch + 1];  // prefix sums of T_b
+    uint8_t lo[kMaxBatchPerLaunch];     // rows of that first tile before the window start
 };
 
 struct DecodeParams {
@@ -284,7 +287,10 @@ struct DecodeParams {
     float *state;              // split decode: fp32 [Lrun][Btot][Hq][D + 4] (o, m, l, pad); null otherwise
     int32_t state_merge;       // 1: merge into the state, 0: overwrite it
     DevStatus *status;
-    BatchRows rows;
+    int32_t layer1;            // first run layer of the second group (n_layers_run: one group)
+    int64_t tile1;             // tiles of the first group
+    int32_t seq[kMaxBatchPerLaunch];
+    GroupRows rows[kMaxWindowGroups];
 };
 
 // -------------------------------------------------------------- launchers --
@@ -410,8 +416,12 @@ struct CacheShape {
 };
 bool cache_shape(const kvg_cache *c, CacheShape *out);
 int32_t cache_seq_pages(const kvg_cache *c, int32_t seq);
-kvg_status cache_plan_decode(const kvg_cache *c, int32_t layer, const int32_t *seq_ids, int32_t B,
+kvg_status cache_plan_decode(const kvg_cache *c, int32_t layer, const int32_t *seq_ids, int32_t B, int G, int w_max,
                              std::vector<DecodeParams> *plan, int64_t *max_units);
+// Bytes of the allocation-free decode's static scratch, and of one partial's
+// slot (G heads: fp32 o, m and l).
+constexpr uint64_t kStaticScratchBytes = 16u << 20;
+inline uint64_t partial_slot_bytes(int G, int head_dim) { return (uint64_t)G * ((uint64_t)head_dim * 4 + 8); }
 void set_last_error(const char *msg);
 // Looks up the device address of the allocation-free decode's static scratch
 // on the current device (once per device) and so makes the module that

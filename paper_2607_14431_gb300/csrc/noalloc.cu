@@ -25,7 +25,7 @@ namespace {
 // Scratch for the split-K partials: float o[units][splits][G][D] followed by
 // float2 (m, l)[units][splits][G].  Every GPU that loads the library holds it
 // until the process exits.
-constexpr size_t kScratchBytes = 16u << 20;
+constexpr size_t kScratchBytes = kvg::kStaticScratchBytes;
 static __device__ __align__(256) unsigned char g_decode_scratch[kScratchBytes];
 
 // Device address of g_decode_scratch per device ordinal.  In host code the
@@ -80,14 +80,26 @@ extern "C" kvg_status kvg_decode_attention_noalloc(kvg_cache *c, int32_t layer, 
     if (cs.device < 0 || cs.device >= kMaxDevices) return reject(KVG_ERR_ARG, "device ordinal out of range");
     for (int32_t b = 0; b < B; ++b)
         if (seq_ids[b] < 0 || seq_ids[b] >= cs.max_seqs) return reject(KVG_ERR_ARG, "bad seq id");
+    int prev = -1;
+    cudaGetDevice(&prev);
+    if (prev != cs.device && cudaSetDevice(cs.device) != cudaSuccess)
+        return reject(KVG_ERR_CUDA, "cudaSetDevice failed");
+    struct Restore {
+        int prev, dev;
+        ~Restore() {
+            if (prev >= 0 && prev != dev) cudaSetDevice(prev);
+        }
+    } restore{prev, cs.device};
+    const int w_max = decode_max_warps(cs.head_dim, G, fp8, cs.n_sm);
+    if (w_max <= 0) return reject(KVG_ERR_CUDA, "decode kernel cannot be made resident");
     // the launches (as kvg_decode_attention makes them); host memory only
     std::vector<DecodeParams> plan;
     int64_t units = 0;
-    const kvg_status pst = cache_plan_decode(c, layer, seq_ids, B, &plan, &units);
+    const kvg_status pst = cache_plan_decode(c, layer, seq_ids, B, G, w_max, &plan, &units);
     if (pst != KVG_OK) return pst;
     // partials: (units + workers) slots of G * (4 * head_dim + 8) bytes; the
     // (m, l) part starts 256-byte aligned after o, so keep 256 bytes of slack
-    const uint64_t per_slot = (uint64_t)G * ((uint64_t)cs.head_dim * 4 + 8);
+    const uint64_t per_slot = partial_slot_bytes(G, cs.head_dim);
     const int64_t cap_slots = (int64_t)((kScratchBytes - 256) / per_slot);
     if (cap_slots - units < 1) {
         char m[320];
@@ -99,16 +111,6 @@ extern "C" kvg_status kvg_decode_attention_noalloc(kvg_cache *c, int32_t layer, 
         return reject(KVG_ERR_CAPACITY, m);
     }
 
-    int prev = -1;
-    cudaGetDevice(&prev);
-    if (prev != cs.device && cudaSetDevice(cs.device) != cudaSuccess)
-        return reject(KVG_ERR_CUDA, "cudaSetDevice failed");
-    struct Restore {
-        int prev, dev;
-        ~Restore() {
-            if (prev >= 0 && prev != dev) cudaSetDevice(prev);
-        }
-    } restore{prev, cs.device};
     void *scratch = nullptr;
     {
         // the address was looked up when the cache was created on this
@@ -117,8 +119,6 @@ extern "C" kvg_status kvg_decode_attention_noalloc(kvg_cache *c, int32_t layer, 
         scratch = g_scratch_dev[cs.device];
     }
     if (!scratch) return reject(KVG_ERR_CUDA, "static decode scratch was not set up on the cache's device");
-    const int w_max = decode_max_warps(cs.head_dim, G, fp8, cs.n_sm);
-    if (w_max <= 0) return reject(KVG_ERR_CUDA, "decode kernel cannot be made resident");
     const int64_t w_cap = cap_slots - units < w_max ? cap_slots - units : w_max;
     const size_t slots = (size_t)units + (size_t)w_cap;
     float *part_o = static_cast<float *>(scratch);

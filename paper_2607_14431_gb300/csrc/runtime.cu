@@ -1997,79 +1997,109 @@ static void window_start(const kvg_cache *c, int32_t seq, int64_t window, int32_
     *row = 0;
 }
 
+// Layers of one decode call that read the same rows: (cache layer, q layer).
+struct WindowGroup {
+    int32_t window;
+    std::vector<std::pair<int32_t, int32_t>> layers;
+};
+
 // The launches of one decode call: the layers run are grouped by their
-// window (one group when no layer is windowed), each group split into
-// launches of at most kMaxLayersPerLaunch layers and kMaxBatchPerLaunch rows.
+// window (one group when no layer is windowed), each group split into parts
+// of at most kMaxLayersPerLaunch layers, and each launch takes one part, or
+// two where their partials fit the allocation-free decode's static scratch
+// with every worker (so that both entry points split the work the same way,
+// and that one refuses nothing that separate launches would fit), over at
+// most kMaxBatchPerLaunch rows.  Two windows in one launch share its ramp, its
+// drained end and the combine: a step of 16 fp8 sequences over 1,000 to 12,001
+// rows, every second of 4 layers windowed to 1,024, 195 us in two launches and
+// 178 in one.
 // Fills every field but the per-call ones (q, out, scale, heads, scratch,
 // workers); *max_units gets the largest layers x rows x kv heads of a launch.
 // page_begin / page_end: only the sequence's pages [page_begin, page_end)
 // are read (a split decode over a slot range); the defaults read them all.
-static kvg_status plan_decode(const kvg_cache *c, int32_t layer, const int32_t *seq_ids, int32_t B,
+static kvg_status plan_decode(const kvg_cache *c, int32_t layer, const int32_t *seq_ids, int32_t B, int G, int w_max,
                               std::vector<DecodeParams> *plan, int64_t *max_units, int32_t page_begin = 0,
                               int32_t page_end = INT32_MAX) {
     const kvg_dims &d = c->dims;
     const int TOK = decode_tile_tokens(d.head_dim, d.kv_dtype == KVG_KV_E4M3);
     const int tpp = (d.page_size + TOK - 1) / TOK;
-    // (window, [(cache layer, q layer)]) in order of first appearance
-    std::vector<std::pair<int32_t, std::vector<std::pair<int32_t, int32_t>>>> groups;
+    std::vector<WindowGroup> parts;  // in order of first appearance
     for (int32_t l = layer < 0 ? 0 : layer; l < (layer < 0 ? d.n_layers : layer + 1); ++l) {
         const int32_t w = c->layer_window[l];
-        auto it = std::find_if(groups.begin(), groups.end(), [w](const auto &g) { return g.first == w; });
-        if (it == groups.end()) {
-            groups.push_back({w, {}});
-            it = groups.end() - 1;
+        auto it = std::find_if(parts.begin(), parts.end(), [w](const WindowGroup &g) {
+            return g.window == w && g.layers.size() < kMaxLayersPerLaunch;
+        });
+        if (it == parts.end()) {
+            parts.push_back({w, {}});
+            it = parts.end() - 1;
         }
-        it->second.push_back({l, layer < 0 ? l : 0});
+        it->layers.push_back({l, layer < 0 ? l : 0});
     }
     plan->clear();
     *max_units = 0;
-    for (const auto &grp : groups) {
-        const int64_t W = grp.first;
-        for (size_t l0 = 0; l0 < grp.second.size(); l0 += kMaxLayersPerLaunch) {
-            const int32_t nl = (int32_t)std::min<size_t>(kMaxLayersPerLaunch, grp.second.size() - l0);
-            for (int64_t b0 = 0; b0 < B; b0 += kMaxBatchPerLaunch) {
-                const int32_t nb = (int32_t)std::min<int64_t>(kMaxBatchPerLaunch, B - b0);
-                plan->emplace_back();
-                DecodeParams &p = plan->back();
-                memset(&p, 0, sizeof p);
+    const int32_t nb_max = std::min<int32_t>(B, kMaxBatchPerLaunch);
+    const int64_t slots = (int64_t)((kStaticScratchBytes - 256) / partial_slot_bytes(G, d.head_dim));
+    for (size_t i0 = 0; i0 < parts.size();) {
+        size_t n_parts = 1, nl = parts[i0].layers.size();
+        if (i0 + 1 < parts.size()) {
+            const size_t both = nl + parts[i0 + 1].layers.size();
+            if (both <= kMaxLayersPerLaunch && (int64_t)both * nb_max * d.n_kv_heads + w_max <= slots) {
+                n_parts = 2;
+                nl = both;
+            }
+        }
+        for (int32_t b0 = 0; b0 < B; b0 += kMaxBatchPerLaunch) {
+            const int32_t nb = std::min<int32_t>(kMaxBatchPerLaunch, B - b0);
+            plan->emplace_back();
+            DecodeParams &p = plan->back();
+            memset(&p, 0, sizeof p);
+            for (int32_t i = 0; i < nb; ++i) p.seq[i] = seq_ids[b0 + i];
+            p.n_layers_run = p.layer1 = (int32_t)nl;
+            int32_t lr = 0;
+            for (size_t k = 0; k < n_parts; ++k) {
+                const WindowGroup &part = parts[i0 + k];
+                GroupRows &rows = p.rows[k];
                 int32_t acc = 0;
                 for (int32_t i = 0; i < nb; ++i) {
                     const int32_t sq = seq_ids[b0 + i];
                     const int32_t np = (int32_t)c->seq_pages[sq].size();
                     int32_t pg = 0, row = 0;
-                    if (W > 0) window_start(c, sq, W, &pg, &row);
+                    if (part.window > 0) window_start(c, sq, part.window, &pg, &row);
                     int32_t t0 = pg * tpp + row / TOK, lo = row % TOK;
                     if (page_begin > 0 && (int64_t)page_begin * tpp > t0) {
                         t0 = page_begin * tpp;
                         lo = 0;
                     }
                     const int32_t t1 = std::min(np, page_end) * tpp;
-                    p.rows.seq[i] = sq;
-                    p.rows.tile0[i] = t0;
-                    p.rows.lo[i] = lo;
-                    p.rows.pref_tiles[i] = acc;
+                    rows.tile0[i] = t0;
+                    rows.lo[i] = (uint8_t)lo;
+                    rows.pref_tiles[i] = acc;
                     acc += std::max(0, t1 - t0);
                 }
-                p.rows.pref_tiles[nb] = acc;
-                for (int32_t i = 0; i < nl; ++i) {
-                    p.layers[i] = (int16_t)grp.second[l0 + i].first;
-                    p.qlayers[i] = (int16_t)grp.second[l0 + i].second;
+                rows.pref_tiles[nb] = acc;
+                for (const auto &l : part.layers) {
+                    p.layers[lr] = (int16_t)l.first;
+                    p.qlayers[lr++] = (int16_t)l.second;
                 }
-                p.n_layers_run = nl;
-                p.n_tiles = (int64_t)nl * d.n_kv_heads * acc;
-                p.B = nb;
-                p.b0 = (int32_t)b0;
-                p.pool = c->pool;
-                p.pool_pages = c->n_pages;
-                p.n_kv_heads = d.n_kv_heads;
-                p.page_size = d.page_size;
-                p.page_table = c->page_table;
-                p.page_fill = c->page_fill;
-                p.max_pages = c->max_pages;
-                p.status = c->status;
-                *max_units = std::max<int64_t>(*max_units, (int64_t)nl * nb * d.n_kv_heads);
+                p.n_tiles += (int64_t)part.layers.size() * d.n_kv_heads * acc;
+                if (k == 0) {
+                    p.layer1 = lr;
+                    p.tile1 = p.n_tiles;
+                }
             }
+            p.B = nb;
+            p.b0 = b0;
+            p.pool = c->pool;
+            p.pool_pages = c->n_pages;
+            p.n_kv_heads = d.n_kv_heads;
+            p.page_size = d.page_size;
+            p.page_table = c->page_table;
+            p.page_fill = c->page_fill;
+            p.max_pages = c->max_pages;
+            p.status = c->status;
+            *max_units = std::max<int64_t>(*max_units, (int64_t)nl * nb * d.n_kv_heads);
         }
+        i0 += n_parts;
     }
     return KVG_OK;
 }
@@ -2111,7 +2141,7 @@ static kvg_status decode_impl(const char *what, kvg_cache *c, int32_t layer, con
     if (w_max <= 0) return fail(KVG_ERR_CUDA, "decode kernel cannot be made resident");
     std::vector<DecodeParams> plan;
     int64_t max_units = 0;
-    kvg_status r = plan_decode(c, layer, seq_ids, B, &plan, &max_units, page_begin, page_end);
+    kvg_status r = plan_decode(c, layer, seq_ids, B, G, w_max, &plan, &max_units, page_begin, page_end);
     if (r != KVG_OK) return r;
     const size_t slots = (size_t)max_units + (size_t)w_max;
     if (!c->part_ev) KVG_CUDA(cudaEventCreateWithFlags(&c->part_ev, cudaEventDisableTiming));
@@ -2285,9 +2315,9 @@ bool cache_shape(const kvg_cache *c, CacheShape *out) {
     return true;
 }
 int32_t cache_seq_pages(const kvg_cache *c, int32_t seq) { return (int32_t)c->seq_pages[seq].size(); }
-kvg_status cache_plan_decode(const kvg_cache *c, int32_t layer, const int32_t *seq_ids, int32_t B,
+kvg_status cache_plan_decode(const kvg_cache *c, int32_t layer, const int32_t *seq_ids, int32_t B, int G, int w_max,
                              std::vector<DecodeParams> *plan, int64_t *max_units) {
-    return plan_decode(c, layer, seq_ids, B, plan, max_units);
+    return plan_decode(c, layer, seq_ids, B, G, w_max, plan, max_units);
 }
 void set_last_error(const char *msg) { g_last_error = msg; }
 }  // namespace kvg
