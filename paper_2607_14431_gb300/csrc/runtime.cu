@@ -752,6 +752,11 @@ extern "C" kvg_status kvg_store_load(kvg_store *s, const char *path, uint32_t fl
 // ------------------------------------------------------------------- cache --
 
 constexpr int kHostVerifyChunks = 16;  // page-range chunks of a verified host-store graft
+// Streams its chunks are hashed on in turn.  A chunk's hash is bound by the
+// latency of one leaf's chain, which work beside it (an append, decodes) makes
+// longer than the next chunk's copy: on one stream the hashes fell behind and
+// ended 0.3 ms after the block had landed.
+constexpr int kHostHashStreams = 2;
 constexpr int32_t kMaxGraftsPerBatch = 4096;
 
 struct kvg_cache {
@@ -775,10 +780,10 @@ struct kvg_cache {
     cudaStream_t part_stream = nullptr;
     bool part_used = false;
     CUtensorMap pool_map;  // decode kernel's 2-D view of the pool
-    // library stream and events for hashing a host-store graft's pages while
+    // library streams and events for hashing a host-store graft's pages while
     // the next pages still cross the host link (made on first use)
-    cudaStream_t aux = nullptr;
-    cudaEvent_t aux_ev[kHostVerifyChunks + 1] = {};
+    cudaStream_t aux[kHostHashStreams] = {};
+    cudaEvent_t aux_ev[kHostVerifyChunks + kHostHashStreams] = {};
     // kvg_graft_batch's job table: staged in pinned host memory, copied to
     // batch_dev on the call's stream; batch_ev marks when the copy has read it
     Scratch batch_dev;
@@ -997,7 +1002,8 @@ extern "C" void kvg_cache_destroy(kvg_cache *c) {
     cudaDeviceSynchronize();
     for (cudaEvent_t &e : c->aux_ev)
         if (e) cudaEventDestroy(e);
-    if (c->aux) cudaStreamDestroy(c->aux);
+    for (cudaStream_t a : c->aux)
+        if (a) cudaStreamDestroy(a);
     if (c->batch_ev) cudaEventDestroy(c->batch_ev);
     if (c->part_ev) cudaEventDestroy(c->part_ev);
     if (c->batch_host) cudaFreeHost(c->batch_host);
@@ -1657,7 +1663,7 @@ static kvg_status graft_impl(kvg_store *s, uint64_t block_id, kvg_cache *c, int3
     // the copy and the leaf hashes are one kernel, and only the page digests
     // follow.  From a pinned-host store the copy instead moves page-range
     // chunks with the copy kernel (whose wide reads keep the host link at its
-    // limit) and a library stream hashes each chunk's restored pages in HBM
+    // limit) and library streams hash each chunk's restored pages in HBM
     // while the next chunk crosses the link; the last, short chunk goes
     // through the one-pass kernel.
     const bool host_src = s->residency == KVG_RESIDENCY_PINNED_HOST;
@@ -1674,10 +1680,14 @@ static kvg_status graft_impl(kvg_store *s, uint64_t block_id, kvg_cache *c, int3
     // follow the transfer, so each chunk's hash must fit in the next one's copy
     std::vector<int64_t> tails;
     if (piped) {
-        if (!c->aux) {
-            KVG_CUDA(cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking));
-            for (cudaEvent_t &e : c->aux_ev) KVG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        }
+        // (the highest priority: a chunk's few CTAs go ahead of the queued ones of
+        // the work beside it)
+        int least = 0, greatest = 0;
+        KVG_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+        for (cudaStream_t &a : c->aux)
+            if (!a) KVG_CUDA(cudaStreamCreateWithPriority(&a, cudaStreamNonBlocking, greatest));
+        for (cudaEvent_t &e : c->aux_ev)
+            if (!e) KVG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         if (npb > kHostVerifyChunks) {
             const int64_t t1 = std::min<int64_t>(std::max<int64_t>(1, npb / 128), kMaxPagesPerLaunch / 3);
             tails = {3 * t1, t1};
@@ -1736,18 +1746,23 @@ static kvg_status graft_impl(kvg_store *s, uint64_t block_id, kvg_cache *c, int3
             // plane; an event is re-recorded after its wait is enqueued)
             cudaEvent_t ev = c->aux_ev[chunk % kHostVerifyChunks];
             KVG_CUDA(cudaEventRecord(ev, st));
-            KVG_CUDA(cudaStreamWaitEvent(c->aux, ev, 0));
+            cudaStream_t aux = c->aux[chunk % kHostHashStreams];
+            KVG_CUDA(cudaStreamWaitEvent(aux, ev, 0));
             PageSource src{c->pool, c->page_bytes, c->page_table + (int64_t)seq * c->max_pages + jdst + base, p.npb,
                            (int64_t)c->n_pages};
             src.out_plane_stride = npb;
             src.out_j0 = (int32_t)base;
+            // in the one-warp form, which needs no shared memory: the append's and
+            // the decode's CTAs leave room for little of it on an SM
             KVG_CUDA(launch_sha256_leaves(src, (int64_t)c->dims.n_layers * 2 * p.npb,
-                                          static_cast<uint32_t *>(c->leaf.ptr), c->n_sm, c->aux));
+                                          static_cast<uint32_t *>(c->leaf.ptr), c->n_sm, aux, false));
         }
     }
     if (piped) {
-        KVG_CUDA(cudaEventRecord(c->aux_ev[kHostVerifyChunks], c->aux));
-        KVG_CUDA(cudaStreamWaitEvent(st, c->aux_ev[kHostVerifyChunks], 0));
+        for (int a = 0; a < kHostHashStreams; ++a) {
+            KVG_CUDA(cudaEventRecord(c->aux_ev[kHostVerifyChunks + a], c->aux[a]));
+            KVG_CUDA(cudaStreamWaitEvent(st, c->aux_ev[kHostVerifyChunks + a], 0));
+        }
     }
     if (verify0) {
         KVG_CUDA(launch_sha256_pages(static_cast<const uint32_t *>(c->leaf.ptr), (int64_t)c->dims.n_layers * 2 * npb, m,
