@@ -249,6 +249,8 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
     }
     __syncwarp();
 
+    after_previous();
+
     const int64_t plane_rows = p.pool_pages * (int64_t)p.n_kv_heads * P;  // rows per (layer, K/V)
 
     // Lane 0's cursor over the tiles it copies: tiles are issued in order, so
@@ -416,6 +418,7 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
     for (int64_t t = t0; t < t1; ++t) {
         const int64_t i = t - t0;
         const int stg = (int)(i % STAGES);
+        if (t == t1 - 1) let_next_start();
         const uint32_t par = (uint32_t)((i / STAGES) & 1);
         if (t >= unit_end) {
             const TilePos tp = locate(p, t);
@@ -635,7 +638,10 @@ __device__ __forceinline__ Merged<D> merge_partials(const DecodeParams &p, int h
     const int grp = lr >= p.layer1;
     const int32_t *pref = p.rows[grp].pref_tiles;
     const int64_t Tb = pref[b + 1] - pref[b];
-    if (Tb <= 0) return res;  // the whole block
+    if (Tb <= 0) {  // the whole block
+        after_previous();
+        return res;
+    }
     const int64_t T = p.n_tiles, W = p.n_warps;
     const int64_t unit = ((int64_t)lr * p.B + b) * p.n_kv_heads + g;
     const int64_t first = (grp ? p.tile1 : 0) + (int64_t)g * Tb +
@@ -645,6 +651,7 @@ __device__ __forceinline__ Merged<D> merge_partials(const DecodeParams &p, int h
     const float2 *ml = p.part_ml + (unit + wa) * G + hh;
     const float4 *po = reinterpret_cast<const float4 *>(p.part_o + ((unit + wa) * G + hh) * D) + d4;
     const int64_t step = (int64_t)G * LANES;  // float4 between consecutive partials
+    after_previous();
     float M = -INFINITY;
     for (int i = threadIdx.x & 31; i < n; i += 32) M = fmaxf(M, ml[(int64_t)i * G].x);
 #pragma unroll
@@ -755,6 +762,7 @@ __global__ void __launch_bounds__(kCombineMaxThreads) combine_state_kernel(const
 
 __global__ void state_finish_kernel(const float *__restrict__ state, int64_t n_rows, int D,
                                     __nv_bfloat16 *__restrict__ out) {
+    after_previous();
     const int64_t n = n_rows * D;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = i / D;
@@ -787,9 +795,7 @@ struct DecodeLaunch {
     static cudaError_t run(const DecodeParams &p, const CUtensorMap &map, cudaStream_t s) {
         if (max_blocks_per_sm() <= 0) return cudaErrorInvalidConfiguration;
         if (p.n_warps <= 0 || p.n_tiles <= 0) return cudaSuccess;
-        decode_kernel<D, G, FP8><<<p.n_warps, 32, Cfg<D, FP8>::SMEM, s>>>(p, map);
-        count_launches(1);
-        return cudaGetLastError();
+        return launch_after(decode_kernel<D, G, FP8>, p.n_warps, 32, Cfg<D, FP8>::SMEM, s, p, map);
     }
 };
 
@@ -904,13 +910,11 @@ cudaError_t launch_combine(int head_dim, int group, const DecodeParams &p, cudaS
     const dim3 grid(p.n_q_heads, p.B, p.n_layers_run);
     const int n = combine_threads(head_dim, p);
     switch (head_dim) {
-        case 64: p.state ? combine_state_kernel<64><<<grid, n, 0, s>>>(p) : combine_kernel<64><<<grid, n, 0, s>>>(p); break;
-        case 128: p.state ? combine_state_kernel<128><<<grid, n, 0, s>>>(p) : combine_kernel<128><<<grid, n, 0, s>>>(p); break;
-        case 256: p.state ? combine_state_kernel<256><<<grid, n, 0, s>>>(p) : combine_kernel<256><<<grid, n, 0, s>>>(p); break;
-        default: return cudaErrorInvalidValue;
+        case 64: return launch_after(p.state ? combine_state_kernel<64> : combine_kernel<64>, grid, n, 0, s, p);
+        case 128: return launch_after(p.state ? combine_state_kernel<128> : combine_kernel<128>, grid, n, 0, s, p);
+        case 256: return launch_after(p.state ? combine_state_kernel<256> : combine_kernel<256>, grid, n, 0, s, p);
     }
-    count_launches(1);
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_state_finish(const float *state, int64_t n_rows, int head_dim, __nv_bfloat16 *out,
@@ -919,9 +923,7 @@ cudaError_t launch_state_finish(const float *state, int64_t n_rows, int head_dim
     if (n == 0) return cudaSuccess;
     int64_t grid = (n + 255) / 256;
     if (grid > 65535) grid = 65535;
-    state_finish_kernel<<<(int)grid, 256, 0, s>>>(state, n_rows, head_dim, out);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(state_finish_kernel, (int)grid, 256, 0, s, state, n_rows, head_dim, out);
 }
 
 }  // namespace kvg

@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <utility>
 #include <vector>
 
 #include "kvg.h"
@@ -431,6 +432,35 @@ cudaError_t noalloc_prepare_device(int device);
 
 // ------------------------------------------------------------ PTX helpers --
 #ifdef __CUDACC__
+// Programmatic dependent launch: a kernel launched with launch_after() may be
+// scheduled while the kernel before it on the stream is still finishing, so
+// that its launch latency (about a microsecond between two short kernels) is
+// hidden; it calls after_previous() before it touches global memory, which
+// waits until that kernel has completed and its writes are visible.  A kernel
+// calls let_next_start() once its own end is near (never long before: what
+// waits holds an SM's resources); the launch of the next needs it from every
+// CTA, or the CTA's exit.
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_after(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                                Args &&...args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    count_launches(1);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }

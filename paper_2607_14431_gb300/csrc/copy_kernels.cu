@@ -180,6 +180,7 @@ __device__ __forceinline__ void rotate_chunk(uint8_t *__restrict__ dst, const ui
 
 template <int ROT>
 __global__ void __launch_bounds__(kCopyThreads) graft_kernel(const GraftParams p) {
+    after_previous();
     const int64_t P = p.page_size;
     graft_metadata(p);
     const uint64_t page_bytes = p.page_bytes;
@@ -225,6 +226,8 @@ __device__ __forceinline__ void append_metadata(const AppendParams &p) {
 }
 
 __global__ void __launch_bounds__(kAppendThreads) append_kernel(const AppendParams p) {
+    after_previous();
+    let_next_start();  // a short kernel
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
     const int64_t P = p.page_size;
@@ -313,6 +316,7 @@ __global__ void __launch_bounds__(32) append_tma_kernel(const AppendParams p,
                                                         const __grid_constant__ CUtensorMap vmap,
                                                         DevStatus *status, int32_t pbox, int32_t n_stages,
                                                         uint64_t limit_ns) {
+    after_previous();
     extern __shared__ __align__(128) uint8_t stage_mem[];
     __shared__ __align__(8) uint64_t bars[kTmaStagesMax];
     append_metadata(p);
@@ -391,6 +395,7 @@ __device__ __forceinline__ uint2 e4m3x8(const uint4 x, float inv_scale) {
 // One warp per (layer, K/V, token) row, like append_kernel; 8 values per lane
 // per step (16 bytes in, 8 bytes out).
 __global__ void __launch_bounds__(kAppendThreads) append_e4m3_kernel(const AppendParams p) {
+    after_previous();
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
     const int64_t P = p.page_size;
@@ -431,6 +436,8 @@ __global__ void __launch_bounds__(kAppendThreads) append_e4m3_kernel(const Appen
 }
 
 __global__ void __launch_bounds__(kAppendThreads) append_batch_e4m3_kernel(const AppendBatchParams p) {
+    after_previous();
+    let_next_start();  // a short kernel
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
     const int64_t P = p.page_size;
@@ -474,6 +481,8 @@ __global__ void __launch_bounds__(kAppendThreads) append_batch_e4m3_kernel(const
 }
 
 __global__ void __launch_bounds__(kAppendThreads) append_batch_kernel(const AppendBatchParams p) {
+    after_previous();
+    let_next_start();  // a short kernel
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
     const int64_t P = p.page_size;
@@ -513,6 +522,7 @@ __global__ void __launch_bounds__(kAppendThreads) append_batch_kernel(const Appe
 // One 16-byte vector at a time with two 64-bit divisions each had taken 100
 // us for the 201 MB of 48 layers x 499 tokens of the 12B shape, against 77.
 __global__ void __launch_bounds__(kCopyThreads) gather_kernel(const GatherParams p) {
+    after_previous();
     const int64_t P = p.page_size;
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
@@ -557,6 +567,8 @@ __global__ void __launch_bounds__(kCopyThreads) gather_kernel(const GatherParams
 }
 
 __global__ void __launch_bounds__(256) alias_kernel(const AliasParams p) {
+    after_previous();
+    let_next_start();  // a short kernel
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
     const int64_t P = p.page_size;
@@ -600,6 +612,8 @@ __global__ void write_ints_kernel(const IntsParams p) {
 
 __global__ void reset_seq_kernel(int32_t *table_row, int32_t *fill_row, int32_t max_pages,
                                  int32_t *pos_row, int32_t max_slots) {
+    after_previous();
+    let_next_start();  // a short kernel
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
     for (int64_t j = gtid; j < max_pages; j += gsz) {
@@ -670,6 +684,7 @@ __device__ __forceinline__ void rotate_stage(uint8_t *stage, int bytes, int64_t 
 template <int ROT>
 __global__ void __launch_bounds__(kTmaGraftThreads) graft_tma_kernel(const GraftParams p, DevStatus *status,
                                                                      int32_t n_stages, uint64_t limit_ns) {
+    after_previous();
     extern __shared__ __align__(128) uint8_t stage_mem[];
     __shared__ __align__(8) uint64_t bars[kTmaStagesMax];
     __shared__ float cs[2 * kMaxHalfDim];
@@ -767,6 +782,7 @@ int grid_for(int64_t work_items, int per_block, int n_sm, int waves) {
 // as the single-graft kernels do; values and own-position grafts copy).
 template <int ROT>
 __global__ void __launch_bounds__(kCopyThreads) graft_batch_kernel(const GraftBatchParams p) {
+    after_previous();
     const uint64_t page_bytes = p.page_bytes;
     const int64_t cpp = (int64_t)(page_bytes / (uint64_t)p.chunk_bytes);
     const int64_t per_job = (int64_t)p.n_layers * 2 * cpp;
@@ -799,13 +815,8 @@ cudaError_t launch_graft_batch(const GraftBatchParams &p, int n_sm, cudaStream_t
     int grid = grid_for(units, 1, n_sm, 4);
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
     if (rotate == 0)
-        graft_batch_kernel<0><<<grid, kCopyThreads, 0, s>>>(p);
-    else if (rotate == 1)
-        graft_batch_kernel<1><<<grid, kCopyThreads, 0, s>>>(p);
-    else
-        graft_batch_kernel<2><<<grid, kCopyThreads, 0, s>>>(p);
-    count_launches(1);
-    return cudaGetLastError();
+        return launch_after(graft_batch_kernel<0>, grid, kCopyThreads, 0, s, p);
+    return launch_after(rotate == 1 ? graft_batch_kernel<1> : graft_batch_kernel<2>, grid, kCopyThreads, 0, s, p);
 }
 
 // Shared-memory stage budget of graft_tma_kernel (KVG_GRAFT_TMA_KB, 0 turns
@@ -845,14 +856,8 @@ static cudaError_t launch_graft_tma(const GraftParams &p, DevStatus *status, int
     }
     const int grid = grid_for(units, 1, n_sm, 1);
     const uint64_t limit_ns = 2000000000ull;
-    if (r == 0)
-        graft_tma_kernel<0><<<grid, kTmaGraftThreads, smem, s>>>(p, status, n_stages, limit_ns);
-    else if (r == 1)
-        graft_tma_kernel<1><<<grid, kTmaGraftThreads, smem, s>>>(p, status, n_stages, limit_ns);
-    else
-        graft_tma_kernel<2><<<grid, kTmaGraftThreads, smem, s>>>(p, status, n_stages, limit_ns);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(r == 0 ? graft_tma_kernel<0> : r == 1 ? graft_tma_kernel<1> : graft_tma_kernel<2>, grid,
+                        kTmaGraftThreads, smem, s, p, status, n_stages, limit_ns);
 }
 
 cudaError_t launch_graft_copy(const GraftParams &p, int n_sm, cudaStream_t s, int max_ctas, DevStatus *status) {
@@ -865,22 +870,14 @@ cudaError_t launch_graft_copy(const GraftParams &p, int n_sm, cudaStream_t s, in
     const int64_t units = (int64_t)p.n_layers * 2 * p.npb * (int64_t)(p.page_bytes / p.chunk_bytes);
     int grid = grid_for(units, 1, n_sm, 4);
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
-    if (p.rotate == 0)
-        graft_kernel<0><<<grid, kCopyThreads, 0, s>>>(p);
-    else if (p.rotate == 1)
-        graft_kernel<1><<<grid, kCopyThreads, 0, s>>>(p);
-    else
-        graft_kernel<2><<<grid, kCopyThreads, 0, s>>>(p);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(p.rotate == 0 ? graft_kernel<0> : p.rotate == 1 ? graft_kernel<1> : graft_kernel<2>, grid,
+                        kCopyThreads, 0, s, p);
 }
 
 cudaError_t launch_append(const AppendParams &p, int n_sm, cudaStream_t s) {
     const int64_t rows = 2ll * p.n_layers * p.n;  // one warp each
     static const int ctas_per_sm = env_knob("KVG_APPEND_CTAS_PER_SM", 2);
-    append_kernel<<<grid_for(rows, kAppendThreads / 32, n_sm, ctas_per_sm), kAppendThreads, 0, s>>>(p);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(append_kernel, grid_for(rows, kAppendThreads / 32, n_sm, ctas_per_sm), kAppendThreads, 0, s, p);
 }
 
 // Rows per tensor copy: a page's rows, at most 256 (the box limit) and at
@@ -927,45 +924,35 @@ cudaError_t launch_append_tma(const AppendParams &p, DevStatus *status, int n_sm
     const int chunks = (p.page_size + pbox - 1) / pbox;
     const int64_t jobs = 2ll * p.n_layers * p.pids.n * p.n_kv_heads * chunks;
     const int grid = grid_for(jobs, 1, n_sm, 1);
-    append_tma_kernel<<<grid, 32, (size_t)n_stages * stage_bytes, s>>>(p, maps[0], maps[1], status, pbox, n_stages,
-                                                                      2000000000ull);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(append_tma_kernel, grid, 32, (size_t)n_stages * stage_bytes, s, p, maps[0], maps[1], status,
+                        pbox, n_stages, 2000000000ull);
 }
 
 cudaError_t launch_append_e4m3(const AppendParams &p, int n_sm, cudaStream_t s) {
     const int64_t rows = 2ll * p.n_layers * p.n;  // one warp each
     static const int ctas_per_sm = env_knob("KVG_APPEND_CTAS_PER_SM", 2);
-    append_e4m3_kernel<<<grid_for(rows, kAppendThreads / 32, n_sm, ctas_per_sm), kAppendThreads, 0, s>>>(p);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(append_e4m3_kernel, grid_for(rows, kAppendThreads / 32, n_sm, ctas_per_sm), kAppendThreads, 0,
+                        s, p);
 }
 
 cudaError_t launch_append_batch_e4m3(const AppendBatchParams &p, int n_sm, cudaStream_t s) {
     const int64_t rows = 2ll * p.n_layers * p.B;
-    append_batch_e4m3_kernel<<<grid_for(rows, kAppendThreads / 32, n_sm, 8), kAppendThreads, 0, s>>>(p);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(append_batch_e4m3_kernel, grid_for(rows, kAppendThreads / 32, n_sm, 8), kAppendThreads, 0, s, p);
 }
 
 cudaError_t launch_append_batch(const AppendBatchParams &p, int n_sm, cudaStream_t s) {
     const int64_t rows = 2ll * p.n_layers * p.B;
-    append_batch_kernel<<<grid_for(rows, kAppendThreads / 32, n_sm, 8), kAppendThreads, 0, s>>>(p);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(append_batch_kernel, grid_for(rows, kAppendThreads / 32, n_sm, 8), kAppendThreads, 0, s, p);
 }
 
 cudaError_t launch_gather(const GatherParams &p, int n_sm, cudaStream_t s) {
     const int64_t units = 2ll * p.n_layers * p.npb * (int64_t)(p.page_bytes / p.chunk_bytes);
-    gather_kernel<<<grid_for(units, 1, n_sm, 4), kCopyThreads, 0, s>>>(p);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(gather_kernel, grid_for(units, 1, n_sm, 4), kCopyThreads, 0, s, p);
 }
 
 cudaError_t launch_alias(const AliasParams &p, int n_sm, cudaStream_t s) {
-    alias_kernel<<<grid_for(p.n_tokens > p.pids.n ? p.n_tokens : p.pids.n, 256, n_sm, 1), 256, 0, s>>>(p);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(alias_kernel, grid_for(p.n_tokens > p.pids.n ? p.n_tokens : p.pids.n, 256, n_sm, 1), 256, 0, s,
+                        p);
 }
 
 cudaError_t launch_touch(const uint8_t *base, uint64_t bytes, uint32_t stride, int n_sm, cudaStream_t s) {
@@ -991,10 +978,8 @@ cudaError_t launch_write_ints(const IntsParams &p, cudaStream_t s) {
 cudaError_t launch_reset_seq(int32_t *table_row, int32_t *fill_row, int32_t max_pages,
                              int32_t *pos_row, int32_t max_slots, cudaStream_t s) {
     const int64_t items = max_pages > max_slots ? max_pages : max_slots;
-    reset_seq_kernel<<<grid_for(items, 256, 152, 1), 256, 0, s>>>(table_row, fill_row, max_pages,
-                                                                   pos_row, max_slots);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(reset_seq_kernel, grid_for(items, 256, 152, 1), 256, 0, s, table_row, fill_row, max_pages,
+                        pos_row, max_slots);
 }
 
 }  // namespace kvg

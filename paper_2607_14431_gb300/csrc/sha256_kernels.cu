@@ -430,6 +430,7 @@ __device__ __forceinline__ bool split_begin(SplitShared &sm) {
         sm.consumer = (int)((slot >> 2) & 1);
     }
     __syncthreads();
+    after_previous();
     return (int)(threadIdx.x >> 5) != sm.consumer;
 }
 
@@ -446,8 +447,10 @@ __device__ __forceinline__ void split_consume(uint32_t st[4], const SplitShared 
         const int buf = k & 1;
         bar_sync_pair(1 + buf);
 #pragma unroll 1
-        for (int h = 0; h < 2 && 2 * k + h < n_blocks; ++h)
+        for (int h = 0; h < 2 && 2 * k + h < n_blocks; ++h) {
+            if (2 * k + h == n_blocks - 1) let_next_start();
             split_rounds(st, ro.a ? &sm.zero[0][c] : &sm.kw[buf][h][0][c], ro, one);
+        }
         if (k + 2 < n_pairs) bar_arrive_pair(3 + buf);
     }
 }
@@ -496,6 +499,7 @@ __device__ __forceinline__ void wide_consume(uint32_t st[8], const SplitShared &
     for (int k = 0; k < n_blocks; ++k) {
         const int buf = k & 1;
         bar_sync_pair(1 + buf);
+        if (k == n_blocks - 1) let_next_start();
         wide_rounds(st, &sm.kw[buf][lane / kSplitChains][0][lane & (kSplitChains - 1)], one);
         if (k + 2 < n_blocks) bar_arrive_pair(3 + buf);
     }
@@ -673,6 +677,7 @@ template <bool LAT>
 __global__ void __launch_bounds__(128) sha256_leaves_kernel(const PageSource src, int64_t n_pages,
                                                             int64_t leaves_per_page,
                                                             uint32_t *__restrict__ out, uint32_t one) {
+    after_previous();
     const int64_t n_leaves = n_pages * leaves_per_page;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n_leaves;
          idx += (int64_t)gridDim.x * blockDim.x) {
@@ -715,6 +720,7 @@ __global__ void __launch_bounds__(128) sha256_leaves_kernel(const PageSource src
 constexpr int kGraftVerifyRing = 3;
 __global__ void __launch_bounds__(128, 5) graft_verify_ring_kernel(const GraftParams p, int64_t leaves_per_page,
                                                                    uint32_t *__restrict__ out, uint32_t one) {
+    after_previous();
     constexpr int R = kGraftVerifyRing;
     extern __shared__ __align__(16) uint4 ring_mem[];
     graft_metadata(p);
@@ -744,6 +750,7 @@ __global__ void __launch_bounds__(128, 5) graft_verify_ring_kernel(const GraftPa
 // hashes it (leaf order of a page digest, Sec. 3.2's integrity check).
 __global__ void __launch_bounds__(128) graft_verify_kernel(const GraftParams p, int64_t leaves_per_page,
                                                            uint32_t *__restrict__ out, uint32_t one) {
+    after_previous();
     graft_metadata(p);
     const uint64_t page_bytes = p.page_bytes;
     const int64_t n_leaves = (int64_t)p.n_layers * 2 * p.npb * leaves_per_page;
@@ -800,6 +807,7 @@ __device__ __forceinline__ BatchLeaf batch_leaf(const GraftBatchParams &p, int64
 __global__ void __launch_bounds__(128, 5) graft_batch_verify_ring_kernel(const GraftBatchParams p,
                                                                          int64_t leaves_per_page,
                                                                          uint32_t *__restrict__ out, uint32_t one) {
+    after_previous();
     constexpr int R = kGraftVerifyRing;
     extern __shared__ __align__(16) uint4 ring_mem[];
     if (p.write_meta) batch_metadata(p);
@@ -821,6 +829,7 @@ __global__ void __launch_bounds__(128, 5) graft_batch_verify_ring_kernel(const G
 template <bool COPY>
 __global__ void __launch_bounds__(128) graft_batch_verify_kernel(const GraftBatchParams p, int64_t leaves_per_page,
                                                                  uint32_t *__restrict__ out, uint32_t one) {
+    after_previous();
     if (p.write_meta) batch_metadata(p);
     const int64_t n_leaves = p.slice_jobs * p.n_layers * 2 * leaves_per_page;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n_leaves;
@@ -914,6 +923,7 @@ template <class Verdict>
 __global__ void __launch_bounds__(128) sha256_pages_kernel(const uint32_t *__restrict__ leaf_words,
                                                            int64_t n_pages, int64_t m, const Verdict verdict,
                                                            uint32_t one) {
+    after_previous();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n_pages) return;
     const uint32_t *lw = leaf_words + p * m * 8;
@@ -1081,6 +1091,7 @@ __device__ __forceinline__ uint32_t msg_word(const uint8_t *seg0, uint64_t n0, c
 __global__ void __launch_bounds__(32) sha256_serial_kernel(const uint8_t *seg0, uint64_t n0, const uint8_t *seg1,
                                                            uint64_t n1, uint8_t *out, const uint8_t *expected,
                                                            DevStatus *status, uint32_t one) {
+    after_previous();
     __shared__ uint32_t buf[2][kSerialChunkWords];
     const int lane = threadIdx.x;
     if (blockIdx.x != 0) return;
@@ -1284,9 +1295,7 @@ cudaError_t launch_sha256_leaves(const PageSource &src, int64_t n_pages, uint32_
     if (split_ok && !split_off() && src.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
         const bool wide = split_wide(n, n_sm);
         auto *kernel = wide ? sha256_leaves_split_kernel<true> : sha256_leaves_split_kernel<false>;
-        kernel<<<split_grid(n, wide), 64, 0, s>>>(src, n_pages, m, leaf_words, 1u);
-        count_launches(1);
-        return cudaGetLastError();
+        return launch_after(kernel, split_grid(n, wide), 64, 0, s, src, n_pages, m, leaf_words, 1u);
     }
     int64_t grid = (n + 127) / 128;
     // One CTA per 128 leaves (no grid-stride cap by default): 4 CTAs of
@@ -1296,9 +1305,7 @@ cudaError_t launch_sha256_leaves(const PageSource &src, int64_t n_pages, uint32_
     if (ctas_per_sm > 0 && grid > (int64_t)n_sm * ctas_per_sm) grid = (int64_t)n_sm * ctas_per_sm;
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
     auto *kernel = lat_order(n, n_sm) ? sha256_leaves_kernel<true> : sha256_leaves_kernel<false>;
-    kernel<<<(int)grid, 128, 0, s>>>(src, n_pages, m, leaf_words, 1u);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(kernel, (int)grid, 128, 0, s, src, n_pages, m, leaf_words, 1u);
 }
 
 cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int n_sm, cudaStream_t s, bool ring_ok,
@@ -1309,9 +1316,7 @@ cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int 
     if (split_ok && !split_off() && p.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
         const bool wide = split_wide(n, n_sm);
         auto *kernel = wide ? graft_verify_split_kernel<true> : graft_verify_split_kernel<false>;
-        kernel<<<split_grid(n, wide), 64, 0, s>>>(p, m, leaf_words, 1u);
-        count_launches(1);
-        return cudaGetLastError();
+        return launch_after(kernel, split_grid(n, wide), 64, 0, s, p, m, leaf_words, 1u);
     }
     int64_t grid = (n + 127) / 128;
     // One CTA per 128 leaves (no grid-stride cap by default): four CTAs of
@@ -1325,12 +1330,9 @@ cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int 
     // form for every size.
     if (ring_ok && !regs_only() && n >= (int64_t)n_sm * 5 * 128 && grid > (int64_t)n_sm * 4) {
         const size_t smem = (size_t)128 * kGraftVerifyRing * 64;  // 24 KiB of ring slots per CTA
-        graft_verify_ring_kernel<<<(int)grid, 128, smem, s>>>(p, m, leaf_words, 1u);
-    } else {
-        graft_verify_kernel<<<(int)grid, 128, 0, s>>>(p, m, leaf_words, 1u);
+        return launch_after(graft_verify_ring_kernel, (int)grid, 128, smem, s, p, m, leaf_words, 1u);
     }
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_after(graft_verify_kernel, (int)grid, 128, 0, s, p, m, leaf_words, 1u);
 }
 
 cudaError_t launch_graft_batch_verify(const GraftBatchParams &p, uint32_t *leaf_words, int n_sm, cudaStream_t s,
@@ -1346,16 +1348,14 @@ cudaError_t launch_graft_batch_verify(const GraftBatchParams &p, uint32_t *leaf_
                                            : graft_batch_verify_split_kernel<false, false>)
                                    : (wide ? graft_batch_verify_split_kernel<true, true>
                                            : graft_batch_verify_split_kernel<true, false>);
-        kernel<<<split_grid(n, wide), 64, 0, s>>>(p, m, leaf_words, 1u);
-    } else if (ring_ok && !p.hash_only && !regs_only() && n >= (int64_t)n_sm * 5 * 128) {
-        const size_t smem = (size_t)128 * kGraftVerifyRing * 64;
-        graft_batch_verify_ring_kernel<<<grid, 128, smem, s>>>(p, m, leaf_words, 1u);
-    } else {
-        auto *kernel = p.hash_only ? graft_batch_verify_kernel<false> : graft_batch_verify_kernel<true>;
-        kernel<<<grid, 128, 0, s>>>(p, m, leaf_words, 1u);
+        return launch_after(kernel, split_grid(n, wide), 64, 0, s, p, m, leaf_words, 1u);
     }
-    count_launches(1);
-    return cudaGetLastError();
+    if (ring_ok && !p.hash_only && !regs_only() && n >= (int64_t)n_sm * 5 * 128) {
+        const size_t smem = (size_t)128 * kGraftVerifyRing * 64;
+        return launch_after(graft_batch_verify_ring_kernel, grid, 128, smem, s, p, m, leaf_words, 1u);
+    }
+    return launch_after(p.hash_only ? graft_batch_verify_kernel<false> : graft_batch_verify_kernel<true>, grid, 128, 0,
+                        s, p, m, leaf_words, 1u);
 }
 
 template <class Verdict>
@@ -1363,13 +1363,10 @@ static cudaError_t launch_pages(const uint32_t *leaf_words, int64_t n_pages, int
                                 const Verdict &verdict, cudaStream_t s) {
     if (n_pages == 0) return cudaSuccess;
     if (!split_off() && n_pages <= (int64_t)current_sm_count() * 8 * kSplitChains)
-        sha256_pages_split_kernel<<<(int)((n_pages + kSplitChains - 1) / kSplitChains), 64, 0, s>>>(
-            leaf_words, n_pages, leaves_per_page, verdict, 1u);
-    else
-        sha256_pages_kernel<<<(int)((n_pages + 127) / 128), 128, 0, s>>>(leaf_words, n_pages, leaves_per_page,
-                                                                         verdict, 1u);
-    count_launches(1);
-    return cudaGetLastError();
+        return launch_after(sha256_pages_split_kernel<Verdict>, (int)((n_pages + kSplitChains - 1) / kSplitChains), 64,
+                            0, s, leaf_words, n_pages, leaves_per_page, verdict, 1u);
+    return launch_after(sha256_pages_kernel<Verdict>, (int)((n_pages + 127) / 128), 128, 0, s, leaf_words, n_pages,
+                        leaves_per_page, verdict, 1u);
 }
 
 cudaError_t launch_sha256_pages(const uint32_t *leaf_words, int64_t n_pages, int64_t leaves_per_page,
