@@ -45,64 +45,38 @@ namespace kvg {
 
 namespace {
 
-template <int D>
-struct TileShape;
-template <>
-struct TileShape<64> {
-    static constexpr int TOK = 64, STAGES = 3;
-};
-// Tile rows and ring stages per head_dim (compile-time knobs, measured on
-// the GB300 decode of the 31B and 12B shapes): head_dim 128, 64 rows x 2
-// stages, 3 warps per SM (7.11 ms for batch 8 x 65,536 rows x 12 layers,
-// against 7.36 with 32 x 3 and 7.22 with 16 x 2); head_dim 256, 16 rows x 3
-// stages, 4 warps per SM (32 x 2 ties; 16 x 2, 16 x 4, 32 x 3, 64 x 2 slower).
-#ifndef KVG_DEC128_TOK
-#define KVG_DEC128_TOK 64
-#endif
-#ifndef KVG_DEC128_STAGES
-#define KVG_DEC128_STAGES 2
-#endif
-#ifndef KVG_DEC256_TOK
-#define KVG_DEC256_TOK 16
-#endif
-#ifndef KVG_DEC256_STAGES
-#define KVG_DEC256_STAGES 3
-#endif
-template <>
-struct TileShape<128> {
-    static constexpr int TOK = KVG_DEC128_TOK, STAGES = KVG_DEC128_STAGES;
-};
-template <>
-struct TileShape<256> {
-    static constexpr int TOK = KVG_DEC256_TOK, STAGES = KVG_DEC256_STAGES;
-};
-
-// fp8 tiles (knobs for head_dim 128 and 256).
-#ifndef KVG_FP8_128_TOK
-#define KVG_FP8_128_TOK 32
-#endif
-#ifndef KVG_FP8_256_TOK
-#define KVG_FP8_256_TOK 16
-#endif
-#ifndef KVG_FP8_STAGES
-#define KVG_FP8_STAGES 2
-#endif
-template <int D>
-struct Fp8TileShape {
-    static constexpr int TOK = D == 256 ? KVG_FP8_256_TOK : (D == 128 ? KVG_FP8_128_TOK : 64);
-    static constexpr int STAGES = KVG_FP8_STAGES;
-};
+// Tile rows and ring stages (measured on the GB300 decode of the 31B and 12B
+// shapes at page size 64): head_dim 128, 64 rows x 2 stages, 3 warps per SM
+// (7.11 ms for batch 8 x 65,536 rows x 12 layers, against 7.36 with 32 x 3 and
+// 7.22 with 16 x 2); head_dim 256, 16 rows x 3 stages, 4 warps per SM (32 x 2
+// ties; 16 x 2, 16 x 4, 32 x 3, 64 x 2 slower).  fp8 tiles carry half the
+// bytes; two stages per warp leave room for 8 warps per SM (the decode is
+// latency-bound per warp: more warps, not deeper rings, keep HBM busy; three
+// stages gave 0.77 of the copy peak, two 0.97).
+// A tile never spans two pages and its boxes have TOK rows whatever the page
+// holds, so pages that are no multiple of the usual tile take 16-row tiles
+// (kSmallTok): with 64-row tiles, pages of 16 rows read four times the bytes.
+// 8 sequences x 8,192 rows x 4 layers of the 31B shape, pages of 16, 32 and 48
+// rows: 1,641, 686 and 428 us before, 329, 329 and 333 with 16-row tiles (64
+// rows a page: 323); fp8 341 us -> 200 with pages of 16; 32 layers of the tiny
+// shape (head_dim 64) 829 -> 178.  Stages per ring of 16-row tiles, head_dim
+// 128: 3, 4 and 6 took 357, 325 and 446 us; head_dim 64: 3, 6 and 8 took 185,
+// 217 and 276; fp8: 3 and 4, 203 and 235.
+constexpr int kSmallTok = 16;
+constexpr int usual_tok(int D, bool fp8) { return D == 256 ? 16 : fp8 ? 32 : 64; }
+constexpr int tile_stages(int D, bool fp8, int tok) {
+    if (D == 256) return fp8 ? 2 : 3;
+    if (tok == usual_tok(D, fp8)) return D == 64 ? 3 : 2;
+    return D == 64 ? 4 : 2;
+}
 
 // FP8: the pool holds E4M3 codes; TMA brings boxes of 128 one-byte columns.
 // Keys go from the fp8 tile straight into MMA fragments; values are expanded
 // into a 16-bit staging tile with the bf16 layout (for ldmatrix.trans).
-// fp8 tiles carry half the bytes; two stages per warp leave room for 8
-// warps per SM (the decode is latency-bound per warp: more warps, not deeper
-// rings, keep HBM busy; three stages gave 0.77 of the copy peak, two 0.97)
-template <int D, bool FP8 = false>
+template <int D, bool FP8, int TOK_>
 struct Cfg {
-    static constexpr int TOK = FP8 ? Fp8TileShape<D>::TOK : TileShape<D>::TOK;
-    static constexpr int STAGES = FP8 ? Fp8TileShape<D>::STAGES : TileShape<D>::STAGES;
+    static constexpr int TOK = TOK_;
+    static constexpr int STAGES = tile_stages(D, FP8, TOK);
     static constexpr int NB = D / 64;                  // 64-column 16-bit boxes per K (or V) tile
     static constexpr int BOX = TOK * 128;              // bytes of one box (TOK rows x 128 B)
     static constexpr int NB8 = FP8 ? D / 128 : 0;      // 128-column fp8 boxes per K (or V) tile
@@ -220,9 +194,9 @@ __device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t two_codes) {
     return d;
 }
 
-template <int D, int G, bool FP8>
+template <int D, int G, bool FP8, int TOK_>
 __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap pool_map) {
-    using C = Cfg<D, FP8>;
+    using C = Cfg<D, FP8, TOK_>;
     constexpr int TOK = C::TOK, STAGES = C::STAGES, KS = C::KS, SUB = C::SUB, NB = C::NB, BOX = C::BOX;
     constexpr int NB8 = C::NB8;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -773,7 +747,7 @@ __global__ void state_finish_kernel(const float *__restrict__ state, int64_t n_r
     }
 }
 
-template <int D, int G, bool FP8>
+template <int D, int G, bool FP8, int TOK>
 struct DecodeLaunch {
     // The shared-memory attribute is per device: set and cached per device.
     static int max_blocks_per_sm() {
@@ -782,10 +756,10 @@ struct DecodeLaunch {
         if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
         int n = cached[dev].load();
         if (n > 0) return n;
-        if (cudaFuncSetAttribute(decode_kernel<D, G, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 Cfg<D, FP8>::SMEM) != cudaSuccess)
+        if (cudaFuncSetAttribute(decode_kernel<D, G, FP8, TOK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 Cfg<D, FP8, TOK>::SMEM) != cudaSuccess)
             return 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_kernel<D, G, FP8>, 32, Cfg<D, FP8>::SMEM) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_kernel<D, G, FP8, TOK>, 32, Cfg<D, FP8, TOK>::SMEM) !=
                 cudaSuccess ||
             n <= 0)
             return 0;
@@ -795,7 +769,7 @@ struct DecodeLaunch {
     static cudaError_t run(const DecodeParams &p, const CUtensorMap &map, cudaStream_t s) {
         if (max_blocks_per_sm() <= 0) return cudaErrorInvalidConfiguration;
         if (p.n_warps <= 0 || p.n_tiles <= 0) return cudaSuccess;
-        return launch_after(decode_kernel<D, G, FP8>, p.n_warps, 32, Cfg<D, FP8>::SMEM, s, p, map);
+        return launch_after(decode_kernel<D, G, FP8, TOK>, p.n_warps, 32, Cfg<D, FP8, TOK>::SMEM, s, p, map);
     }
 };
 
@@ -832,14 +806,14 @@ cudaError_t encode_tensor_map(CUtensorMap *out, int rank, void *base, const cuui
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-cudaError_t make_pool_tensor_map(CUtensorMap *out, void *pool, int head_dim, bool fp8, uint64_t rows) {
+cudaError_t make_pool_tensor_map(CUtensorMap *out, void *pool, int head_dim, bool fp8, int page_size, uint64_t rows) {
     const EncodeTiled encode = tensor_map_encoder();
     if (!encode) return cudaErrorSymbolNotFound;
     if (fp8 && head_dim % 128) {  // no fp8 decode for this head_dim: nothing to map
         memset(out, 0, sizeof *out);
         return cudaSuccess;
     }
-    const int tok = decode_tile_tokens(head_dim, fp8);  // the box height the kernel for this element type expects
+    const int tok = decode_tile_tokens(head_dim, fp8, page_size);  // the box height the kernel for this element type expects
     if (tok == 0 || rows == 0 || rows > 0x7fffffffull) return cudaErrorInvalidValue;
     // 128-byte rows per box: 64 bf16 columns, or 128 fp8 columns
     const cuuint64_t dims[2] = {(cuuint64_t)head_dim, (cuuint64_t)rows};
@@ -860,23 +834,30 @@ bool decode_supported(int head_dim, int group, bool fp8) {
     return head_dim * group <= 512;
 }
 
-int decode_tile_tokens(int head_dim, bool fp8) {
-    switch (head_dim) {
-        case 64: return fp8 ? 0 : Cfg<64>::TOK;
-        case 128: return fp8 ? Cfg<128, true>::TOK : Cfg<128>::TOK;
-        case 256: return fp8 ? Cfg<256, true>::TOK : Cfg<256>::TOK;
-    }
-    return 0;
+// The usual tile where it reads at most a tenth more rows of a page than
+// 16-row tiles do (the two are within 2% of each other on whole tiles, so what
+// decides is the rows read in vain), else those.
+int decode_tile_tokens(int head_dim, bool fp8, int page_size) {
+    if (head_dim != 64 && head_dim != 128 && head_dim != 256) return 0;
+    if (fp8 && head_dim == 64) return 0;
+    const int tok = usual_tok(head_dim, fp8);
+    const int64_t usual = ((int64_t)page_size + tok - 1) / tok * tok;
+    const int64_t small = ((int64_t)page_size + kSmallTok - 1) / kSmallTok * kSmallTok;
+    return usual * 10 <= small * 11 ? tok : kSmallTok;
 }
 
-#define KVG_DECODE_CASES(X)                                                                              \
-    X(64, 1, false) X(64, 2, false) X(64, 4, false) X(64, 8, false) X(128, 1, false) X(128, 2, false)   \
-    X(128, 4, false) X(256, 1, false) X(256, 2, false) X(128, 1, true) X(128, 2, true) X(128, 4, true) \
-    X(256, 1, true) X(256, 2, true)
+#define KVG_DECODE_CASES(X)                                                                                  \
+    X(64, 1, false, 64) X(64, 2, false, 64) X(64, 4, false, 64) X(64, 8, false, 64) X(64, 1, false, 16)     \
+    X(64, 2, false, 16) X(64, 4, false, 16) X(64, 8, false, 16) X(128, 1, false, 64) X(128, 2, false, 64)   \
+    X(128, 4, false, 64) X(128, 1, false, 16) X(128, 2, false, 16) X(128, 4, false, 16)                     \
+    X(256, 1, false, 16) X(256, 2, false, 16) X(128, 1, true, 32) X(128, 2, true, 32) X(128, 4, true, 32)   \
+    X(128, 1, true, 16) X(128, 2, true, 16) X(128, 4, true, 16) X(256, 1, true, 16) X(256, 2, true, 16)
 
-int decode_max_warps(int head_dim, int group, bool fp8, int n_sm) {
-#define KVG_CASE(DD, GG, FF) \
-    if (head_dim == DD && group == GG && fp8 == FF) return DecodeLaunch<DD, GG, FF>::max_blocks_per_sm() * n_sm;
+int decode_max_warps(int head_dim, int group, bool fp8, int page_size, int n_sm) {
+    const int tok = decode_tile_tokens(head_dim, fp8, page_size);
+#define KVG_CASE(DD, GG, FF, TT)                                        \
+    if (head_dim == DD && group == GG && fp8 == FF && tok == TT)        \
+        return DecodeLaunch<DD, GG, FF, TT>::max_blocks_per_sm() * n_sm;
     KVG_DECODE_CASES(KVG_CASE)
 #undef KVG_CASE
     return 0;
@@ -884,8 +865,10 @@ int decode_max_warps(int head_dim, int group, bool fp8, int n_sm) {
 
 cudaError_t launch_decode(int head_dim, int group, bool fp8, const DecodeParams &p, const CUtensorMap &pool_map,
                           cudaStream_t s) {
-#define KVG_CASE(DD, GG, FF) \
-    if (head_dim == DD && group == GG && fp8 == FF) return DecodeLaunch<DD, GG, FF>::run(p, pool_map, s);
+    const int tok = decode_tile_tokens(head_dim, fp8, p.page_size);
+#define KVG_CASE(DD, GG, FF, TT)                                        \
+    if (head_dim == DD && group == GG && fp8 == FF && tok == TT)        \
+        return DecodeLaunch<DD, GG, FF, TT>::run(p, pool_map, s);
     KVG_DECODE_CASES(KVG_CASE)
 #undef KVG_CASE
     return cudaErrorInvalidValue;

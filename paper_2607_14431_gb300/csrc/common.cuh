@@ -380,7 +380,7 @@ bool sha256_parts_ok();
 
 // Persistent decode: p.n_warps one-warp CTAs over p.n_tiles tiles, then the
 // combine over every (layer, row, query head).  decode_tile_tokens() is the
-// tile height TOK of the kernel for that element type (tiles per page =
+// tile height TOK of the kernel for that element type and page size (tiles per page =
 // ceil(P / TOK); the host plan and the tensor map's box must use the same
 // one as the kernel); decode_max_warps() the
 // number of co-resident warps the decode kernel can keep on the device.
@@ -392,16 +392,16 @@ cudaError_t launch_decode(int head_dim, int group, bool fp8, const DecodeParams 
                           cudaStream_t s);
 // Tensor map of a cache pool for the decode kernel: a 2-D bf16 tensor of
 // head_dim columns and n_layers*2*n_pages*n_kv_heads*page_size rows, boxes of
-// 64 columns x decode_tile_tokens(head_dim, fp8) rows, 128-byte swizzle.
-cudaError_t make_pool_tensor_map(CUtensorMap *out, void *pool, int head_dim, bool fp8, uint64_t rows);
+// 64 columns x decode_tile_tokens(head_dim, fp8, page_size) rows, 128-byte swizzle.
+cudaError_t make_pool_tensor_map(CUtensorMap *out, void *pool, int head_dim, bool fp8, int page_size, uint64_t rows);
 // A rank-`rank` bf16 tensor map (no swizzle, zero fill out of bounds): dims
 // innermost first, byte strides of dims 1.., box extents per dim.
 cudaError_t encode_tensor_map(CUtensorMap *out, int rank, void *base, const cuuint64_t *dims,
                               const cuuint64_t *strides, const cuuint32_t *box);
 cudaError_t launch_combine(int head_dim, int group, const DecodeParams &p, cudaStream_t s);
 bool decode_supported(int head_dim, int group, bool fp8 = false);
-int decode_tile_tokens(int head_dim, bool fp8);
-int decode_max_warps(int head_dim, int group, bool fp8, int n_sm);
+int decode_tile_tokens(int head_dim, bool fp8, int page_size);
+int decode_max_warps(int head_dim, int group, bool fp8, int page_size, int n_sm);
 
 // ------------------------------------- runtime.cu <-> noalloc.cu interface --
 // Read-only view of a cache's geometry and device buffers (runtime.cu fills

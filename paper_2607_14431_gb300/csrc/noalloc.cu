@@ -90,7 +90,7 @@ extern "C" kvg_status kvg_decode_attention_noalloc(kvg_cache *c, int32_t layer, 
             if (prev >= 0 && prev != dev) cudaSetDevice(prev);
         }
     } restore{prev, cs.device};
-    const int w_max = decode_max_warps(cs.head_dim, G, fp8, cs.n_sm);
+    const int w_max = decode_max_warps(cs.head_dim, G, fp8, cs.page_size, cs.n_sm);
     if (w_max <= 0) return reject(KVG_ERR_CUDA, "decode kernel cannot be made resident");
     // the launches (as kvg_decode_attention makes them); host memory only
     std::vector<DecodeParams> plan;

@@ -977,7 +977,8 @@ extern "C" kvg_status kvg_cache_create(const kvg_dims *dims, int32_t n_pages, in
     if (pool_rows > 0x7fffffffull)
         return cleanup(fail(KVG_ERR_ARG, "pool of %llu rows exceeds the decode kernel's 2^31-row addressing",
                             (unsigned long long)pool_rows));
-    if (make_pool_tensor_map(&c->pool_map, c->pool, dims->head_dim, dims->kv_dtype == KVG_KV_E4M3, pool_rows) !=
+    if (make_pool_tensor_map(&c->pool_map, c->pool, dims->head_dim, dims->kv_dtype == KVG_KV_E4M3, dims->page_size,
+                             pool_rows) !=
         cudaSuccess)
         return cleanup(fail(KVG_ERR_CUDA, "tensor map of the pool could not be encoded"));
     // the allocation-free decode's static scratch becomes resident on this
@@ -2036,7 +2037,7 @@ static kvg_status plan_decode(const kvg_cache *c, int32_t layer, const int32_t *
                               std::vector<DecodeParams> *plan, int64_t *max_units, int32_t page_begin = 0,
                               int32_t page_end = INT32_MAX) {
     const kvg_dims &d = c->dims;
-    const int TOK = decode_tile_tokens(d.head_dim, d.kv_dtype == KVG_KV_E4M3);
+    const int TOK = decode_tile_tokens(d.head_dim, d.kv_dtype == KVG_KV_E4M3, d.page_size);
     const int tpp = (d.page_size + TOK - 1) / TOK;
     std::vector<WindowGroup> parts;  // in order of first appearance
     for (int32_t l = layer < 0 ? 0 : layer; l < (layer < 0 ? d.n_layers : layer + 1); ++l) {
@@ -2152,7 +2153,7 @@ static kvg_status decode_impl(const char *what, kvg_cache *c, int32_t layer, con
         if (seq_ids[b] < 0 || seq_ids[b] >= c->max_seqs) return fail(KVG_ERR_ARG, "bad seq id %d", seq_ids[b]);
     DeviceGuard g(c->device);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int w_max = decode_max_warps(d.head_dim, G, fp8, c->n_sm);
+    const int w_max = decode_max_warps(d.head_dim, G, fp8, d.page_size, c->n_sm);
     if (w_max <= 0) return fail(KVG_ERR_CUDA, "decode kernel cannot be made resident");
     std::vector<DecodeParams> plan;
     int64_t max_units = 0;
