@@ -282,33 +282,44 @@ __global__ void __launch_bounds__(kAppendThreads) append_kernel(const AppendPara
 // the one-warp CTA keeps up to kTmaStagesMax stages in flight; the other lanes only
 // write the metadata.  The SM's ALUs stay free for concurrent work (hashing).
 // kTmaSmemBytes is the largest stage budget (KVG_APPEND_TMA_KB tunes it).
+// A small page's job is a few KiB, so what one lane does per job decides: the
+// jobs are walked with counters (four 64-bit divisions a job, twice, had taken
+// 1.1 us of it), and several CTAs share the stage budget of an SM where eight
+// stages do not fill it (8,192 rows of 4 layers, 31B shape, pages of 16, 32 and
+// 64 rows: 483, 248 and 132 us before, 103, 96 and 100 now).
 constexpr int kTmaStagesMax = 8;
+constexpr int kTmaCtasMax = 6;
 constexpr uint32_t kTmaSmemBytes = 192 * 1024;
 
-struct TmaJob {
-    int32_t lkv, jj, h, row_lo, row_hi;  // rows [row_lo, row_hi) of page jj (launch-relative)
-    int64_t tok;                          // source token (row of k/v) of row_lo
+// Job J of the launch as digits (chunk fastest, then head, page, plane), and
+// the walk over jobs J, J + gridDim.x, ...
+struct TmaWalk {
+    int32_t c, h, jj, lkv;
+    __device__ __forceinline__ TmaWalk(int64_t J, int chunks, int heads, int pages) {
+        c = (int32_t)(J % chunks);
+        J /= chunks;
+        h = (int32_t)(J % heads);
+        J /= heads;
+        jj = (int32_t)(J % pages);
+        lkv = (int32_t)(J / pages);
+    }
+    __device__ __forceinline__ void advance(const TmaWalk &by, int chunks, int heads, int pages) {
+        c += by.c;
+        h += by.h;
+        jj += by.jj;
+        lkv += by.lkv;
+        if (c >= chunks) c -= chunks, ++h;
+        if (h >= heads) h -= heads, ++jj;
+        if (jj >= pages) jj -= pages, ++lkv;
+    }
 };
 
-__device__ __forceinline__ TmaJob tma_job(const AppendParams &p, int64_t J, int chunks, int pbox) {
-    TmaJob j;
-    const int c = (int)(J % chunks);
-    J /= chunks;
-    j.h = (int32_t)(J % p.n_kv_heads);
-    J /= p.n_kv_heads;
-    j.jj = (int32_t)(J % p.pids.n);
-    j.lkv = (int32_t)(J / p.pids.n);
-    const int64_t P = p.page_size;
-    const int64_t pg = p.page0 + j.jj;
-    int64_t lo = (int64_t)p.slot0 - pg * P, hi = (int64_t)p.slot0 + p.n - pg * P;
-    if (lo < (int64_t)c * pbox) lo = (int64_t)c * pbox;
-    if (hi > (int64_t)(c + 1) * pbox) hi = (int64_t)(c + 1) * pbox;
-    if (hi > P) hi = P;
+// Rows [lo, hi) of page jj (launch-relative) that chunk c's job writes.
+__device__ __forceinline__ void tma_rows(const AppendParams &p, int jj, int c, int pbox, int &lo, int &hi) {
+    const int first = p.slot0 - (p.page0 + jj) * p.page_size;  // the launch's first row, relative to the page
+    lo = max(first, c * pbox);
+    hi = min(min(first + p.n, (c + 1) * pbox), p.page_size);
     if (hi < lo) hi = lo;
-    j.row_lo = (int32_t)lo;
-    j.row_hi = (int32_t)hi;
-    j.tok = (int64_t)p.row0 + pg * P + lo - p.slot0;
-    return j;
 }
 
 __global__ void __launch_bounds__(32) append_tma_kernel(const AppendParams p,
@@ -321,49 +332,60 @@ __global__ void __launch_bounds__(32) append_tma_kernel(const AppendParams p,
     __shared__ __align__(8) uint64_t bars[kTmaStagesMax];
     append_metadata(p);
     if (threadIdx.x != 0) return;
-    const int D = p.head_dim;
+    const int D = p.head_dim, H = p.n_kv_heads, pages = p.pids.n;
     const int64_t P = p.page_size;
     const int chunks = (int)((P + pbox - 1) / pbox);
-    const int64_t n_jobs = (int64_t)p.n_layers * 2 * p.pids.n * p.n_kv_heads * chunks;
+    const int64_t n_jobs = (int64_t)p.n_layers * 2 * pages * H * chunks;
     if (blockIdx.x >= n_jobs) return;
     const int64_t K = (n_jobs - blockIdx.x + gridDim.x - 1) / gridDim.x;  // this CTA's jobs
     const uint32_t stage_bytes = (uint32_t)pbox * D * 2;
     for (int i = 0; i < n_stages; ++i) mbar_init(&bars[i], 1);
     fence_mbar_init();
-    auto job = [&](int64_t k) { return tma_job(p, blockIdx.x + k * gridDim.x, chunks, pbox); };
-    auto load = [&](int64_t k) {
-        const TmaJob j = job(k);
-        const int st = (int)(k % n_stages);
-        if (j.row_hi == j.row_lo) {
+    const TmaWalk by(gridDim.x, chunks, H, pages);
+    TmaWalk next(blockIdx.x, chunks, H, pages), cur = next;  // the next job to load, the job to store
+    int next_stage = 0;
+    auto load = [&]() {
+        const int st = next_stage;
+        next_stage = st + 1 == n_stages ? 0 : st + 1;
+        int lo, hi;
+        tma_rows(p, next.jj, next.c, pbox, lo, hi);
+        if (hi == lo) {
             mbar_arrive(&bars[st]);
-            return;
+        } else {
+            mbar_arrive_expect_tx(&bars[st], stage_bytes);
+            const int tok = p.row0 + (p.page0 + next.jj) * (int)P + lo - p.slot0;
+            tma_load_4d(stage_mem + (size_t)st * stage_bytes, (next.lkv & 1) ? &vmap : &kmap, 0, next.h, tok,
+                        next.lkv >> 1, &bars[st]);
         }
-        mbar_arrive_expect_tx(&bars[st], stage_bytes);
-        tma_load_4d(stage_mem + (size_t)st * stage_bytes, (j.lkv & 1) ? &vmap : &kmap, 0, j.h, (int32_t)j.tok,
-                    j.lkv >> 1, &bars[st]);
+        next.advance(by, chunks, H, pages);
     };
     const int64_t pro = K < n_stages ? K : n_stages;
-    for (int64_t k = 0; k < pro; ++k) load(k);
+    for (int64_t k = 0; k < pro; ++k) load();
     int64_t loaded = pro;  // jobs [0, loaded) have a load issued
     int64_t k = 0;
+    int st = 0;
+    uint32_t phase = 0;
     for (; k < K; ++k) {
-        const int st = (int)(k % n_stages);
-        if (!mbar_wait_bounded(&bars[st], (uint32_t)((k / n_stages) & 1), limit_ns)) {
+        if (!mbar_wait_bounded(&bars[st], phase, limit_ns)) {
             record_error(status, KVG_ERR_DEVICE_CHECK, 2);
             break;
         }
-        const TmaJob j = job(k);
-        if (j.row_hi > j.row_lo) {
+        int lo, hi;
+        tma_rows(p, cur.jj, cur.c, pbox, lo, hi);
+        if (hi > lo) {
             fence_proxy_async_shared();
-            uint8_t *dst = p.pool + ((((uint64_t)j.lkv * p.pool_pages + (uint64_t)p.pids.pid[j.jj]) * p.n_kv_heads +
-                                      j.h) * P + j.row_lo) * (uint64_t)D * 2;
-            bulk_s2g(dst, stage_mem + (size_t)st * stage_bytes, (uint32_t)(j.row_hi - j.row_lo) * D * 2);
+            uint8_t *dst = p.pool + ((((uint64_t)cur.lkv * p.pool_pages + (uint64_t)p.pids.pid[cur.jj]) * H + cur.h) * P +
+                                     lo) * (uint64_t)D * 2;
+            bulk_s2g(dst, stage_mem + (size_t)st * stage_bytes, (uint32_t)(hi - lo) * D * 2);
         }
         bulk_commit();
+        cur.advance(by, chunks, H, pages);
+        if (++st == n_stages) st = 0, phase ^= 1;
         // refill the previous job's stage once its store has read it
         if (k >= 1 && loaded < K) {
             bulk_wait_read<1>();
-            load(loaded++);
+            load();
+            ++loaded;
         }
     }
     if (k < K) {
@@ -880,12 +902,13 @@ cudaError_t launch_append(const AppendParams &p, int n_sm, cudaStream_t s) {
     return launch_after(append_kernel, grid_for(rows, kAppendThreads / 32, n_sm, ctas_per_sm), kAppendThreads, 0, s, p);
 }
 
-// Rows per tensor copy: a page's rows, at most 256 (the box limit) and at
-// most 48 KiB of one kv head's rows, so that at least four stages fit.
+// Rows per tensor copy: a page's rows, or equal parts of at most 256 (the box
+// limit) and at most 48 KiB of one kv head's rows, so that at least two stages
+// fit the default budget.
 int32_t append_tma_rows(int32_t page_size, int32_t head_dim) {
-    int32_t r = page_size < 256 ? page_size : 256;
-    const int32_t cap = 49152 / (2 * head_dim);
-    return r < cap ? r : cap;
+    const int32_t cap = std::min<int32_t>(256, 49152 / (2 * head_dim));
+    const int32_t parts = (page_size + cap - 1) / cap;
+    return (page_size + parts - 1) / parts;
 }
 
 cudaError_t launch_append_tma(const AppendParams &p, DevStatus *status, int n_sm, cudaStream_t s) {
@@ -900,6 +923,7 @@ cudaError_t launch_append_tma(const AppendParams &p, DevStatus *status, int n_sm
     int n_stages = (int)(smem_budget / stage_bytes);
     if (n_stages > kTmaStagesMax) n_stages = kTmaStagesMax;
     if (n_stages < 2) return cudaErrorNotSupported;
+    const int ctas_per_sm = std::min<int>(smem_budget / ((uint32_t)n_stages * stage_bytes), kTmaCtasMax);
     // k and v: 4-D bf16 tensors (D, Hkv, n_rows_total, L); box (D, 1, pbox, 1)
     CUtensorMap maps[2];
     const cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)p.n_kv_heads, (cuuint64_t)p.n_rows_total,
@@ -923,7 +947,7 @@ cudaError_t launch_append_tma(const AppendParams &p, DevStatus *status, int n_sm
     }
     const int chunks = (p.page_size + pbox - 1) / pbox;
     const int64_t jobs = 2ll * p.n_layers * p.pids.n * p.n_kv_heads * chunks;
-    const int grid = grid_for(jobs, 1, n_sm, 1);
+    const int grid = grid_for(jobs, 1, n_sm, ctas_per_sm);
     return launch_after(append_tma_kernel, grid, 32, (size_t)n_stages * stage_bytes, s, p, maps[0], maps[1], status,
                         pbox, n_stages, 2000000000ull);
 }
