@@ -59,6 +59,7 @@ struct GraftParams {
     int32_t page_base;         // block page index of the first page of this launch
     int32_t block_pages;       // block pages per (l, kv) (stride of src planes)
     int32_t chunk_bytes;       // unit of work: divides page_bytes, multiple of 16
+    int32_t unit_pages;        // where that is a whole page: pages of a plane per unit (copy_unit_pages)
     int32_t rotate;            // 0 copy, 1 half-split rotation, 2 interleaved rotation
     int32_t n_kv_heads, page_size, head_dim;
     int64_t n_tokens;          // block tokens (rows >= n_tokens are padding)
@@ -125,6 +126,7 @@ struct GraftBatchParams {
     int64_t n_jobs;
     int32_t n_grafts;
     int32_t n_layers, page_size, chunk_bytes;
+    int32_t unit_pages;        // where a chunk is a whole page: jobs per unit
     int32_t n_kv_heads, head_dim;
     uint64_t page_bytes;
     int64_t pool_pages;
@@ -209,6 +211,7 @@ struct GatherParams {
     int32_t n_layers, npb, page_base, block_pages;
     int32_t n_kv_heads, page_size, head_dim;
     int32_t chunk_bytes;       // unit of work: divides page_bytes, whole rows
+    int32_t unit_pages;        // where that is a whole page: pages of a plane per unit
     int64_t n_tokens;          // rows >= n_tokens are written as zero
     const int32_t *src_pos;    // positions row + slot0 (nullable: no position copy)
     int32_t *dst_pos;          // block positions
@@ -302,6 +305,16 @@ uint64_t launch_count();
 // a grid-stride kernel; `fallback` when unset or not positive.
 int env_knob(const char *name, int fallback);
 
+// Pages that a copy's unit of work takes together: as many as fill 64 KiB, but
+// no more than leave four units for every SM.  A unit of one 4 KiB page keeps
+// too few bytes in flight per CTA (a plain graft of 32 layers x 8,192 tokens of
+// the tiny shape, pages of 4 KiB: 211 us, with 16 of them a unit 63).
+inline int32_t copy_unit_pages(uint64_t page_bytes, int32_t chunk_bytes, int64_t pages, int n_sm) {
+    if ((uint64_t)chunk_bytes != page_bytes) return 1;
+    int64_t q = 65536 / (int64_t)page_bytes;
+    if (q > pages / (4 * n_sm)) q = pages / (4 * n_sm);
+    return (int32_t)(q < 1 ? 1 : q);
+}
 // max_ctas > 0 caps the grid (a copy from host memory needs only enough
 // CTAs to keep the host link busy; the rest of the SMs stay free).
 // max_ctas > 0: a host-mapped source, read by at most max_ctas CTAs of

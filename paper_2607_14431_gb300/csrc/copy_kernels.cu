@@ -41,6 +41,28 @@ __device__ __forceinline__ void copy_chunk(uint8_t *__restrict__ dst, const uint
     }
 }
 
+// `pages` whole pages of vpp vectors each: page i from src(i) to dst(i).
+template <class Src, class Dst>
+__device__ __forceinline__ void copy_pages(int pages, int vpp, const Src &src, const Dst &dst) {
+    const int nvec = pages * vpp;
+    for (int base = threadIdx.x; base < nvec; base += kCopyThreads * kCopyUnroll) {
+        uint4 r[kCopyUnroll];
+        uint4 *to[kCopyUnroll];
+#pragma unroll
+        for (int u = 0; u < kCopyUnroll; ++u) {
+            const int i = base + u * kCopyThreads;
+            if (i < nvec) {
+                const int pg = i / vpp, off = i - pg * vpp;
+                r[u] = __ldcs(reinterpret_cast<const uint4 *>(src(pg)) + off);
+                to[u] = reinterpret_cast<uint4 *>(dst(pg)) + off;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kCopyUnroll; ++u)
+            if (base + u * kCopyThreads < nvec) __stcs(to[u], r[u]);
+    }
+}
+
 __device__ __forceinline__ void unpack8(const uint4 &v, float *f) {
     const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
 #pragma unroll
@@ -184,9 +206,27 @@ __global__ void __launch_bounds__(kCopyThreads) graft_kernel(const GraftParams p
     const int64_t P = p.page_size;
     graft_metadata(p);
     const uint64_t page_bytes = p.page_bytes;
+    const int row_bytes = 2 * p.head_dim;
+    if (p.unit_pages > 1) {  // small pages, several per unit
+        const int q = p.unit_pages, gpp = (p.npb + q - 1) / q;
+        const int rows_bytes = (int)page_bytes;
+        for (int64_t unit = blockIdx.x; unit < (int64_t)p.n_layers * 2 * gpp; unit += gridDim.x) {
+            const int64_t lkv = unit / gpp;
+            const int j0 = (int)(unit - lkv * gpp) * q, n = min(q, p.npb - j0);
+            const uint8_t *src0 = p.src + ((uint64_t)lkv * p.block_pages + p.page_base + j0) * page_bytes;
+            auto src = [&](int j) { return src0 + (uint64_t)j * page_bytes; };
+            auto dst = [&](int j) { return p.pool + ((uint64_t)lkv * p.pool_pages + p.pids.pid[j0 + j]) * page_bytes; };
+            if (ROT == 0 || (lkv & 1))
+                copy_pages(n, rows_bytes >> 4, src, dst);
+            else
+                for (int j = 0; j < n; ++j)
+                    rotate_chunk<ROT>(dst(j), src(j), rows_bytes, 0, (int64_t)(p.page_base + j0 + j) * P, p.head_dim,
+                                      p.page_size, p.n_tokens, ParamTrig{p});
+        }
+        return;
+    }
     const int cpp = (int)(page_bytes / (uint64_t)p.chunk_bytes);
     const int64_t n_units = (int64_t)p.n_layers * 2 * p.npb * cpp;
-    const int row_bytes = 2 * p.head_dim;
     for (int64_t unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
         const int64_t page_u = unit / cpp;
         const int chunk = (int)(unit - page_u * cpp);
@@ -562,13 +602,29 @@ __global__ void __launch_bounds__(kCopyThreads) gather_kernel(const GatherParams
                 reinterpret_cast<uint32_t *>(p.frame.base + p.frame.gap_off[g])[i] = 0;
     }
     const int cpp = (int)(p.page_bytes / (uint64_t)p.chunk_bytes);
-    const int64_t n_units = (int64_t)p.n_layers * 2 * p.npb * cpp;
+    const int q = p.unit_pages, gpp = (p.npb + q - 1) / q;  // (several whole pages a unit only where cpp is 1)
+    const int64_t n_units = (int64_t)p.n_layers * 2 * gpp * cpp;
     const int row_bytes = (int)(p.page_bytes / ((uint64_t)p.n_kv_heads * P));
     for (int64_t unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
-        const int64_t page_u = unit / cpp;
-        const uint64_t off = (uint64_t)(unit - page_u * cpp) * (uint64_t)p.chunk_bytes;
-        const int64_t lkv = page_u / p.npb;
-        const int jj = (int)(page_u - lkv * p.npb);
+        const int64_t group = unit / cpp;
+        const uint64_t off = (uint64_t)(unit - group * cpp) * (uint64_t)p.chunk_bytes;
+        const int64_t lkv = group / gpp;
+        const int j0 = (int)(group - lkv * gpp) * q;
+        int jj = j0, last = min(j0 + q, p.npb) - 1;  // the unit's pages
+        if (q > 1) {
+            // all but a ragged last page of the block together
+            const int whole = p.n_tokens - (tok0 + last * P) >= P ? last + 1 - j0 : last - j0;
+            copy_pages(
+                whole, (int)(p.page_bytes >> 4),
+                [&](int j) { return p.pool + ((uint64_t)lkv * p.pool_pages + p.pids.pid[j0 + j]) * p.page_bytes; },
+                [&](int j) {
+                    return p.dst_pids.n
+                               ? p.dst + ((uint64_t)lkv * p.pool_pages + p.dst_pids.pid[j0 + j]) * p.page_bytes
+                               : p.dst + ((uint64_t)lkv * p.block_pages + p.page_base + j0 + j) * p.page_bytes;
+                });
+            if (whole == last + 1 - j0) continue;
+            jj = last;
+        }
         const uint8_t *src = p.pool + ((uint64_t)lkv * p.pool_pages + p.pids.pid[jj]) * p.page_bytes + off;
         uint8_t *dst = off + (p.dst_pids.n
                                   ? p.dst + ((uint64_t)lkv * p.pool_pages + p.dst_pids.pid[jj]) * p.page_bytes
@@ -658,22 +714,28 @@ constexpr int kTmaGraftThreads = 256;
 
 template <int ROT>
 __device__ __forceinline__ void rotate_stage(uint8_t *stage, int bytes, int64_t first_row_in_page,
-                                             int64_t page_token0, const GraftParams &p, const float *cs) {
+                                             int64_t page_token0, int pages, const GraftParams &p, const float *cs) {
     const int D = p.head_dim;
     const int vec_per_row = D >> 3;
     const int rows = bytes / (2 * D);
     uint4 *v4 = reinterpret_cast<uint4 *>(stage);
     const int P = p.page_size;
     const int64_t nv = p.n_tokens - page_token0;
-    const int n_valid = nv < P ? (int)nv : P;
+    const bool ragged = nv < (int64_t)pages * P;  // the unit has padding rows
+    const int n_valid = ragged ? (int)nv : 0;
     const int r0 = (int)(first_row_in_page % P);
+    const int page_rows = p.n_kv_heads * P;
+    // whether row rr of the stage is padding (only a block's last page has any)
+    auto padding = [&](int rr) {
+        return ragged && (pages > 1 ? rr / page_rows * P : 0) + (r0 + rr) % P >= n_valid;
+    };
     if (ROT == 1) {
         const int half_vecs = vec_per_row >> 1;
         const int hv_shift = __ffs(half_vecs) - 1;
         const int n_items = rows * half_vecs;
         for (int it = threadIdx.x; it < n_items; it += blockDim.x) {
             const int rr = it >> hv_shift;
-            if (n_valid < P && (r0 + rr) % P >= n_valid) continue;  // padding row: unchanged
+            if (padding(rr)) continue;  // unchanged
             const int c = it & (half_vecs - 1);
             const int lo_i = rr * vec_per_row + c;
             float a[8], b[8], ra[8], rb[8];
@@ -689,7 +751,7 @@ __device__ __forceinline__ void rotate_stage(uint8_t *stage, int bytes, int64_t 
         const int n_items = rows * vec_per_row;
         for (int it = threadIdx.x; it < n_items; it += blockDim.x) {
             const int rr = it >> vr_shift;
-            if (n_valid < P && (r0 + rr) % P >= n_valid) continue;
+            if (padding(rr)) continue;
             const int c = it & (vec_per_row - 1);
             float f[8], g[8];
             unpack8(v4[it], f);
@@ -712,9 +774,10 @@ __global__ void __launch_bounds__(kTmaGraftThreads) graft_tma_kernel(const Graft
     __shared__ float cs[2 * kMaxHalfDim];
     graft_metadata(p);
     const uint64_t page_bytes = p.page_bytes;
-    const uint32_t cb = (uint32_t)p.chunk_bytes;
-    const int cpp = (int)(page_bytes / cb);
-    const int64_t n_units = (int64_t)p.n_layers * 2 * p.npb * cpp;
+    const int q = p.unit_pages, gpp = (p.npb + q - 1) / q;  // (several whole pages a unit only where cpp is 1)
+    const int cpp = (int)(page_bytes / (uint32_t)p.chunk_bytes);
+    const uint32_t cb = (uint32_t)p.chunk_bytes * q;
+    const int64_t n_units = (int64_t)p.n_layers * 2 * gpp * cpp;
     if ((int64_t)blockIdx.x >= n_units) return;  // the whole CTA
     const int64_t K = (n_units - blockIdx.x + gridDim.x - 1) / gridDim.x;  // this CTA's units
     if (ROT != 0)
@@ -729,25 +792,28 @@ __global__ void __launch_bounds__(kTmaGraftThreads) graft_tma_kernel(const Graft
     __syncthreads();
     struct Unit {
         const uint8_t *src;
-        uint8_t *dst;
-        int64_t lkv, jj;
-        uint64_t off;
+        int64_t lkv;
+        int jj, pages;   // first page, pages
+        uint64_t off;    // of a chunk within its page
+        uint32_t bytes;
     };
     auto unit = [&](int64_t k) {
         const int64_t u = (int64_t)blockIdx.x + k * gridDim.x;
-        const int64_t page_u = u / cpp;
+        const int64_t group = u / cpp;
         Unit r;
-        r.off = (uint64_t)(u - page_u * cpp) * cb;
-        r.lkv = page_u / p.npb;
-        r.jj = page_u - r.lkv * p.npb;
+        r.off = (uint64_t)(u - group * cpp) * (uint32_t)p.chunk_bytes;
+        r.lkv = group / gpp;
+        r.jj = (int)(group - r.lkv * gpp) * q;
+        r.pages = min(q, p.npb - r.jj);
+        r.bytes = (uint32_t)p.chunk_bytes * r.pages;
         r.src = p.src + ((uint64_t)r.lkv * p.block_pages + p.page_base + r.jj) * page_bytes + r.off;
-        r.dst = p.pool + ((uint64_t)r.lkv * p.pool_pages + p.pids.pid[r.jj]) * page_bytes + r.off;
         return r;
     };
     auto load = [&](int64_t k) {  // thread 0
         const int st = (int)(k % n_stages);
-        mbar_arrive_expect_tx(&bars[st], cb);
-        bulk_g2s(stage_mem + (size_t)st * cb, unit(k).src, cb, &bars[st]);
+        const Unit u = unit(k);
+        mbar_arrive_expect_tx(&bars[st], u.bytes);
+        bulk_g2s(stage_mem + (size_t)st * cb, u.src, u.bytes, &bars[st]);
     };
     const int64_t pro = K < n_stages ? K : n_stages;
     if (threadIdx.x == 0)
@@ -764,13 +830,15 @@ __global__ void __launch_bounds__(kTmaGraftThreads) graft_tma_kernel(const Graft
         const Unit u = unit(k);
         uint8_t *stage = stage_mem + (size_t)st * cb;
         if (ROT != 0 && !(u.lkv & 1)) {
-            rotate_stage<ROT>(stage, (int)cb, (int64_t)(u.off / (uint64_t)(2 * p.head_dim)),
-                              (int64_t)(p.page_base + u.jj) * p.page_size, p, cs);
+            rotate_stage<ROT>(stage, (int)u.bytes, (int64_t)(u.off / (uint64_t)(2 * p.head_dim)),
+                              (int64_t)(p.page_base + u.jj) * p.page_size, u.pages, p, cs);
             fence_proxy_async_shared();  // this thread's writes, before the bulk copy reads them
             __syncthreads();
         }
         if (threadIdx.x == 0) {
-            bulk_s2g(u.dst, stage, cb);
+            for (int j = 0; j < u.pages; ++j)
+                bulk_s2g(p.pool + ((uint64_t)u.lkv * p.pool_pages + p.pids.pid[u.jj + j]) * page_bytes + u.off,
+                         stage + (size_t)j * page_bytes, (uint32_t)p.chunk_bytes);
             bulk_commit();
             // refill the previous unit's stage once its store has read it
             if (k >= 1 && loaded < K) {
@@ -808,8 +876,33 @@ __global__ void __launch_bounds__(kCopyThreads) graft_batch_kernel(const GraftBa
     const uint64_t page_bytes = p.page_bytes;
     const int64_t cpp = (int64_t)(page_bytes / (uint64_t)p.chunk_bytes);
     const int64_t per_job = (int64_t)p.n_layers * 2 * cpp;
-    const int64_t n_units = p.n_jobs * per_job;
+    const int64_t n_units = p.unit_pages > 1 ? 0 : p.n_jobs * per_job;
     const int row_bytes = 2 * p.head_dim;
+    if (p.unit_pages > 1) {  // small pages, several jobs of a plane per unit
+        const int64_t q = p.unit_pages, gpp = (p.n_jobs + q - 1) / q;
+        for (int64_t unit = blockIdx.x; unit < (int64_t)p.n_layers * 2 * gpp; unit += gridDim.x) {
+            const int64_t lkv = unit / gpp, j0 = (unit - lkv * gpp) * q;
+            const int n = (int)(q < p.n_jobs - j0 ? q : p.n_jobs - j0);
+            auto src = [&](int j) {
+                const GraftJob &job = p.jobs[j0 + j];
+                return job.src + (uint64_t)lkv * job.block_pages * page_bytes;
+            };
+            auto dst = [&](int j) {
+                return p.pool + ((uint64_t)lkv * p.pool_pages + (uint64_t)p.jobs[j0 + j].pid) * page_bytes;
+            };
+            if (!p.rotated_only) copy_pages(n, (int)(page_bytes >> 4), src, dst);
+            if (ROT == 0 || (lkv & 1)) continue;
+            __syncthreads();  // the copies of re-based pages, before they are written again
+            for (int j = 0; j < n; ++j) {
+                const GraftJob job = p.jobs[j0 + j];
+                const GraftMeta &m = p.metas[job.meta];
+                if (m.trig < 0) continue;
+                const int half = p.head_dim >> 1;
+                rotate_chunk<ROT>(dst(j), src(j), (int)page_bytes, 0, (int64_t)job.page * p.page_size, p.head_dim,
+                                  p.page_size, m.n_tokens, TableTrig{p.trig + (int64_t)m.trig * 2 * half, half});
+            }
+        }
+    }
     for (int64_t unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
         const int64_t jb = unit / per_job;
         const int64_t rem = unit - jb * per_job;
@@ -833,7 +926,8 @@ __global__ void __launch_bounds__(kCopyThreads) graft_batch_kernel(const GraftBa
 }
 
 cudaError_t launch_graft_batch(const GraftBatchParams &p, int n_sm, cudaStream_t s, int max_ctas, int rotate) {
-    const int64_t units = p.n_jobs * p.n_layers * 2 * (int64_t)(p.page_bytes / p.chunk_bytes);
+    const int64_t units = (p.n_jobs + p.unit_pages - 1) / p.unit_pages * p.n_layers * 2 *
+                          (int64_t)(p.page_bytes / p.chunk_bytes);
     int grid = grid_for(units, 1, n_sm, 4);
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
     if (rotate == 0)
@@ -856,15 +950,17 @@ static int graft_tma_budget() {
 // The staged graft for HBM sources: one persistent CTA per SM; -1 if the
 // unit does not fit twice in the stage budget (then graft_kernel runs).
 static cudaError_t launch_graft_tma(const GraftParams &p, DevStatus *status, int n_sm, cudaStream_t s) {
-    const int64_t units = (int64_t)p.n_layers * 2 * p.npb * (int64_t)(p.page_bytes / p.chunk_bytes);
+    const int64_t units = (int64_t)p.n_layers * 2 * ((p.npb + p.unit_pages - 1) / p.unit_pages) *
+                          (int64_t)(p.page_bytes / p.chunk_bytes);
     const uint32_t budget = (uint32_t)std::min(graft_tma_budget(), 200) * 1024u;
-    int n_stages = (int)(budget / (uint32_t)p.chunk_bytes);
+    const uint32_t unit_bytes = (uint32_t)p.chunk_bytes * p.unit_pages;
+    int n_stages = (int)(budget / unit_bytes);
     if (n_stages > kTmaStagesMax) n_stages = kTmaStagesMax;
     if (n_stages < 2 || units == 0) return cudaErrorNotSupported;
     static std::atomic<bool> attr_set[kMaxDevices][3];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorNotSupported;
-    const size_t smem = (size_t)n_stages * p.chunk_bytes;
+    const size_t smem = (size_t)n_stages * unit_bytes;
     const int r = p.rotate;
     if (!attr_set[dev][r].load()) {
         cudaError_t e = r == 0 ? cudaFuncSetAttribute(graft_tma_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -889,7 +985,8 @@ cudaError_t launch_graft_copy(const GraftParams &p, int n_sm, cudaStream_t s, in
         const cudaError_t e = launch_graft_tma(p, status, n_sm, s);
         if (e != cudaErrorNotSupported) return e;
     }
-    const int64_t units = (int64_t)p.n_layers * 2 * p.npb * (int64_t)(p.page_bytes / p.chunk_bytes);
+    const int64_t units = (int64_t)p.n_layers * 2 * ((p.npb + p.unit_pages - 1) / p.unit_pages) *
+                          (int64_t)(p.page_bytes / p.chunk_bytes);
     int grid = grid_for(units, 1, n_sm, 4);
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
     return launch_after(p.rotate == 0 ? graft_kernel<0> : p.rotate == 1 ? graft_kernel<1> : graft_kernel<2>, grid,
@@ -970,7 +1067,8 @@ cudaError_t launch_append_batch(const AppendBatchParams &p, int n_sm, cudaStream
 }
 
 cudaError_t launch_gather(const GatherParams &p, int n_sm, cudaStream_t s) {
-    const int64_t units = 2ll * p.n_layers * p.npb * (int64_t)(p.page_bytes / p.chunk_bytes);
+    const int64_t units = 2ll * p.n_layers * ((p.npb + p.unit_pages - 1) / p.unit_pages) *
+                          (int64_t)(p.page_bytes / p.chunk_bytes);
     return launch_after(gather_kernel, grid_for(units, 1, n_sm, 4), kCopyThreads, 0, s, p);
 }
 

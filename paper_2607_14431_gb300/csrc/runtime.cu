@@ -1246,6 +1246,7 @@ static kvg_status pool_deposit(kvg_store *s, kvg_cache *c, int32_t seq, int32_t 
         p.pool_pages = c->n_pages;
         p.n_layers = c->dims.n_layers;
         p.npb = (int32_t)std::min<int64_t>(kMaxPagesPerLaunch, lay.n_pages - base);
+        p.unit_pages = copy_unit_pages(c->page_bytes, p.chunk_bytes, (int64_t)c->dims.n_layers * 2 * p.npb, s->n_sm);
         p.page_base = (int32_t)base;
         p.block_pages = (int32_t)lay.n_pages;
         p.n_kv_heads = c->dims.n_kv_heads;
@@ -1331,6 +1332,7 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
         p.pool_pages = c->n_pages;
         p.n_layers = c->dims.n_layers;
         p.npb = (int32_t)std::min<int64_t>(kMaxPagesPerLaunch, lay.n_pages - base);
+        p.unit_pages = copy_unit_pages(c->page_bytes, p.chunk_bytes, (int64_t)c->dims.n_layers * 2 * p.npb, s->n_sm);
         p.page_base = (int32_t)base;
         p.block_pages = (int32_t)lay.n_pages;
         p.n_kv_heads = c->dims.n_kv_heads;
@@ -1542,6 +1544,7 @@ static kvg_status pool_graft(kvg_store *s, const kvg_store::Blk &blk, kvg_cache 
         p.page_size = (int32_t)P;
         p.head_dim = c->dims.head_dim;
         p.chunk_bytes = copy_chunk_bytes(c->dims);
+        p.unit_pages = 1;
         p.n_tokens = n;
         p.src_pos = nullptr;
         p.pids.n = 1;
@@ -1716,6 +1719,7 @@ static kvg_status graft_impl(kvg_store *s, uint64_t block_id, kvg_cache *c, int3
     for (int64_t chunk = 0; chunk < n_chunks; ++chunk) {
         const int64_t base = plan[chunk].first;
         p.npb = plan[chunk].second;
+        p.unit_pages = copy_unit_pages(c->page_bytes, p.chunk_bytes, (int64_t)c->dims.n_layers * 2 * p.npb, c->n_sm);
         p.page_base = (int32_t)base;
         p.src_pos = bpos + base * P;
         p.dst_pos = c->positions + (int64_t)seq * c->max_slots + dst + base * P;
@@ -1934,6 +1938,7 @@ extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, k
     p.n_layers = c->dims.n_layers;
     p.page_size = (int32_t)P;
     p.chunk_bytes = copy_chunk_bytes(c->dims);
+    p.unit_pages = copy_unit_pages(c->page_bytes, p.chunk_bytes, (int64_t)c->dims.n_layers * 2 * pages, c->n_sm);
     p.n_kv_heads = c->dims.n_kv_heads;
     p.head_dim = c->dims.head_dim;
     p.page_bytes = c->page_bytes;

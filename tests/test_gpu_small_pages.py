@@ -1,0 +1,68 @@
+"""Copies that take several small pages at a time (graft, re-based graft, batch,
+deposit): page counts that fill units, leave a short last unit and a ragged
+last page, from HBM and pinned host memory, against grafts that take one page
+at a time (the batch of one-page units of a small block) and the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import kvg_synth as syn
+import oracle as orc
+from kvg_testlib import CANARY, append, dims_for, fill_canary, need_gpu, oracle_dims, pool_u16, tables
+
+pytestmark = pytest.mark.gpu
+
+
+# 4 KiB pages in 2 x 16 planes: from 4 x 152 pages a unit has two, from 16 x 4 x 152 sixteen
+@pytest.mark.parametrize("pages,ragged", [(18, 3), (40, 0), (57, 5), (304, 1), (700, 0), (701, 15)])
+@pytest.mark.parametrize("style", [0, 1])
+@pytest.mark.parametrize("residency", [0, 1])
+def test_units_of_several_pages(pages, ragged, style, residency):
+    kvg = need_gpu()
+    w = syn.Workload("small", 16, 2, 2, 64, 16, 10000.0, 0x90)
+    n = pages * 16 - ragged
+    dims = dims_for(kvg, w, style)
+    od = oracle_dims(orc, w, style)
+    k, v = (syn.as_u16(x) for x in syn.kv_rows(w, n, 91))
+    pos = syn.positions(0, n)
+    src = kvg.Cache(dims, pages, 1, n)
+    kvg.kvg_cache_set_free_order(src.h, syn.permutation(pages, 92))
+    append(kvg, src, 0, k, v, pos)
+    store = kvg.Store(dims, residency, 1 << 30)
+    bid = kvg.kvg_deposit(store.h, src.h, 0, 0, n)
+    blk = orc.block_from_kv(od, k, v, pos)
+    assert kvg.kvg_store_export(store.h, bid) == blk.serialize()
+    # own position; re-based; a batch of both
+    cp = 2 * pages + 5
+    slots = 2 * pages * 16
+    for how in ("graft", "batch"):
+        c = kvg.Cache(dims, cp, 2, slots)
+        fill_canary(c)
+        kvg.kvg_cache_set_free_order(c.h, syn.permutation(cp, 93))
+        oc = orc.OracleCache(od, cp, 2, slots, fill=CANARY)
+        oc.set_free_order(syn.permutation(cp, 93))
+        if how == "graft":
+            kvg.kvg_graft(store.h, bid, c.h, 0, -1, 0, 0)
+            kvg.kvg_graft(store.h, bid, c.h, 1, -1, 4097, 0)
+        else:
+            kvg.kvg_graft_batch(store.h, [bid, bid], c.h, [0, 1], 0, deltas=[0, 4097])
+        oc.graft(0, blk)
+        oc.graft(1, blk, delta=4097)
+        torch.cuda.synchronize()
+        got, want = pool_u16(c, w), oc.pool
+        pt, pf, ps = tables(c)
+        assert np.array_equal(pt, oc.page_table) and np.array_equal(pf, oc.page_fill)
+        assert np.array_equal(ps, oc.positions)
+        moved = pt[1][pt[1] >= 0]
+        keys = np.zeros(cp, bool)
+        keys[moved] = True
+        assert np.array_equal(got[:, 1], want[:, 1]) and np.array_equal(got[:, 0, ~keys], want[:, 0, ~keys])
+        # re-based keys: within the fp32 rotation's rounding of the fp64 one (the
+        # last bf16 bit), padding rows untouched
+        a, b = got[:, 0, keys].astype(np.int32), want[:, 0, keys].astype(np.int32)
+        assert (a != b).mean() < 1e-3
+        if how == "graft":
+            single = got
+        else:
+            assert np.array_equal(got, single)
+        kvg.kvg_sync(c.h)
