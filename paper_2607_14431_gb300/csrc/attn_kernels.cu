@@ -593,22 +593,26 @@ __device__ __forceinline__ int64_t warp_of(int64_t t, int64_t T, int64_t W) { re
 // divisions per partial; now the whole call takes 53.5 us instead of 98.6
 // (42 us of it the decode kernel), and one layer of the 31B shape over 2,111
 // rows 14.3 us instead of 30.7.
-template <int D>
+// Where heads x rows x layers leave most SMs idle, each head's columns are
+// shared by D / COLS blocks (COLS = 64): a block's groups are then 16 lanes, so
+// four times as many partials are in flight (one layer of the 12B shape over
+// 32,768 rows 49.1 -> 47.4 us, of the 31B shape over 2,111 rows 8.15 -> 7.84).
 struct Merged {
     float4 o;    // sum of o_w 2^(m_w - M) (threads of the first group)
     float M, L;  // maximum, sum of l_w 2^(m_w - M)
 };
 constexpr int kCombineMaxThreads = 512;
+constexpr int kNarrowBlocks = 152;  // up to this many (layer, row, head)s: a block per 64 columns
 
-template <int D>
-__device__ __forceinline__ Merged<D> merge_partials(const DecodeParams &p, int h, int b, int lr) {
-    constexpr int LANES = D / 4;
+template <int D, int COLS>
+__device__ __forceinline__ Merged merge_partials(const DecodeParams &p, int h, int col0, int b, int lr) {
+    constexpr int LANES = COLS / 4;
     __shared__ float4 sum_o[kCombineMaxThreads];
     __shared__ float sum_l[kCombineMaxThreads / LANES];
     const int G = p.n_q_heads / p.n_kv_heads;
     const int g = h / G, hh = h - g * G;
     const int d4 = threadIdx.x % LANES, r = threadIdx.x / LANES, R = blockDim.x / LANES;
-    Merged<D> res{make_float4(0.f, 0.f, 0.f, 0.f), -INFINITY, 0.f};
+    Merged res{make_float4(0.f, 0.f, 0.f, 0.f), -INFINITY, 0.f};
     const int grp = lr >= p.layer1;
     const int32_t *pref = p.rows[grp].pref_tiles;
     const int64_t Tb = pref[b + 1] - pref[b];
@@ -623,8 +627,8 @@ __device__ __forceinline__ Merged<D> merge_partials(const DecodeParams &p, int h
     const int64_t wa = warp_of(first, T, W);
     const int n = (int)(warp_of(first + Tb - 1, T, W) - wa) + 1;
     const float2 *ml = p.part_ml + (unit + wa) * G + hh;
-    const float4 *po = reinterpret_cast<const float4 *>(p.part_o + ((unit + wa) * G + hh) * D) + d4;
-    const int64_t step = (int64_t)G * LANES;  // float4 between consecutive partials
+    const float4 *po = reinterpret_cast<const float4 *>(p.part_o + ((unit + wa) * G + hh) * D + col0) + d4;
+    const int64_t step = (int64_t)G * (D / 4);  // float4 between consecutive partials
     after_previous();
     float M = -INFINITY;
     for (int i = threadIdx.x & 31; i < n; i += 32) M = fmaxf(M, ml[(int64_t)i * G].x);
@@ -675,17 +679,18 @@ __device__ __forceinline__ Merged<D> merge_partials(const DecodeParams &p, int h
     return res;
 }
 
-template <int D>
+template <int D, int COLS>
 __global__ void __launch_bounds__(kCombineMaxThreads) combine_kernel(const DecodeParams p) {
-    const int h = blockIdx.x, b = blockIdx.y, lr = blockIdx.z;
-    const Merged<D> m = merge_partials<D>(p, h, b, lr);
-    if (threadIdx.x >= D / 4) return;
+    constexpr int PARTS = D / COLS;
+    const int h = blockIdx.x / PARTS, col0 = blockIdx.x % PARTS * COLS, b = blockIdx.y, lr = blockIdx.z;
+    const Merged m = merge_partials<D, COLS>(p, h, col0, b, lr);
+    if (threadIdx.x >= COLS / 4) return;
     float r[4] = {m.o.x, m.o.y, m.o.z, m.o.w};
 #pragma unroll
     for (int e = 0; e < 4; ++e) r[e] = m.L > 0.f ? __fdiv_rn(r[e], m.L) * p.vscale : 0.f;
     const __nv_bfloat162 lo = __floats2bfloat162_rn(r[0], r[1]), hi = __floats2bfloat162_rn(r[2], r[3]);
     uint2 *out = reinterpret_cast<uint2 *>(
-        p.out + ((int64_t)(p.qlayers[lr] * p.q_row_stride_b + p.b0 + b) * p.n_q_heads + h) * D);
+        p.out + ((int64_t)(p.qlayers[lr] * p.q_row_stride_b + p.b0 + b) * p.n_q_heads + h) * D + col0);
     out[threadIdx.x] = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
 }
 
@@ -697,7 +702,7 @@ __global__ void __launch_bounds__(kCombineMaxThreads) combine_kernel(const Decod
 template <int D>
 __global__ void __launch_bounds__(kCombineMaxThreads) combine_state_kernel(const DecodeParams p) {
     const int h = blockIdx.x, b = blockIdx.y, lr = blockIdx.z;
-    const Merged<D> m = merge_partials<D>(p, h, b, lr);
+    const Merged m = merge_partials<D, D>(p, h, 0, b, lr);
     float L = m.L, M = m.M;
     float O[4] = {__fmul_rn(m.o.x, p.vscale), __fmul_rn(m.o.y, p.vscale), __fmul_rn(m.o.z, p.vscale),
                   __fmul_rn(m.o.w, p.vscale)};
@@ -874,15 +879,16 @@ cudaError_t launch_decode(int head_dim, int group, bool fp8, const DecodeParams 
     return cudaErrorInvalidValue;
 }
 
-// Threads of a combine block: a group of D/4 lanes per up to four partials of
-// the row with the most of them (the loads one thread keeps in flight).
-static int combine_threads(int head_dim, const DecodeParams &p) {
+// Threads of a combine block over `cols` columns of a head: a group of cols / 4
+// lanes per up to four partials of the row with the most of them (the loads
+// one thread keeps in flight).
+static int combine_threads(int cols, const DecodeParams &p) {
     int64_t tb = 0;
     for (int g = 0; g < (p.layer1 < p.n_layers_run ? 2 : 1); ++g)
         for (int b = 0; b < p.B; ++b)
             tb = std::max<int64_t>(tb, p.rows[g].pref_tiles[b + 1] - p.rows[g].pref_tiles[b]);
     const int64_t most = p.n_tiles > 0 ? tb * p.n_warps / p.n_tiles + 2 : 1;
-    const int lanes = head_dim / 4;
+    const int lanes = cols / 4;
     int threads = std::max(lanes, 32);
     while (threads < kCombineMaxThreads && (int64_t)(threads / lanes) * 4 < most) threads *= 2;
     return threads;
@@ -890,12 +896,18 @@ static int combine_threads(int head_dim, const DecodeParams &p) {
 
 cudaError_t launch_combine(int head_dim, int group, const DecodeParams &p, cudaStream_t s) {
     (void)group;
-    const dim3 grid(p.n_q_heads, p.B, p.n_layers_run);
-    const int n = combine_threads(head_dim, p);
+    const bool narrow = !p.state && (int64_t)p.n_q_heads * p.B * p.n_layers_run <= kNarrowBlocks;
+    const int cols = narrow ? 64 : head_dim;
+    const dim3 grid(p.n_q_heads * (head_dim / cols), p.B, p.n_layers_run);
+    const int n = combine_threads(cols, p);
     switch (head_dim) {
-        case 64: return launch_after(p.state ? combine_state_kernel<64> : combine_kernel<64>, grid, n, 0, s, p);
-        case 128: return launch_after(p.state ? combine_state_kernel<128> : combine_kernel<128>, grid, n, 0, s, p);
-        case 256: return launch_after(p.state ? combine_state_kernel<256> : combine_kernel<256>, grid, n, 0, s, p);
+        case 64: return launch_after(p.state ? combine_state_kernel<64> : combine_kernel<64, 64>, grid, n, 0, s, p);
+        case 128:
+            return launch_after(p.state ? combine_state_kernel<128>
+                                        : narrow ? combine_kernel<128, 64> : combine_kernel<128, 128>, grid, n, 0, s, p);
+        case 256:
+            return launch_after(p.state ? combine_state_kernel<256>
+                                        : narrow ? combine_kernel<256, 64> : combine_kernel<256, 256>, grid, n, 0, s, p);
     }
     return cudaErrorInvalidValue;
 }
