@@ -1299,7 +1299,6 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (!s->digest_stream) {
         KVG_CUDA(cudaStreamCreateWithFlags(&s->digest_stream, cudaStreamNonBlocking));
-        KVG_CUDA(cudaStreamCreateWithFlags(&s->page_stream, cudaStreamNonBlocking));
         KVG_CUDA(cudaEventCreateWithFlags(&s->chunk_done, cudaEventDisableTiming));
         KVG_CUDA(cudaEventCreateWithFlags(&s->pages_done, cudaEventDisableTiming));
         KVG_CUDA(cudaEventCreateWithFlags(&s->stage_free, cudaEventDisableTiming));
@@ -1365,8 +1364,6 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
     const int64_t m = (int64_t)((pb + kLeafBytes - 1) / kLeafBytes);
     const int64_t n_pages = (int64_t)d.n_layers * 2 * lay.n_pages;
     const uint64_t pos_bytes = 4ull * n;
-    KVG_CUDA(cudaEventRecord(s->chunk_done, st));
-    KVG_CUDA(cudaStreamWaitEvent(s->page_stream, s->chunk_done, 0));  // the rows are gathered
     KVG_CUDA(wait_for_leaf_scratch(s, st));
     KVG_CUDA(s->leaf.ensure((size_t)n_pages * m * 32));
     uint32_t *leaf = static_cast<uint32_t *>(s->leaf.ptr);
@@ -1375,19 +1372,33 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
     const bool parts = sha256_parts_ok() && n_pages > wave + wave / 4 &&
                        serial_blocks(pos_bytes + (uint64_t)n_pages * 32) < (1ll << 30);
     std::vector<int32_t> pos(n);
+    cudaStream_t rows = st;  // the stream the position tags are read back on
+    if (parts) {
+        if (!s->page_stream) KVG_CUDA(cudaStreamCreateWithFlags(&s->page_stream, cudaStreamNonBlocking));
+        rows = s->page_stream;
+        KVG_CUDA(cudaEventRecord(s->chunk_done, st));
+        KVG_CUDA(cudaStreamWaitEvent(rows, s->chunk_done, 0));
+    }
+    auto read_tags = [&]() {
+        const cudaError_t e = cudaMemcpyAsync(pos.data(), tgt + lay.pos_off, pos_bytes, cudaMemcpyDeviceToHost, rows);
+        return e == cudaSuccess ? cudaStreamSynchronize(rows) : e;
+    };
+    if (!parts) KVG_CUDA(read_tags());
     double grow = 1.0;
     int64_t chained = 0;  // blocks of the chain enqueued so far
+    if (parts) {  // the position tags' blocks, while the first leaves are hashed
+        KVG_CUDA(cudaStreamWaitEvent(s->digest_stream, s->chunk_done, 0));
+        KVG_CUDA(launch_sha256_serial_part(tgt + lay.pos_off, pos_bytes, tgt + lay.dig_off, (uint64_t)n_pages * 32, 0,
+                                           (int64_t)(pos_bytes / 64), tgt + 96, tgt + 96, s->digest_stream));
+        chained = (int64_t)(pos_bytes / 64);
+    }
     for (int64_t p0 = 0; p0 < n_pages;) {
         int64_t np = parts ? wave * std::max<int64_t>(1, (int64_t)grow) : n_pages;
         if (n_pages - p0 - np < wave / 2) np = n_pages - p0;
         grow *= 1.3;
         const PageSource src{tgt + lay.pages_off + (uint64_t)p0 * pb, pb, nullptr, 1, 0};
         KVG_CUDA(launch_sha256_leaves(src, np, leaf + p0 * m * 8, s->n_sm, st, !parts, parts ? leaf_ctas : 0));
-        if (p0 == 0) {
-            KVG_CUDA(cudaMemcpyAsync(pos.data(), tgt + lay.pos_off, pos_bytes, cudaMemcpyDeviceToHost,
-                                     s->page_stream));
-            KVG_CUDA(cudaStreamSynchronize(s->page_stream));
-        }
+        if (parts && p0 == 0) KVG_CUDA(read_tags());
         cudaStream_t ps = parts ? s->page_stream : st;
         if (parts) {
             KVG_CUDA(cudaEventRecord(s->chunk_done, st));
