@@ -50,29 +50,34 @@ namespace {
 // (7.11 ms for batch 8 x 65,536 rows x 12 layers, against 7.36 with 32 x 3 and
 // 7.22 with 16 x 2); head_dim 256, 16 rows x 3 stages, 4 warps per SM (32 x 2
 // ties; 16 x 2, 16 x 4, 32 x 3, 64 x 2 slower).  fp8 tiles carry half the
-// bytes; two stages per warp leave room for 8 warps per SM (the decode is
-// latency-bound per warp: more warps, not deeper rings, keep HBM busy; three
-// stages gave 0.77 of the copy peak, two 0.97).
+// bytes; their stages are at Cfg.
 // A tile never spans two pages and its boxes have TOK rows whatever the page
 // holds, so pages that are no multiple of the usual tile take 16-row tiles
 // (kSmallTok): with 64-row tiles, pages of 16 rows read four times the bytes.
 // 8 sequences x 8,192 rows x 4 layers of the 31B shape, pages of 16, 32 and 48
 // rows: 1,641, 686 and 428 us before, 329, 329 and 333 with 16-row tiles (64
-// rows a page: 323); fp8 341 us -> 200 with pages of 16; 32 layers of the tiny
-// shape (head_dim 64) 829 -> 178.  Stages per ring of 16-row tiles, head_dim
-// 128: 3, 4 and 6 took 357, 325 and 446 us; head_dim 64: 3, 6 and 8 took 185,
-// 217 and 276; fp8: 3 and 4, 203 and 235.
+// rows a page: 323); fp8 341 us -> 200 with pages of 16 (175 since the values
+// skip the staging tile); 32 layers of the tiny shape (head_dim 64) 829 -> 178.
+// Stages per ring of 16-row tiles, head_dim 128: 3, 4 and 6 took 357, 325 and
+// 446 us; head_dim 64: 3, 6 and 8 took 185, 217 and 276.
 constexpr int kSmallTok = 16;
 constexpr int usual_tok(int D, bool fp8) { return D == 256 ? 16 : fp8 ? 32 : 64; }
 constexpr int tile_stages(int D, bool fp8, int tok) {
-    if (D == 256) return fp8 ? 2 : 3;
+    if (fp8 || D == 256) return 3;
     if (tok == usual_tok(D, fp8)) return D == 64 ? 3 : 2;
     return D == 64 ? 4 : 2;
 }
 
 // FP8: the pool holds E4M3 codes; TMA brings boxes of 128 one-byte columns.
-// Keys go from the fp8 tile straight into MMA fragments; values are expanded
-// into a 16-bit staging tile with the bf16 layout (for ldmatrix.trans).
+// Keys and values go from the fp8 tile straight into fp16 MMA fragments, the
+// values through the transposing 8-bit ldmatrix: one pass over the tile, no
+// staging buffer, and a stage is refilled while the next two are read.  With
+// the values expanded into a 16-bit staging tile first the lane's own loads,
+// conversions and stores bounded it: a layer set of the 31B shape (fp8, pages
+// of 16 / 64) took 200 / 180 us and takes 175 / 171, of the 12B shape 182 / 181
+// -> 172 / 173 (6.2 TB/s).  Stages: 2 took 174 to 182, 4 took 190 and more;
+// tiles of 64 rows 182 / 174 (2 stages) and 173 / 172 (3), but 3 to 5% more on
+// short ragged sequences.
 template <int D, bool FP8, int TOK_>
 struct Cfg {
     static constexpr int TOK = TOK_;
@@ -82,8 +87,7 @@ struct Cfg {
     static constexpr int NB8 = FP8 ? D / 128 : 0;      // 128-column fp8 boxes per K (or V) tile
     static constexpr int STAGE_BYTES = FP8 ? 2 * NB8 * BOX : 2 * NB * BOX;  // K boxes then V boxes
     static constexpr int RING_BYTES = STAGES * STAGE_BYTES;
-    static constexpr int STAGING_BYTES = FP8 ? NB * BOX : 0;  // the current tile's values, expanded
-    static constexpr int SMEM = RING_BYTES + STAGING_BYTES + STAGES * (8 + 4 + 4) + 1024;  // + alignment slack
+    static constexpr int SMEM = RING_BYTES + STAGES * (8 + 4 + 4) + 1024;  // + alignment slack
     static constexpr int KS = D / 16;                  // k-steps of q.k, m-tiles of p.v
     static constexpr int SUB = TOK / 16;               // 16-row sub-tiles per tile
     static_assert(BOX % 1024 == 0, "a swizzle atom is 8 rows of 128 bytes");
@@ -135,6 +139,15 @@ __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t &r0, uint32_t &r
 
 __device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+                 : "r"(addr));
+}
+
+// Two 16x16 matrices of 8-bit elements, transposed: lanes 0-15 give the row
+// addresses of the first, lanes 16-31 of the second.  Lane (g = lane / 4, t =
+// lane % 4) gets, of each, column g's rows 4t .. 4t + 3 and column g + 8's.
+__device__ __forceinline__ void ldsm8_x2_t(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
+    asm volatile("ldmatrix.sync.aligned.m16n16.x2.trans.shared.b8 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
                  : "r"(addr));
 }
@@ -212,9 +225,8 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
     const int tpp = (P + TOK - 1) / TOK;
 
     uint8_t *ring = smem;
-    uint8_t *staging = smem + C::RING_BYTES;  // fp8: the current tile's values expanded to fp16
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + C::RING_BYTES + C::STAGING_BYTES);
-    int *vrs = reinterpret_cast<int *>(smem + C::RING_BYTES + C::STAGING_BYTES + STAGES * 8);  // valid rows [los, vrs)
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + C::RING_BYTES);
+    int *vrs = reinterpret_cast<int *>(smem + C::RING_BYTES + STAGES * 8);  // valid rows [los, vrs)
     int *los = vrs + STAGES;
     if (lane == 0) {
 #pragma unroll
@@ -267,27 +279,24 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
             ++cur.jj;
         }
         int fill, pid;
-        if (!FP8 && ahead.seq == seq && ahead.jj == jj) {
+        if (ahead.seq == seq && ahead.jj == jj) {
             fill = ahead.fill;
             pid = ahead.pid;
         } else {
             fill = p.page_fill[(int64_t)seq * p.max_pages + jj];
             pid = p.page_table[(int64_t)seq * p.max_pages + jj];
         }
-        // the next tile of this unit (same page, or the next one); the fp8
-        // kernel issues in mid-tile and measured no faster with it
-        if constexpr (!FP8) {
-            if (cur.t < cur.end && cur.jj != jj) {
-                ahead.seq = cur.seq;
-                ahead.jj = cur.jj;
-                ahead.fill = p.page_fill[(int64_t)cur.seq * p.max_pages + cur.jj];
-                ahead.pid = p.page_table[(int64_t)cur.seq * p.max_pages + cur.jj];
-            } else if (cur.jj == jj) {
-                ahead.seq = seq;
-                ahead.jj = jj;
-                ahead.fill = fill;
-                ahead.pid = pid;
-            }
+        // the next tile of this unit (same page, or the next one)
+        if (cur.t < cur.end && cur.jj != jj) {
+            ahead.seq = cur.seq;
+            ahead.jj = cur.jj;
+            ahead.fill = p.page_fill[(int64_t)cur.seq * p.max_pages + cur.jj];
+            ahead.pid = p.page_table[(int64_t)cur.seq * p.max_pages + cur.jj];
+        } else if (cur.jj == jj) {
+            ahead.seq = seq;
+            ahead.jj = jj;
+            ahead.fill = fill;
+            ahead.pid = pid;
         }
         int vr = fill - k * TOK;
         vr = vr < 0 ? 0 : (vr > TOK ? TOK : vr);
@@ -408,54 +417,25 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
             break;
         }
         const int vr = vrs[stg], lo = los[stg];
-        bool zeroed = false;
-        if constexpr (FP8) {
-            if (vr > 0) {
-                // expand the value codes into the fp16 staging tile (the swizzled
-                // box layout of a bf16 tile); rows outside [lo, vr) become zeros.
-                // All loads first, then the conversions and stores.
-                constexpr int GPR = D / 8;             // 8-value groups per row
-                constexpr int ITEMS = TOK * GPR / 32;  // per lane
-                const uint8_t *v8 = ring + stg * C::STAGE_BYTES + NB8 * BOX;
-                uint2 w[ITEMS];
-#pragma unroll
-                for (int i = 0; i < ITEMS; ++i) {
-                    const int item = i * 32 + lane, r = item / GPR, g = item % GPR;
-                    w[i] = make_uint2(0, 0);
-                    if (r >= lo && r < vr)
-                        w[i] = *reinterpret_cast<const uint2 *>(v8 + (g >> 4) * BOX + r * 128 +
-                                                                ((((g & 15) >> 1) ^ (r & 7)) << 4) + (g & 1) * 8);
-                }
-#pragma unroll
-                for (int i = 0; i < ITEMS; ++i) {
-                    const int item = i * 32 + lane, r = item / GPR, g = item % GPR;
-                    *reinterpret_cast<uint4 *>(staging + (g >> 3) * BOX + r * 128 + (((g & 7) ^ (r & 7)) << 4)) =
-                        make_uint4(e4m3x2_to_f16x2(w[i].x), e4m3x2_to_f16x2(w[i].x >> 16), e4m3x2_to_f16x2(w[i].y),
-                                   e4m3x2_to_f16x2(w[i].y >> 16));
-                }
-                __syncwarp();
-            } else if (lane == 0 && t + STAGES < t1) {
-                issue(stg);  // an empty tile: nothing to read from the stage
-            }
-        } else if (vr > 0 && (vr < TOK || lo > 0)) {
+        if (vr > 0 && (vr < TOK || lo > 0)) {
             // value rows past the fill hold whatever the pool had there, and
             // rows before a window's start are outside the attention: zero
             // both so their zero weights contribute exactly 0
-            uint4 *vz = reinterpret_cast<uint4 *>(ring + stg * C::STAGE_BYTES + NB * BOX);
+            constexpr int VB = FP8 ? NB8 : NB;  // boxes of the value tile, after as many of keys
+            uint4 *vz = reinterpret_cast<uint4 *>(ring + stg * C::STAGE_BYTES + VB * BOX);
             const int n_out = TOK - vr + lo;  // rows [0, lo) and [vr, TOK)
-            for (int idx = lane; idx < NB * n_out * 8; idx += 32) {
+            for (int idx = lane; idx < VB * n_out * 8; idx += 32) {
                 const int b = idx / (n_out * 8);
                 const int rem = idx - b * n_out * 8;
                 const int r = rem / 8 < lo ? rem / 8 : vr + (rem / 8 - lo);
                 vz[(b * BOX + r * 128) / 16 + (rem & 7)] = make_uint4(0, 0, 0, 0);
             }
             fence_proxy_async_shared();
-            zeroed = true;
             __syncwarp();
         }
         if (vr > 0) {
             const uint32_t ks_base = ring_s + stg * C::STAGE_BYTES;
-            const uint32_t vs_base = FP8 ? smem_addr(staging) : ks_base + NB * BOX;
+            const uint32_t vs_base = ks_base + (FP8 ? NB8 : NB) * BOX;
             // ---- scores S[16 rows][8 heads] per sub-tile
             float sc[SUB][4];
 #pragma unroll
@@ -500,11 +480,6 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
                 sc[sb][2] = in1 ? (acc0[2] + acc1[2]) * p.qscale : -INFINITY;
                 sc[sb][3] = in1 ? (acc0[3] + acc1[3]) * p.qscale : -INFINITY;
             }
-            if constexpr (FP8) {
-                // the keys have been read: the stage can take the next tile
-                __syncwarp();
-                if (lane == 0 && t + STAGES < t1) issue(stg);
-            }
             // ---- online softmax for heads 2*tq (e = 0) and 2*tq+1 (e = 1)
             float mt_[2] = {-INFINITY, -INFINITY};
 #pragma unroll
@@ -547,6 +522,25 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
                 uint32_t b1 = __byte_perm(y0, y1, sel);
                 if (gq >= G) b0 = b1 = 0u;
                 // ---- O^T[D][8] += V^T[D][16 rows] . P^T[16][8]
+                if constexpr (FP8) {
+                    // A's k = 2t, 2t + 1 (2t + 8, 2t + 9) are the matrix rows 4t, 4t + 1
+                    // (4t + 2, 4t + 3), so those rows are the weights' tokens 2t, 2t + 1
+                    // (8 + 2t, 8 + 2t + 1): row i comes from token 2 (i / 4) + i % 2, + 8
+                    // where i % 4 > 1
+                    const int tok = 16 * sb + 2 * ((lane & 15) >> 2) + (lane & 1) + ((lane & 2) << 2);
+                    const uint32_t v_row = vs_base + tok * 128;
+#pragma unroll
+                    for (int mt = 0; mt < KS; mt += 2) {
+                        const int m16 = mt + (lane >> 4);  // 16-byte chunk of the lane's matrix
+                        uint32_t r0, r1, r2, r3;
+                        ldsm8_x2_t(v_row + (mt >> 3) * BOX + (((m16 & 7) ^ (tok & 7)) << 4), r0, r1, r2, r3);
+                        mma16<true>(o[mt], e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r0 >> 16),
+                                    e4m3x2_to_f16x2(r1 >> 16), b0, b1);
+                        mma16<true>(o[mt + 1], e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r2 >> 16),
+                                    e4m3x2_to_f16x2(r3 >> 16), b0, b1);
+                    }
+                    continue;
+                }
                 const uint32_t v_row = vs_base + (16 * sb + (lane & 7) + ((lane >> 4) & 1) * 8) * 128;
                 const int v_hi = (lane >> 3) & 1;
 #pragma unroll
@@ -559,8 +553,7 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
             }
         }
         __syncwarp();
-        (void)zeroed;
-        if (!FP8 && lane == 0 && t + STAGES < t1) issue(stg);
+        if (lane == 0 && t + STAGES < t1) issue(stg);
     }
     if (!alive) {
         // a copy never completed: wait (bounded) on every stage once more so

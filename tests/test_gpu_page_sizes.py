@@ -69,3 +69,30 @@ def test_fp8_decode(page):
         vv = orc.e4m3_dequant(orc.e4m3_quantize(v[l], vs), vs)
         compare_decode(orc, o[l, 0], orc.gqa_decode_f64kv(q[l, 0], kk, vv, 1.0 / math.sqrt(128)), what=f"page {page}")
     kvg.kvg_sync(c.h)
+
+
+@pytest.mark.parametrize("d,g", [(128, 1), (128, 4), (256, 2)])
+@pytest.mark.parametrize("page", [16, 32, 64])
+def test_fp8_decode_rows_outside_are_not_read_as_values(page, d, g):
+    """A pool of NaN codes around the rows: a last tile that is partly filled,
+    and windows whose first row lies inside a tile."""
+    kvg = need_gpu()
+    hkv = 1
+    w = syn.Workload("nan8", 2, hkv * g, hkv, d, page, 10000.0, 0x87)
+    n = 3 * page + 7
+    ks = vs = syn.FP8_K_SCALE
+    c = kvg.Cache(kvg.make_dims(2, hkv, d, page, 10000.0, 0, kvg.KVG_KV_E4M3, ks, vs), 5, 1, n)
+    fill_canary(c)  # 0x7F, the NaN code, in every second byte
+    k, v = (syn.as_u16(x) for x in syn.kv_rows(w, n, 88))
+    append(kvg, c, 0, k, v, syn.positions(0, n))
+    q = syn.as_u16(syn.queries(w, 2, 1, 89))
+    for first in (0, 5, page + 9):
+        kvg.kvg_cache_set_layer_windows(c.h, [0, n - first if first else 0])
+        o = decode(kvg, c, w, [0], q)
+        for l in range(2):
+            lo = first if l == 1 else 0
+            kk = orc.e4m3_dequant(orc.e4m3_quantize(k[l][lo:], ks), ks)
+            vv = orc.e4m3_dequant(orc.e4m3_quantize(v[l][lo:], vs), vs)
+            compare_decode(orc, o[l, 0], orc.gqa_decode_f64kv(q[l, 0], kk, vv, 1.0 / math.sqrt(d)),
+                           what=f"page {page} layer {l} from {lo}")
+    kvg.kvg_sync(c.h)
