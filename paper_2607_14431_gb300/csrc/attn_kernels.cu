@@ -90,6 +90,7 @@ struct Cfg {
     static constexpr int SMEM = RING_BYTES + STAGES * (8 + 4 + 4) + 1024;  // + alignment slack
     static constexpr int KS = D / 16;                  // k-steps of q.k, m-tiles of p.v
     static constexpr int SUB = TOK / 16;               // 16-row sub-tiles per tile
+    static constexpr bool WALK = FP8 || D == 64;       // steps from unit to unit instead of searching
     static_assert(BOX % 1024 == 0, "a swizzle atom is 8 rows of 128 bytes");
     static_assert(!FP8 || D % 128 == 0, "fp8 tiles are whole 128-byte boxes");
 };
@@ -128,6 +129,31 @@ __device__ __forceinline__ TilePos locate(const DecodeParams &p, int64_t t) {
     r.unit = ((int64_t)r.lr * p.B + r.b) * p.n_kv_heads + r.g;
     return r;
 }
+
+// The first tile of the unit after r's; there is one if any tile is left.
+__device__ __forceinline__ void next_unit(const DecodeParams &p, TilePos &r) {
+    r.tile = 0;
+    if (++r.g == p.n_kv_heads) {
+        r.g = 0;
+        do {
+            if (++r.b == p.B) {
+                r.b = 0;
+                if (++r.lr == p.layer1) r.grp = 1;
+            }
+            const int32_t *pref = p.rows[r.grp].pref_tiles;
+            r.n_tiles = pref[r.b + 1] - pref[r.b];
+        } while (r.n_tiles == 0);
+    }
+    r.unit = ((int64_t)r.lr * p.B + r.b) * p.n_kv_heads + r.g;
+}
+
+// Row of q that the unit's first query head has.
+template <int G>
+__device__ __forceinline__ int64_t q_row(const DecodeParams &p, const TilePos &r) {
+    return (int64_t)(p.qlayers[r.lr] * p.q_row_stride_b + p.b0 + r.b) * p.n_q_heads + r.g * G;
+}
+
+__device__ __forceinline__ void prefetch_l1(const void *ptr) { asm volatile("prefetch.global.L1 [%0];" ::"l"(ptr)); }
 
 __device__ __forceinline__ int64_t warp_start(int64_t w, int64_t T, int64_t W) { return w * T / W; }
 
@@ -208,7 +234,7 @@ __device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t two_codes) {
 }
 
 template <int D, int G, bool FP8, int TOK_>
-__global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap pool_map) {
+__global__ void __launch_bounds__(32, FP8 && D == 128 ? 16 : 0) decode_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap pool_map) {
     using C = Cfg<D, FP8, TOK_>;
     constexpr int TOK = C::TOK, STAGES = C::STAGES, KS = C::KS, SUB = C::SUB, NB = C::NB, BOX = C::BOX;
     constexpr int NB8 = C::NB8;
@@ -240,19 +266,30 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
     const int64_t plane_rows = p.pool_pages * (int64_t)p.n_kv_heads * P;  // rows per (layer, K/V)
 
     // Lane 0's cursor over the tiles it copies: tiles are issued in order, so
-    // the position advances by one; it is re-located only at a unit boundary.
+    // the position advances by one.  At a unit's end it steps to the unit after
+    // (WALK), with the row's first page entry and the queries at hand, where
+    // a search for the tile and the loads that follow it cost 2 to 5 us, much
+    // where a warp has several units: 38 rows x 149 .. 206 fp8 tokens x 10
+    // layers of the 31B shape 89.5 -> 83.5 us, 28 x 3,878 .. 13,730 tokens x 4
+    // layers of the tiny shape 54.1 -> 49.3, 3 x 142 .. 253 fp8 tokens x 11
+    // layers of the 12B shape 17.8 -> 17.2.  bf16 tiles of head_dim 128 and 256
+    // hold up to 32 KB, so a unit is few tiles and the step gains 1 to 2% on
+    // short rows, but costs a one-layer call over 2,111 rows 7.81 -> 8.01 us
+    // and 32 x 8,192 .. 24,576 rows of the 12B shape 1,266 -> 1,297: they search.
     struct Cursor {
         int64_t t, end;  // next tile to issue; first tile past its unit
-        int lr, b, g, seq, jj, k;
+        TilePos tp;      // its unit
+        int seq, jj, k;
         int lo;          // rows before the window start in the next tile (its unit's first only)
     } cur;
     cur.t = t0;
     cur.end = t0;
     auto advance_to_unit = [&]() {
-        const TilePos tp = locate(p, cur.t);
-        cur.lr = tp.lr;
-        cur.b = tp.b;
-        cur.g = tp.g;
+        if (!C::WALK || cur.t == t0)
+            cur.tp = locate(p, cur.t);
+        else
+            next_unit(p, cur.tp);
+        const TilePos &tp = cur.tp;
         cur.seq = p.seq[tp.b];
         const int tile = tp.tile + p.rows[tp.grp].tile0[tp.b];
         cur.jj = tile / tpp;
@@ -266,12 +303,20 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
     // tile's compute instead of stalling the warp at the issue.
     struct PageAhead {
         int seq = -1, jj = -1, fill = 0, pid = -1;
-    } ahead;
+    } ahead, first;  // first: of the unit's first page, which the row's next kv head reads too
     // lane 0: arm the stage's barrier and copy the next tile's K and V boxes
     auto issue = [&](int stg) {
-        if (cur.t >= cur.end) advance_to_unit();
+        const bool entered = cur.t >= cur.end;
+        if (entered) {
+            advance_to_unit();
+            if (C::WALK && cur.t != t0) {
+                // the unit's queries, some tiles before they are read
+                const uint8_t *qp = reinterpret_cast<const uint8_t *>(p.q + q_row<G>(p, cur.tp) * D);
+#pragma unroll
+                for (int i = 0; i < G * D * 2; i += 128) prefetch_l1(qp + i);
+            }
+        }
         const int seq = cur.seq, jj = cur.jj, k = cur.k, lo = cur.lo;
-        struct { int lr, g; } tp{cur.lr, cur.g};
         ++cur.t;
         cur.lo = 0;
         if (++cur.k == tpp) {
@@ -282,9 +327,18 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
         if (ahead.seq == seq && ahead.jj == jj) {
             fill = ahead.fill;
             pid = ahead.pid;
+        } else if (C::WALK && first.seq == seq && first.jj == jj) {
+            fill = first.fill;
+            pid = first.pid;
         } else {
             fill = p.page_fill[(int64_t)seq * p.max_pages + jj];
             pid = p.page_table[(int64_t)seq * p.max_pages + jj];
+        }
+        if (C::WALK && entered) {
+            first.seq = seq;
+            first.jj = jj;
+            first.fill = fill;
+            first.pid = pid;
         }
         // the next tile of this unit (same page, or the next one)
         if (cur.t < cur.end && cur.jj != jj) {
@@ -310,8 +364,8 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
         uint64_t *bar = &bars[stg];
         if (vr > 0) {
             mbar_arrive_expect_tx(bar, (uint32_t)C::STAGE_BYTES);
-            const int l = p.layers[tp.lr];
-            const int32_t row_k = (int32_t)((2 * l) * plane_rows + ((int64_t)pid * p.n_kv_heads + tp.g) * P +
+            const int l = p.layers[cur.tp.lr];
+            const int32_t row_k = (int32_t)((2 * l) * plane_rows + ((int64_t)pid * p.n_kv_heads + cur.tp.g) * P +
                                             (int64_t)k * TOK);
             const int32_t row_v = (int32_t)(row_k + plane_rows);
             uint8_t *dst = ring + stg * C::STAGE_BYTES;
@@ -336,7 +390,6 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
     uint32_t qb[KS][2];   // B fragments of q (heads gq < G), per k-step
     float o[KS][4];       // O^T accumulators: dims 16*mt + gq (+8), heads 2*tq (+1)
     float m[2], lsum[2];  // running max / partial sum of heads 2*tq, 2*tq+1
-    int64_t cur_unit = -1;
 
     auto flush = [&](int64_t unit) {
         float lt[2];
@@ -365,8 +418,7 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
     };
 
     auto begin = [&](const TilePos &tp) {
-        const __nv_bfloat16 *qrow =
-            p.q + ((int64_t)(p.qlayers[tp.lr] * p.q_row_stride_b + p.b0 + tp.b) * p.n_q_heads + tp.g * G) * D;
+        const __nv_bfloat16 *qrow = p.q + q_row<G>(p, tp) * D;
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) {
             if (gq < G) {
@@ -397,18 +449,21 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
 
     const uint32_t ring_s = smem_addr(ring);
     bool alive = true;
-    int64_t unit_end = t0;  // first tile past the current unit
+    TilePos rd;             // the current unit
+    int64_t unit_end = t0;  // first tile past it
     for (int64_t t = t0; t < t1; ++t) {
         const int64_t i = t - t0;
         const int stg = (int)(i % STAGES);
         if (t == t1 - 1) let_next_start();
         const uint32_t par = (uint32_t)((i / STAGES) & 1);
         if (t >= unit_end) {
-            const TilePos tp = locate(p, t);
-            if (cur_unit >= 0) flush(cur_unit);
-            begin(tp);
-            cur_unit = tp.unit;
-            unit_end = t - tp.tile + tp.n_tiles;
+            if (unit_end > t0) flush(rd.unit);
+            if (!C::WALK || unit_end == t0)
+                rd = locate(p, t);
+            else
+                next_unit(p, rd);
+            begin(rd);
+            unit_end = t - rd.tile + rd.n_tiles;
         }
         const bool ok = mbar_wait_bounded(&bars[stg], par);
         if (!__all_sync(0xffffffffu, ok)) {
@@ -567,7 +622,7 @@ __global__ void __launch_bounds__(32) decode_kernel(const DecodeParams p, const 
         m[0] = m[1] = -INFINITY;
         lsum[0] = lsum[1] = 0.f;
     }
-    if (cur_unit >= 0) flush(cur_unit);
+    if (unit_end > t0) flush(rd.unit);
 }
 
 // Largest warp index whose range starts at or before tile t.
