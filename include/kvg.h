@@ -307,9 +307,9 @@ kvg_status kvg_cache_release(kvg_cache *cache, int32_t seq, void *stream);
  * same rows anywhere else.  KVG_ERR_CAPACITY if the store is full.
  * Ordering: the call returns once the rows are gathered (it reads the
  * position tags back to bound later relocations).  The page digests follow
- * on `stream`, so work enqueued later on `stream` (a graft, a verification)
- * sees the whole block but its block digest, which one serial SHA-256 chain
- * computes on a library stream; kvg_store_block_info, kvg_store_export and
+ * in `stream` order, so work enqueued later on `stream` (a graft, a
+ * verification) sees the whole block but its block digest, which one serial
+ * SHA-256 chain computes on a library stream; kvg_store_block_info, kvg_store_export and
  * kvg_store_save wait for it.  A pinned-host store's block is assembled and
  * hashed in an HBM staging buffer (grown to the largest block deposited into
  * that store) and copied out: everything but the 256-byte header in `stream`
@@ -399,8 +399,8 @@ kvg_status kvg_graft_chunked(kvg_store *store, uint64_t block_id, kvg_cache *cac
  * grafted (KVG_ERR_POSITION when tags + delta leave [0, 2^31), KVG_ERR_ARG
  * for a nonzero delta on an fp8 cache).  Not for pool-resident stores
  * (KVG_ERR_ARG; use kvg_graft).  flags as for kvg_graft: KVG_GRAFT_VERIFY
- * hashes each own-position graft's restored pages, and each re-based
- * graft's stored pages, after the copies; the report's seq is the (last)
+ * hashes each own-position graft's pages as it copies them, and each
+ * re-based graft's stored pages after the copies; the report's seq is the (last)
  * failing graft's sequence and mismatch_pages its block page indices.  The
  * call stages its job table in library-owned pinned memory and waits for
  * the previous batch's table copy on this cache before reusing it. */
@@ -523,8 +523,8 @@ kvg_status kvg_decode_attention_noalloc(kvg_cache *cache, int32_t layer, const i
 /* SHA-256 (FIPS 180-4) on the GPU.
  * KVG_SHA256_PLAIN: out[32] = SHA-256 of bytes[0, n): one serial chain (one
  *   warp expands each block's message schedule while another runs the
- *   rounds when bytes is 4-byte aligned), about 0.85 us per 64-byte block
- *   (~75 MB/s; 1.5 us unaligned) — meant for short messages such as
+ *   rounds when bytes is 4-byte aligned), about 0.74 us per 64-byte block
+ *   (~86 MB/s; 1.5 us unaligned) — meant for short messages such as
  *   headers and test vectors; page contents use KVG_SHA256_PAGED.
  * KVG_SHA256_PAGED: n must be a multiple of page_bytes; out[32 * i] = the
  *   two-level digest of page i = bytes[i * page_bytes, (i+1) * page_bytes).

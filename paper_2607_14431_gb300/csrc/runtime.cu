@@ -1355,10 +1355,10 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
     // takes in, and the page digests and the chain have the others to themselves
     // (beside a leaf CTA a page chunk's digests took 92 us instead of 35, and a
     // block of the chain 0.88 instead of 0.80).  A chunk is one round of those
-    // CTAs; later ones grow, since the hashing runs ahead.  The call waits for the rows (it reads the position
-    // tags back, which bound later relocations) but not for the digests, and
-    // everything that reads a block digest (block info, export, save)
-    // synchronizes the device first.
+    // CTAs; later ones grow, since the hashing runs ahead.  The call waits for
+    // the rows (it reads the position tags back, which bound later
+    // relocations) but not for the digests, and everything that reads a block
+    // digest (block info, export, save) synchronizes the device first.
     const kvg_dims &d = s->dims;
     const uint64_t pb = page_bytes_of(d);
     const int64_t m = (int64_t)((pb + kLeafBytes - 1) / kLeafBytes);

@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(128) sha256_leaves_kernel(const PageSource src
 // registers, measured slower in the step).  For smaller launches each leaf's
 // chain latency decides: the register form is faster there (the tiny
 // verified graft 0.099 against 0.133 ms), and the two-warp form faster still
-// for launches of up to 64 leaves per SM (0.071 ms).
+// for launches of up to 64 leaves per SM (0.057 ms).
 constexpr int kGraftVerifyRing = 3;
 __global__ void __launch_bounds__(128, 5) graft_verify_ring_kernel(const GraftParams p, int64_t leaves_per_page,
                                                                    uint32_t *__restrict__ out, uint32_t one) {
