@@ -200,14 +200,18 @@ __device__ __forceinline__ void rotate_chunk(uint8_t *__restrict__ dst, const ui
     }
 }
 
-template <int ROT>
+// MANY: small pages, several per unit.  An instance of its own: with both loops
+// in one kernel the copies out of host memory kept more registers, and beside an
+// append and the chunks' hashes their CTAs found room later (one 3.2 GB block
+// with its decode 15.64 ms -> 16.65, a 403 MB one 2.11 -> 2.27).
+template <int ROT, bool MANY>
 __global__ void __launch_bounds__(kCopyThreads) graft_kernel(const GraftParams p) {
     after_previous();
     const int64_t P = p.page_size;
     graft_metadata(p);
     const uint64_t page_bytes = p.page_bytes;
     const int row_bytes = 2 * p.head_dim;
-    if (p.unit_pages > 1) {  // small pages, several per unit
+    if constexpr (MANY) {
         const int q = p.unit_pages, gpp = (p.npb + q - 1) / q;
         const int rows_bytes = (int)page_bytes;
         for (int64_t unit = blockIdx.x; unit < (int64_t)p.n_layers * 2 * gpp; unit += gridDim.x) {
@@ -870,15 +874,16 @@ int grid_for(int64_t work_items, int per_block, int n_sm, int waves) {
 // SM busy to its end instead of draining after each graft.  ROT > 0: some
 // grafts are re-based (their key chunks rotate with their own cos/sin table,
 // as the single-graft kernels do; values and own-position grafts copy).
-template <int ROT>
+// MANY: small pages, several jobs of a plane per unit.
+template <int ROT, bool MANY>
 __global__ void __launch_bounds__(kCopyThreads) graft_batch_kernel(const GraftBatchParams p) {
     after_previous();
     const uint64_t page_bytes = p.page_bytes;
     const int64_t cpp = (int64_t)(page_bytes / (uint64_t)p.chunk_bytes);
     const int64_t per_job = (int64_t)p.n_layers * 2 * cpp;
-    const int64_t n_units = p.unit_pages > 1 ? 0 : p.n_jobs * per_job;
+    const int64_t n_units = MANY ? 0 : p.n_jobs * per_job;
     const int row_bytes = 2 * p.head_dim;
-    if (p.unit_pages > 1) {  // small pages, several jobs of a plane per unit
+    if constexpr (MANY) {
         const int64_t q = p.unit_pages, gpp = (p.n_jobs + q - 1) / q;
         for (int64_t unit = blockIdx.x; unit < (int64_t)p.n_layers * 2 * gpp; unit += gridDim.x) {
             const int64_t lkv = unit / gpp, j0 = (unit - lkv * gpp) * q;
@@ -930,9 +935,15 @@ cudaError_t launch_graft_batch(const GraftBatchParams &p, int n_sm, cudaStream_t
                           (int64_t)(p.page_bytes / p.chunk_bytes);
     int grid = grid_for(units, 1, n_sm, 4);
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
-    if (rotate == 0)
-        return launch_after(graft_batch_kernel<0>, grid, kCopyThreads, 0, s, p);
-    return launch_after(rotate == 1 ? graft_batch_kernel<1> : graft_batch_kernel<2>, grid, kCopyThreads, 0, s, p);
+    if (p.unit_pages > 1)
+        return launch_after(rotate == 0   ? graft_batch_kernel<0, true>
+                            : rotate == 1 ? graft_batch_kernel<1, true>
+                                          : graft_batch_kernel<2, true>,
+                            grid, kCopyThreads, 0, s, p);
+    return launch_after(rotate == 0   ? graft_batch_kernel<0, false>
+                        : rotate == 1 ? graft_batch_kernel<1, false>
+                                      : graft_batch_kernel<2, false>,
+                        grid, kCopyThreads, 0, s, p);
 }
 
 // Shared-memory stage budget of graft_tma_kernel (KVG_GRAFT_TMA_KB, 0 turns
@@ -989,8 +1000,15 @@ cudaError_t launch_graft_copy(const GraftParams &p, int n_sm, cudaStream_t s, in
                           (int64_t)(p.page_bytes / p.chunk_bytes);
     int grid = grid_for(units, 1, n_sm, 4);
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
-    return launch_after(p.rotate == 0 ? graft_kernel<0> : p.rotate == 1 ? graft_kernel<1> : graft_kernel<2>, grid,
-                        kCopyThreads, 0, s, p);
+    if (p.unit_pages > 1)
+        return launch_after(p.rotate == 0   ? graft_kernel<0, true>
+                            : p.rotate == 1 ? graft_kernel<1, true>
+                                            : graft_kernel<2, true>,
+                            grid, kCopyThreads, 0, s, p);
+    return launch_after(p.rotate == 0   ? graft_kernel<0, false>
+                        : p.rotate == 1 ? graft_kernel<1, false>
+                                        : graft_kernel<2, false>,
+                        grid, kCopyThreads, 0, s, p);
 }
 
 cudaError_t launch_append(const AppendParams &p, int n_sm, cudaStream_t s) {
