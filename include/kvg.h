@@ -428,11 +428,11 @@ kvg_status kvg_verify(kvg_store *store, uint64_t block_id, kvg_cache *cache, int
  * over every valid row of the sequence (pages in logical order, rows below
  * their fill) — on a windowed layer (kvg_cache_set_layer_windows) over its
  * last W valid rows — accumulated in fp32 and rounded to bf16 (RNE).  An
- * empty sequence gives o = 0.  Layers with more than two different windows
- * run as several launches on the stream.
+ * empty sequence gives o = 0.  Layers of different windows may run as several
+ * launches on the stream; a layer's reduction is the same either way.
  * q, out: device bf16 [n_layers_run][B][n_q_heads][head_dim] where
  * layer >= 0 runs that layer only (n_layers_run = 1) and layer == -1 runs all
- * layers in one launch.  The reduction order depends only on the logical
+ * layers in one call.  The reduction order depends only on the logical
  * token index, never on physical page placement, so results are bitwise
  * reproducible and identical for grafted and freshly written rows.
  * n_q_heads must be a multiple of n_kv_heads with group size in {1, 2, 4, 8}
@@ -496,13 +496,12 @@ kvg_status kvg_decode_state_finish(const float *state, int64_t n_rows, int32_t h
  * (no cudaMalloc, cudaFree or library allocator).  Arguments, results and
  * errors are those of kvg_decode_attention, with these differences:
  *   - the partials take (units + workers) * G * (4 * head_dim + 8) bytes,
- *     units = (layers of one launch: those sharing a window, or those of two
- *     windows where that fits with every worker; at most 256)
- *     * min(B, 256) * n_kv_heads, G = n_q_heads /
- *     n_kv_heads; the number of decode workers (warps) is capped so they fit
- *     in 16 MiB - 256 bytes, and a call that does not fit even with one
- *     worker returns KVG_ERR_CAPACITY with an explanatory kvg_last_error()
- *     and enqueues nothing;
+ *     units = (layers of one launch: those sharing a window, at most 256)
+ *     * min(B, 256) * n_kv_heads, G = n_q_heads / n_kv_heads; the number of
+ *     decode workers (warps) is capped so they fit in 16 MiB - 256 bytes, and
+ *     a call that does not fit even with one worker returns KVG_ERR_CAPACITY
+ *     with an explanatory kvg_last_error() and enqueues nothing.  (Two windows
+ *     share a launch only where both fit with every worker for each.);
  *   - the array's device address is looked up (cudaGetSymbolAddress, with
  *     the device current) by kvg_cache_create, once per device: that is when
  *     the module holding the array is made resident on the device and its

@@ -155,7 +155,10 @@ __device__ __forceinline__ int64_t q_row(const DecodeParams &p, const TilePos &r
 
 __device__ __forceinline__ void prefetch_l1(const void *ptr) { asm volatile("prefetch.global.L1 [%0];" ::"l"(ptr)); }
 
-__device__ __forceinline__ int64_t warp_start(int64_t w, int64_t T, int64_t W) { return w * T / W; }
+// First tile (of the group's) of warp w's range.
+__device__ __forceinline__ int64_t warp_start(const DecodeParams &p, int g, int64_t w) {
+    return w * p.group_tiles(g) / p.n_warps[g];
+}
 
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -244,9 +247,11 @@ __global__ void __launch_bounds__(32, FP8 && D == 128 ? 16 : 0) decode_kernel(co
 
     const int lane = threadIdx.x;
     const int gq = lane >> 2, tq = lane & 3;  // mma fragment coordinates
-    const int64_t w = blockIdx.x;
-    const int64_t t0 = warp_start(w, p.n_tiles, p.n_warps);
-    const int64_t t1 = warp_start(w + 1, p.n_tiles, p.n_warps);
+    const int grp = (int)blockIdx.x >= p.n_warps[0];  // the second group's warps follow the first's
+    const int w = (int)blockIdx.x - (grp ? p.n_warps[0] : 0);
+    const int64_t base = grp ? p.tile1 : 0;
+    const int64_t t0 = base + warp_start(p, grp, w);
+    const int64_t t1 = base + warp_start(p, grp, w + 1);
     const int P = p.page_size;
     const int tpp = (P + TOK - 1) / TOK;
 
@@ -401,7 +406,7 @@ __global__ void __launch_bounds__(32, FP8 && D == 128 ? 16 : 0) decode_kernel(co
             v += __shfl_xor_sync(0xffffffffu, v, 16);
             lt[e] = v;
         }
-        const int64_t slot = unit + w;
+        const int64_t slot = unit + blockIdx.x;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int h = 2 * tq + e;
@@ -668,14 +673,15 @@ __device__ __forceinline__ Merged merge_partials(const DecodeParams &p, int h, i
         after_previous();
         return res;
     }
-    const int64_t T = p.n_tiles, W = p.n_warps;
+    const int64_t T = p.group_tiles(grp), W = p.n_warps[grp];
     const int64_t unit = ((int64_t)lr * p.B + b) * p.n_kv_heads + g;
-    const int64_t first = (grp ? p.tile1 : 0) + (int64_t)g * Tb +
+    const int64_t first = (int64_t)g * Tb +  // of the group's tiles
                           (int64_t)p.n_kv_heads * ((int64_t)(lr - (grp ? p.layer1 : 0)) * pref[p.B] + pref[b]);
     const int64_t wa = warp_of(first, T, W);
     const int n = (int)(warp_of(first + Tb - 1, T, W) - wa) + 1;
-    const float2 *ml = p.part_ml + (unit + wa) * G + hh;
-    const float4 *po = reinterpret_cast<const float4 *>(p.part_o + ((unit + wa) * G + hh) * D + col0) + d4;
+    const int64_t slot = unit + wa + (grp ? p.n_warps[0] : 0);
+    const float2 *ml = p.part_ml + slot * G + hh;
+    const float4 *po = reinterpret_cast<const float4 *>(p.part_o + (slot * G + hh) * D + col0) + d4;
     const int64_t step = (int64_t)G * (D / 4);  // float4 between consecutive partials
     after_previous();
     float M = -INFINITY;
@@ -821,8 +827,9 @@ struct DecodeLaunch {
     }
     static cudaError_t run(const DecodeParams &p, const CUtensorMap &map, cudaStream_t s) {
         if (max_blocks_per_sm() <= 0) return cudaErrorInvalidConfiguration;
-        if (p.n_warps <= 0 || p.n_tiles <= 0) return cudaSuccess;
-        return launch_after(decode_kernel<D, G, FP8, TOK>, p.n_warps, 32, Cfg<D, FP8, TOK>::SMEM, s, p, map);
+        if (p.n_tiles <= 0) return cudaSuccess;
+        return launch_after(decode_kernel<D, G, FP8, TOK>, p.n_warps[0] + p.n_warps[1], 32, Cfg<D, FP8, TOK>::SMEM, s,
+                            p, map);
     }
 };
 
@@ -931,11 +938,14 @@ cudaError_t launch_decode(int head_dim, int group, bool fp8, const DecodeParams 
 // lanes per up to four partials of the row with the most of them (the loads
 // one thread keeps in flight).
 static int combine_threads(int cols, const DecodeParams &p) {
-    int64_t tb = 0;
-    for (int g = 0; g < (p.layer1 < p.n_layers_run ? 2 : 1); ++g)
+    int64_t most = 1;
+    for (int g = 0; g < kMaxWindowGroups; ++g) {
+        if (p.group_tiles(g) <= 0) continue;
+        int64_t tb = 0;
         for (int b = 0; b < p.B; ++b)
             tb = std::max<int64_t>(tb, p.rows[g].pref_tiles[b + 1] - p.rows[g].pref_tiles[b]);
-    const int64_t most = p.n_tiles > 0 ? tb * p.n_warps / p.n_tiles + 2 : 1;
+        most = std::max(most, tb * p.n_warps[g] / p.group_tiles(g) + 2);
+    }
     const int lanes = cols / 4;
     int threads = std::max(lanes, 32);
     while (threads < kCombineMaxThreads && (int64_t)(threads / lanes) * 4 < most) threads *= 2;

@@ -256,11 +256,14 @@ struct PageSource {
 // A launch covers Lrun layers x B batch rows x Hkv kv heads ("units").  Unit
 // (l, b, g) owns the T_b tiles its layer reads of row b (all of them, or a
 // window's), in page order; the global tile list orders units (l, b, g) with
-// g fastest.  Warp w of W takes the contiguous range [w*T/W, (w+1)*T/W) and
-// writes one partial per unit it touches, at slot unit + w (unique because
-// both ranges are contiguous).  The run layers are ordered in up to
-// kMaxWindowGroups groups that read the same tiles of a row: layers
-// [0, layer1) by rows[0], the others by rows[1].
+// g fastest.  The run layers are ordered in up to kMaxWindowGroups groups that
+// read the same tiles of a row: layers [0, layer1) by rows[0], the others by
+// rows[1].  Of each group's T tiles warp w of the group's W takes the
+// contiguous range [w*T/W, (w+1)*T/W) and writes one partial per unit it
+// touches, at slot unit + w (second group, whose warps are the CTAs after the
+// first's: unit + W of the first + w; unique because the ranges are
+// contiguous).  So a layer's reduction order is the one it has in a launch of
+// its group alone.
 constexpr int kMaxWindowGroups = 2;
 struct GroupRows {
     int32_t tile0[kMaxBatchPerLaunch];  // first tile of the row's pages that is read (window start)
@@ -275,8 +278,8 @@ struct DecodeParams {
     int32_t n_layers_run, B;
     int16_t layers[kMaxLayersPerLaunch];   // run layer lr -> cache layer
     int16_t qlayers[kMaxLayersPerLaunch];  // run layer lr -> layer index of q and out
-    int32_t n_warps;           // W
-    int64_t n_tiles;           // T
+    int32_t n_warps[kMaxWindowGroups];  // W per group
+    int64_t n_tiles;           // of both groups
     const int32_t *page_table;
     const int32_t *page_fill;
     int32_t max_pages;
@@ -285,8 +288,8 @@ struct DecodeParams {
     int32_t b0;                // first batch row of this launch
     float qscale;              // softmax scale * log2(e) (* k_scale for fp8 keys)
     float vscale;              // 1, or v_scale for fp8 values (applied by the combine)
-    float *part_o;             // [U + W][G][D]
-    float2 *part_ml;           // [U + W][G]
+    float *part_o;             // [U + W of the groups][G][D]
+    float2 *part_ml;           // [U + W of the groups][G]
     __nv_bfloat16 *out;        // [Lrun][Btot][Hq][D] (combine)
     float *state;              // split decode: fp32 [Lrun][Btot][Hq][D + 4] (o, m, l, pad); null otherwise
     int32_t state_merge;       // 1: merge into the state, 0: overwrite it
@@ -295,7 +298,26 @@ struct DecodeParams {
     int64_t tile1;             // tiles of the first group
     int32_t seq[kMaxBatchPerLaunch];
     GroupRows rows[kMaxWindowGroups];
+    __host__ __device__ __forceinline__ int64_t group_tiles(int g) const { return g ? n_tiles - tile1 : tile1; }
 };
+// A group's workers: at most w_max, and a tile for each.
+inline void set_decode_warps(DecodeParams *p, int64_t w_max) {
+    for (int g = 0; g < kMaxWindowGroups; ++g) {
+        const int64_t T = p->group_tiles(g);
+        p->n_warps[g] = (int32_t)(T < w_max ? T : w_max);
+    }
+}
+// Slots of partials that the launches of one call need with up to w_max
+// workers per group, whatever the lengths of the sequences.
+inline int64_t decode_slots(const std::vector<DecodeParams> &plan, int64_t w_max) {
+    int64_t most = 0;
+    for (const DecodeParams &p : plan) {
+        const int64_t groups = p.layer1 < p.n_layers_run ? 2 : 1;
+        const int64_t n = (int64_t)p.n_layers_run * p.B * p.n_kv_heads + groups * w_max;
+        if (n > most) most = n;
+    }
+    return most;
+}
 
 // -------------------------------------------------------------- launchers --
 // Every launcher counts the kernels it launches (kvg_launch_count()).
@@ -391,7 +413,7 @@ cudaError_t launch_sha256_serial_part(const uint8_t *seg0, uint64_t n0, const ui
 // Whether the hashing in parts is there (the two-warp forms are not turned off).
 bool sha256_parts_ok();
 
-// Persistent decode: p.n_warps one-warp CTAs over p.n_tiles tiles, then the
+// Persistent decode: p.n_warps one-warp CTAs per group, then the
 // combine over every (layer, row, query head).  decode_tile_tokens() is the
 // tile height TOK of the kernel for that element type and page size (tiles per page =
 // ceil(P / TOK); the host plan and the tensor map's box must use the same
@@ -431,7 +453,7 @@ struct CacheShape {
 bool cache_shape(const kvg_cache *c, CacheShape *out);
 int32_t cache_seq_pages(const kvg_cache *c, int32_t seq);
 kvg_status cache_plan_decode(const kvg_cache *c, int32_t layer, const int32_t *seq_ids, int32_t B, int G, int w_max,
-                             std::vector<DecodeParams> *plan, int64_t *max_units);
+                             std::vector<DecodeParams> *plan);
 // Bytes of the allocation-free decode's static scratch, and of one partial's
 // slot (G heads: fp32 o, m and l).
 constexpr uint64_t kStaticScratchBytes = 16u << 20;

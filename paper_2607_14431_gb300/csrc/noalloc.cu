@@ -94,9 +94,9 @@ extern "C" kvg_status kvg_decode_attention_noalloc(kvg_cache *c, int32_t layer, 
     if (w_max <= 0) return reject(KVG_ERR_CUDA, "decode kernel cannot be made resident");
     // the launches (as kvg_decode_attention makes them); host memory only
     std::vector<DecodeParams> plan;
-    int64_t units = 0;
-    const kvg_status pst = cache_plan_decode(c, layer, seq_ids, B, G, w_max, &plan, &units);
+    const kvg_status pst = cache_plan_decode(c, layer, seq_ids, B, G, w_max, &plan);
     if (pst != KVG_OK) return pst;
+    const int64_t units = decode_slots(plan, 0);
     // partials: (units + workers) slots of G * (4 * head_dim + 8) bytes; the
     // (m, l) part starts 256-byte aligned after o, so keep 256 bytes of slack
     const uint64_t per_slot = partial_slot_bytes(G, cs.head_dim);
@@ -120,13 +120,14 @@ extern "C" kvg_status kvg_decode_attention_noalloc(kvg_cache *c, int32_t layer, 
     }
     if (!scratch) return reject(KVG_ERR_CUDA, "static decode scratch was not set up on the cache's device");
     const int64_t w_cap = cap_slots - units < w_max ? cap_slots - units : w_max;
-    const size_t slots = (size_t)units + (size_t)w_cap;
+    // (launches of two windows fit with w_max workers for each: plan_decode)
+    const size_t slots = (size_t)decode_slots(plan, w_cap);
     float *part_o = static_cast<float *>(scratch);
     float2 *part_ml = reinterpret_cast<float2 *>(static_cast<unsigned char *>(scratch) +
                                                  ((slots * G * cs.head_dim * 4 + 255) / 256) * 256);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     for (DecodeParams &p : plan) {
-        p.n_warps = (int32_t)(p.n_tiles < w_cap ? (p.n_tiles > 1 ? p.n_tiles : 1) : w_cap);
+        set_decode_warps(&p, w_cap);
         p.n_q_heads = n_q_heads;
         p.q = static_cast<const __nv_bfloat16 *>(q);
         p.q_row_stride_b = B;

@@ -2043,14 +2043,19 @@ struct WindowGroup {
 // and that one refuses nothing that separate launches would fit), over at
 // most kMaxBatchPerLaunch rows.  Two windows in one launch share its ramp, its
 // drained end and the combine: a step of 16 fp8 sequences over 1,000 to 12,001
-// rows, every second of 4 layers windowed to 1,024, 195 us in two launches and
-// 178 in one.
+// rows, every second of 4 layers windowed to 1,024, 201 us in two launches and
+// 169 in one (other changes to the kernel in between included).  Each window's
+// tiles are split over the workers by themselves, as in a launch of their own,
+// so sharing one changes no layer's reduction order.  (One list of both
+// windows' tiles took 166 us, and 30 instead of 36 for 4 fp8 rows of 1,000 to
+// 3,000 tokens of the 12B shape, but then a layer's partials ended where the
+// other window's lengths put them, which moved its outputs by 7.5e-4.)
 // Fills every field but the per-call ones (q, out, scale, heads, scratch,
-// workers); *max_units gets the largest layers x rows x kv heads of a launch.
+// workers).
 // page_begin / page_end: only the sequence's pages [page_begin, page_end)
 // are read (a split decode over a slot range); the defaults read them all.
 static kvg_status plan_decode(const kvg_cache *c, int32_t layer, const int32_t *seq_ids, int32_t B, int G, int w_max,
-                              std::vector<DecodeParams> *plan, int64_t *max_units, int32_t page_begin = 0,
+                              std::vector<DecodeParams> *plan, int32_t page_begin = 0,
                               int32_t page_end = INT32_MAX) {
     const kvg_dims &d = c->dims;
     const int TOK = decode_tile_tokens(d.head_dim, d.kv_dtype == KVG_KV_E4M3, d.page_size);
@@ -2068,14 +2073,13 @@ static kvg_status plan_decode(const kvg_cache *c, int32_t layer, const int32_t *
         it->layers.push_back({l, layer < 0 ? l : 0});
     }
     plan->clear();
-    *max_units = 0;
     const int32_t nb_max = std::min<int32_t>(B, kMaxBatchPerLaunch);
     const int64_t slots = (int64_t)((kStaticScratchBytes - 256) / partial_slot_bytes(G, d.head_dim));
     for (size_t i0 = 0; i0 < parts.size();) {
         size_t n_parts = 1, nl = parts[i0].layers.size();
         if (i0 + 1 < parts.size()) {
             const size_t both = nl + parts[i0 + 1].layers.size();
-            if (both <= kMaxLayersPerLaunch && (int64_t)both * nb_max * d.n_kv_heads + w_max <= slots) {
+            if (both <= kMaxLayersPerLaunch && (int64_t)both * nb_max * d.n_kv_heads + 2 * w_max <= slots) {
                 n_parts = 2;
                 nl = both;
             }
@@ -2087,7 +2091,7 @@ static kvg_status plan_decode(const kvg_cache *c, int32_t layer, const int32_t *
             memset(&p, 0, sizeof p);
             for (int32_t i = 0; i < nb; ++i) p.seq[i] = seq_ids[b0 + i];
             p.n_layers_run = p.layer1 = (int32_t)nl;
-            int32_t lr = 0;
+            int64_t tiles[2] = {};
             for (size_t k = 0; k < n_parts; ++k) {
                 const WindowGroup &part = parts[i0 + k];
                 GroupRows &rows = p.rows[k];
@@ -2109,16 +2113,21 @@ static kvg_status plan_decode(const kvg_cache *c, int32_t layer, const int32_t *
                     acc += std::max(0, t1 - t0);
                 }
                 rows.pref_tiles[nb] = acc;
-                for (const auto &l : part.layers) {
+                tiles[k] = (int64_t)part.layers.size() * d.n_kv_heads * acc;
+            }
+            // the part with more tiles first: the short ranges fill in behind the long ones
+            const bool swapped = tiles[1] > tiles[0];
+            if (swapped) std::swap(p.rows[0], p.rows[1]);
+            int32_t lr = 0;
+            for (size_t k = 0; k < n_parts; ++k) {
+                for (const auto &l : parts[i0 + (swapped ? 1 - k : k)].layers) {
                     p.layers[lr] = (int16_t)l.first;
                     p.qlayers[lr++] = (int16_t)l.second;
                 }
-                p.n_tiles += (int64_t)part.layers.size() * d.n_kv_heads * acc;
-                if (k == 0) {
-                    p.layer1 = lr;
-                    p.tile1 = p.n_tiles;
-                }
+                if (k == 0) p.layer1 = lr;
             }
+            p.tile1 = tiles[swapped];
+            p.n_tiles = tiles[0] + tiles[1];
             p.B = nb;
             p.b0 = b0;
             p.pool = c->pool;
@@ -2129,7 +2138,6 @@ static kvg_status plan_decode(const kvg_cache *c, int32_t layer, const int32_t *
             p.page_fill = c->page_fill;
             p.max_pages = c->max_pages;
             p.status = c->status;
-            *max_units = std::max<int64_t>(*max_units, (int64_t)nl * nb * d.n_kv_heads);
         }
         i0 += n_parts;
     }
@@ -2172,16 +2180,15 @@ static kvg_status decode_impl(const char *what, kvg_cache *c, int32_t layer, con
     const int w_max = decode_max_warps(d.head_dim, G, fp8, d.page_size, c->n_sm);
     if (w_max <= 0) return fail(KVG_ERR_CUDA, "decode kernel cannot be made resident");
     std::vector<DecodeParams> plan;
-    int64_t max_units = 0;
-    kvg_status r = plan_decode(c, layer, seq_ids, B, G, w_max, &plan, &max_units, page_begin, page_end);
+    kvg_status r = plan_decode(c, layer, seq_ids, B, G, w_max, &plan, page_begin, page_end);
     if (r != KVG_OK) return r;
-    const size_t slots = (size_t)max_units + (size_t)w_max;
+    const size_t slots = (size_t)decode_slots(plan, w_max);
     if (!c->part_ev) KVG_CUDA(cudaEventCreateWithFlags(&c->part_ev, cudaEventDisableTiming));
     if (c->part_used && st != c->part_stream) KVG_CUDA(cudaStreamWaitEvent(st, c->part_ev, 0));
     KVG_CUDA(c->part_o.ensure(slots * G * d.head_dim * sizeof(float)));
     KVG_CUDA(c->part_ml.ensure(slots * G * sizeof(float2)));
     for (DecodeParams &p : plan) {
-        p.n_warps = (int32_t)std::min<int64_t>(w_max, std::max<int64_t>(p.n_tiles, 1));
+        set_decode_warps(&p, w_max);
         p.n_q_heads = n_q_heads;
         p.q = static_cast<const __nv_bfloat16 *>(q);
         p.q_row_stride_b = B;
@@ -2348,8 +2355,8 @@ bool cache_shape(const kvg_cache *c, CacheShape *out) {
 }
 int32_t cache_seq_pages(const kvg_cache *c, int32_t seq) { return (int32_t)c->seq_pages[seq].size(); }
 kvg_status cache_plan_decode(const kvg_cache *c, int32_t layer, const int32_t *seq_ids, int32_t B, int G, int w_max,
-                             std::vector<DecodeParams> *plan, int64_t *max_units) {
-    return plan_decode(c, layer, seq_ids, B, G, w_max, plan, max_units);
+                             std::vector<DecodeParams> *plan) {
+    return plan_decode(c, layer, seq_ids, B, G, w_max, plan);
 }
 void set_last_error(const char *msg) { g_last_error = msg; }
 }  // namespace kvg

@@ -51,3 +51,36 @@ def test_windows_of_several_sizes(windows, d, g, page):
     # only the sequences of one row and none: the windowed layers read as much as the others
     o2 = decode(kvg, c, w, [2, 0], np.ascontiguousarray(q[:, :2]))
     assert not o2[:, 0].any() and o2[:, 1].any()
+
+
+@pytest.mark.parametrize("d,g,page,fp8", [(128, 2, 64, True), (256, 2, 64, True), (128, 4, 64, False),
+                                          (64, 2, 16, False)])
+def test_sharing_a_launch_keeps_the_reduction(d, g, page, fp8):
+    """A layer gives the same bytes whether or not another window's layers run in the call."""
+    kvg = need_gpu()
+    w = syn.Workload("share", 4, 4 * g, 4, d, page, 10000.0, 0x73)
+    batch, n, window = 12, 1500, 700
+    pages = -(-n // page)
+    rows = [[to_dev(syn.as_u16(x)) for x in syn.kv_rows(w, n, 74 + i)] for i in range(batch)]
+    pos = to_dev(syn.positions(0, n).astype(np.int32))
+
+    def run(layers, windows):
+        dims = kvg.make_dims(len(layers), w.n_kv_heads, d, page, w.rope_theta, 0,
+                             kvg.KVG_KV_E4M3 if fp8 else kvg.KVG_KV_BF16, 0.0625, 0.0625)
+        c = kvg.Cache(dims, batch * pages, batch, n)
+        for i, (k, v) in enumerate(rows):
+            kk, vv = k[layers].contiguous(), v[layers].contiguous()
+            kvg.kvg_cache_append(c.h, i, kk.data_ptr(), vv.data_ptr(), pos.data_ptr(), n)
+            torch.cuda.synchronize()
+        kvg.kvg_cache_set_layer_windows(c.h, windows)
+        qd = to_dev(q[layers])
+        out = torch.empty_like(qd)
+        kvg.kvg_decode_attention(c.h, -1, list(range(batch)), qd.data_ptr(), w.n_q_heads, out.data_ptr(),
+                                 1.0 / math.sqrt(d))
+        torch.cuda.synchronize()
+        return u16(out)
+
+    q = syn.as_u16(syn.queries(w, w.n_layers, batch, 75))
+    together = run([0, 1, 2, 3], [window, 0, window, 0])
+    assert np.array_equal(together[[1, 3]], run([1, 3], [0, 0]))
+    assert np.array_equal(together[[0, 2]], run([0, 2], [window, window]))
