@@ -403,7 +403,9 @@ kvg_status kvg_graft_chunked(kvg_store *store, uint64_t block_id, kvg_cache *cac
  * re-based graft's stored pages after the copies; the report's seq is the (last)
  * failing graft's sequence and mismatch_pages its block page indices.  The
  * call stages its job table in library-owned pinned memory and waits for
- * the previous batch's table copy on this cache before reusing it. */
+ * the previous batch's table copy on this cache before reusing it; on the GPU
+ * a batch on another stream than the cache's previous one runs after it (they
+ * share the table's device memory). */
 kvg_status kvg_graft_batch(kvg_store *store, const uint64_t *block_ids, kvg_cache *cache, const int32_t *seq_ids,
                            const int64_t *deltas, int32_t n, uint32_t flags, void *stream,
                            kvg_graft_report *report);

@@ -785,12 +785,13 @@ struct kvg_cache {
     cudaStream_t aux[kHostHashStreams] = {};
     cudaEvent_t aux_ev[kHostVerifyChunks + kHostHashStreams] = {};
     // kvg_graft_batch's job table: staged in pinned host memory, copied to
-    // batch_dev on the call's stream; batch_ev marks when the copy has read it
+    // batch_dev on the call's stream; batch_ev marks when the copy has read it,
+    // batch_done when the batch's last kernel has read batch_dev
     Scratch batch_dev;
     uint32_t batch_calls = 0;  // verified batches so far: orders their mismatches in the status word
     uint8_t *batch_host = nullptr;
     size_t batch_host_cap = 0;
-    cudaEvent_t batch_ev = nullptr;
+    cudaEvent_t batch_ev = nullptr, batch_done = nullptr;
     std::vector<uint8_t> pinned;  // per page: owned by a pool-resident store block
     std::vector<int32_t> alias;   // per pinned page: sequences whose page tables point at it
     // cos/sin tables of the deltas grafts have used (cos[D/2] then sin[D/2]),
@@ -1006,6 +1007,7 @@ extern "C" void kvg_cache_destroy(kvg_cache *c) {
     for (cudaStream_t a : c->aux)
         if (a) cudaStreamDestroy(a);
     if (c->batch_ev) cudaEventDestroy(c->batch_ev);
+    if (c->batch_done) cudaEventDestroy(c->batch_done);
     if (c->part_ev) cudaEventDestroy(c->part_ev);
     if (c->batch_host) cudaFreeHost(c->batch_host);
     c->batch_dev.release();
@@ -1889,6 +1891,7 @@ extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, k
     const size_t trig_off = (meta_bytes + (size_t)pages * sizeof(GraftJob) + 15) / 16 * 16;
     const size_t bytes = trig_off + table_delta.size() * 2 * half * sizeof(float);
     if (!c->batch_ev) KVG_CUDA(cudaEventCreateWithFlags(&c->batch_ev, cudaEventDisableTiming));
+    if (!c->batch_done) KVG_CUDA(cudaEventCreateWithFlags(&c->batch_done, cudaEventDisableTiming));
     KVG_CUDA(cudaEventSynchronize(c->batch_ev));  // the previous batch's copy has read the staging
     if (bytes > c->batch_host_cap) {
         if (c->batch_host) cudaFreeHost(c->batch_host);
@@ -1938,6 +1941,13 @@ extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, k
     float *trig = reinterpret_cast<float *>(c->batch_host + trig_off);
     for (size_t t = 0; t < table_delta.size(); ++t)
         memcpy(trig + t * 2 * half, rope_table_memo(c, s->dims, table_delta[t]), (size_t)2 * half * sizeof(float));
+    // the table is one per cache: a batch on another stream may still read it
+    KVG_CUDA(cudaStreamWaitEvent(st, c->batch_done, 0));
+    struct TableRead {  // recorded whichever way the call ends
+        cudaEvent_t done;
+        cudaStream_t st;
+        ~TableRead() { cudaEventRecord(done, st); }
+    } table_read{c->batch_done, st};
     KVG_CUDA(cudaMemcpyAsync(c->batch_dev.ptr, c->batch_host, bytes, cudaMemcpyHostToDevice, st));
     KVG_CUDA(cudaEventRecord(c->batch_ev, st));
     GraftBatchParams p{};
