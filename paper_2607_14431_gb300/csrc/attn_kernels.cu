@@ -793,8 +793,7 @@ __global__ void __launch_bounds__(kCombineMaxThreads) combine_state_kernel(const
     if (threadIdx.x == 0) reinterpret_cast<float4 *>(st)[D / 4] = make_float4(M, L, 0.f, 0.f);
 }
 
-__global__ void state_finish_kernel(const float *__restrict__ state, int64_t n_rows, int D,
-                                    __nv_bfloat16 *__restrict__ out) {
+__global__ void state_finish_kernel(const float *state, int64_t n_rows, int D, __nv_bfloat16 *out) {
     after_previous();
     const int64_t n = n_rows * D;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {

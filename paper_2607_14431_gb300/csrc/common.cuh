@@ -475,6 +475,11 @@ cudaError_t noalloc_prepare_device(int device);
 // calls let_next_start() once its own end is near (never long before: what
 // waits holds an SM's resources); the launch of the next needs it from every
 // CTA, or the CTA's exit.
+// So such a kernel's lifetime overlaps the writes of the one before it: none of
+// its loads may go through the read-only path, which assumes data unchanged
+// over that lifetime (no __ldg, no const __restrict__ kernel parameter), and
+// none of its parameters is __restrict__, which would let an access move across
+// the wait.
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -112,7 +112,7 @@ struct TableTrig {
         const float4 *s4 = reinterpret_cast<const float4 *>(cs + half + i0);
 #pragma unroll
         for (int q = 0; q < N / 4; ++q) {
-            const float4 x = __ldg(c4 + q), y = __ldg(s4 + q);
+            const float4 x = c4[q], y = s4[q];
             c[4 * q] = x.x, c[4 * q + 1] = x.y, c[4 * q + 2] = x.z, c[4 * q + 3] = x.w;
             s[4 * q] = y.x, s[4 * q + 1] = y.y, s[4 * q + 2] = y.z, s[4 * q + 3] = y.w;
         }

@@ -237,8 +237,8 @@ __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uin
     uint4 n1[4], n2[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        if (nfull > 0) n1[q] = __ldg(v + q);
-        if (nfull > 1) n2[q] = __ldg(v + 4 + q);
+        if (nfull > 0) n1[q] = v[q];
+        if (nfull > 1) n2[q] = v[4 + q];
     }
     for (int blk = 0; blk < nfull; ++blk) {
         uint32_t w[16];
@@ -250,7 +250,7 @@ __device__ __forceinline__ void hash_leaf(const uint8_t *leaf, uint64_t len, uin
         }
         if (blk + 2 < nfull) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) n2[q] = __ldg(v + 4 * (blk + 2) + q);
+            for (int q = 0; q < 4; ++q) n2[q] = v[4 * (blk + 2) + q];
         }
         if (COPY) {
 #pragma unroll
@@ -539,8 +539,8 @@ __device__ __forceinline__ void split_produce_leaf(SplitShared &sm, const uint4 
     uint4 n1[4], n2[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        n1[q] = v ? __ldg(v + q) : make_uint4(0, 0, 0, 0);
-        n2[q] = v ? __ldg(v + kStep + q) : make_uint4(0, 0, 0, 0);
+        n1[q] = v ? v[q] : make_uint4(0, 0, 0, 0);
+        n2[q] = v ? v[kStep + q] : make_uint4(0, 0, 0, 0);
     }
     for (int k = 0; k < kHandOvers; ++k) {
         uint4 x[4];
@@ -551,7 +551,7 @@ __device__ __forceinline__ void split_produce_leaf(SplitShared &sm, const uint4 
         }
         if (v && k + 2 < kHandOvers) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) n2[q] = __ldg(v + kStep * (k + 2) + q);
+            for (int q = 0; q < 4; ++q) n2[q] = v[kStep * (k + 2) + q];
         }
         if (COPY && o) {
 #pragma unroll
@@ -614,7 +614,7 @@ __device__ __forceinline__ void split_whole_state(uint32_t full[8], const uint32
 // 4 KiB leaves and launches of a few such CTAs per SM.
 template <bool WIDE>
 __global__ void __launch_bounds__(64) graft_verify_split_kernel(const GraftParams p, int64_t leaves_per_page,
-                                                                uint32_t *__restrict__ out, uint32_t one) {
+                                                                uint32_t *out, uint32_t one) {
     __shared__ SplitShared sm;
     const bool produce = split_begin(sm);
     graft_metadata(p);
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(64) graft_verify_split_kernel(const GraftParam
 template <bool WIDE>
 __global__ void __launch_bounds__(64) sha256_leaves_split_kernel(const PageSource src, int64_t n_pages,
                                                                  int64_t leaves_per_page,
-                                                                 uint32_t *__restrict__ out, uint32_t one) {
+                                                                 uint32_t *out, uint32_t one) {
     __shared__ SplitShared sm;
     const bool produce = split_begin(sm);
     const int lane = threadIdx.x & 31;
@@ -676,7 +676,7 @@ __global__ void __launch_bounds__(64) sha256_leaves_split_kernel(const PageSourc
 template <bool LAT>
 __global__ void __launch_bounds__(128) sha256_leaves_kernel(const PageSource src, int64_t n_pages,
                                                             int64_t leaves_per_page,
-                                                            uint32_t *__restrict__ out, uint32_t one) {
+                                                            uint32_t *out, uint32_t one) {
     after_previous();
     const int64_t n_leaves = n_pages * leaves_per_page;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n_leaves;
@@ -719,7 +719,7 @@ __global__ void __launch_bounds__(128) sha256_leaves_kernel(const PageSource src
 // for launches of up to 64 leaves per SM (0.057 ms).
 constexpr int kGraftVerifyRing = 3;
 __global__ void __launch_bounds__(128, 5) graft_verify_ring_kernel(const GraftParams p, int64_t leaves_per_page,
-                                                                   uint32_t *__restrict__ out, uint32_t one) {
+                                                                   uint32_t *out, uint32_t one) {
     after_previous();
     constexpr int R = kGraftVerifyRing;
     extern __shared__ __align__(16) uint4 ring_mem[];
@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(128, 5) graft_verify_ring_kernel(const GraftPa
 // per 4 KiB leaf reads it from the block once, writes it to its cache page and
 // hashes it (leaf order of a page digest, Sec. 3.2's integrity check).
 __global__ void __launch_bounds__(128) graft_verify_kernel(const GraftParams p, int64_t leaves_per_page,
-                                                           uint32_t *__restrict__ out, uint32_t one) {
+                                                           uint32_t *out, uint32_t one) {
     after_previous();
     graft_metadata(p);
     const uint64_t page_bytes = p.page_bytes;
@@ -806,7 +806,7 @@ __device__ __forceinline__ BatchLeaf batch_leaf(const GraftBatchParams &p, int64
 // graft_verify_ring_kernel for a batch (the same launch sizes).
 __global__ void __launch_bounds__(128, 5) graft_batch_verify_ring_kernel(const GraftBatchParams p,
                                                                          int64_t leaves_per_page,
-                                                                         uint32_t *__restrict__ out, uint32_t one) {
+                                                                         uint32_t *out, uint32_t one) {
     after_previous();
     constexpr int R = kGraftVerifyRing;
     extern __shared__ __align__(16) uint4 ring_mem[];
@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(128, 5) graft_batch_verify_ring_kernel(const G
 // graft_verify_kernel for a batch.
 template <bool COPY>
 __global__ void __launch_bounds__(128) graft_batch_verify_kernel(const GraftBatchParams p, int64_t leaves_per_page,
-                                                                 uint32_t *__restrict__ out, uint32_t one) {
+                                                                 uint32_t *out, uint32_t one) {
     after_previous();
     if (p.write_meta) batch_metadata(p);
     const int64_t n_leaves = p.slice_jobs * p.n_layers * 2 * leaves_per_page;
@@ -845,7 +845,7 @@ __global__ void __launch_bounds__(128) graft_batch_verify_kernel(const GraftBatc
 template <bool COPY, bool WIDE>
 __global__ void __launch_bounds__(64) graft_batch_verify_split_kernel(const GraftBatchParams p,
                                                                       int64_t leaves_per_page,
-                                                                      uint32_t *__restrict__ out, uint32_t one) {
+                                                                      uint32_t *out, uint32_t one) {
     __shared__ SplitShared sm;
     const bool produce = split_begin(sm);
     if (p.write_meta) batch_metadata(p);
@@ -864,7 +864,7 @@ __global__ void __launch_bounds__(64) graft_batch_verify_split_kernel(const Graf
 
 // Whether the digest with state words st (written big-endian) differs from
 // the 32 bytes at expected.
-__device__ __forceinline__ bool digest_differs(const uint32_t st[8], const uint8_t *__restrict__ expected) {
+__device__ __forceinline__ bool digest_differs(const uint32_t st[8], const uint8_t *expected) {
     bool same = true;
 #pragma unroll
     for (int k = 0; k < 32; ++k) same &= (uint8_t)(st[k >> 2] >> (24 - 8 * (k & 3))) == expected[k];
@@ -920,7 +920,7 @@ struct BatchCheck {
 // Page digest from its leaf digests: the message is the leaf digests' bytes,
 // i.e. (big-endian) exactly the 8 state words of each leaf in order.
 template <class Verdict>
-__global__ void __launch_bounds__(128) sha256_pages_kernel(const uint32_t *__restrict__ leaf_words,
+__global__ void __launch_bounds__(128) sha256_pages_kernel(const uint32_t *leaf_words,
                                                            int64_t n_pages, int64_t m, const Verdict verdict,
                                                            uint32_t one) {
     after_previous();
@@ -962,7 +962,7 @@ __global__ void __launch_bounds__(128) sha256_pages_kernel(const uint32_t *__res
 // sha256_pages_kernel in the two-warp form: the loading warp feeds each page's
 // leaf digests (already big-endian words) and the final block.
 template <class Verdict>
-__global__ void __launch_bounds__(64) sha256_pages_split_kernel(const uint32_t *__restrict__ leaf_words,
+__global__ void __launch_bounds__(64) sha256_pages_split_kernel(const uint32_t *leaf_words,
                                                                 int64_t n_pages, int64_t m, const Verdict verdict,
                                                                 uint32_t one) {
     __shared__ SplitShared sm;
