@@ -126,7 +126,8 @@ struct TableTrig {
 template <int ROT, class Trig>
 __device__ __forceinline__ void rotate_chunk(uint8_t *__restrict__ dst, const uint8_t *__restrict__ src,
                                              int bytes, int64_t first_row_in_page, int64_t page_token0,
-                                             int head_dim, int page_size, int64_t n_tokens, const Trig &trig) {
+                                             int head_dim, int page_size, int64_t n_tokens, const Trig &trig,
+                                             int tid = threadIdx.x, int threads = kCopyThreads) {
     const int D = head_dim;
     const int vec_per_row = D >> 3;
     const int rows = bytes / (2 * D);
@@ -144,11 +145,11 @@ __device__ __forceinline__ void rotate_chunk(uint8_t *__restrict__ dst, const ui
         const int half_vecs = vec_per_row >> 1;  // D/16: a power of two
         const int hv_shift = __ffs(half_vecs) - 1;
         const int n_items = rows * half_vecs;
-        for (int base = threadIdx.x; base < n_items; base += kCopyThreads * kRotUnroll) {
+        for (int base = tid; base < n_items; base += threads * kRotUnroll) {
             uint4 lo[kRotUnroll], hi[kRotUnroll];
 #pragma unroll
             for (int u = 0; u < kRotUnroll; ++u) {
-                const int it = base + u * kCopyThreads;
+                const int it = base + u * threads;
                 if (it < n_items) {
                     const int rr = it >> hv_shift;
                     const int lo_i = rr * vec_per_row + (it & (half_vecs - 1));
@@ -158,7 +159,7 @@ __device__ __forceinline__ void rotate_chunk(uint8_t *__restrict__ dst, const ui
             }
 #pragma unroll
             for (int u = 0; u < kRotUnroll; ++u) {
-                const int it = base + u * kCopyThreads;
+                const int it = base + u * threads;
                 if (it < n_items) {
                     const int rr = it >> hv_shift;
                     const int c = it & (half_vecs - 1);
@@ -182,7 +183,7 @@ __device__ __forceinline__ void rotate_chunk(uint8_t *__restrict__ dst, const ui
     } else {
         const int vr_shift = __ffs(vec_per_row) - 1;  // D/8: a power of two
         const int n_items = rows * vec_per_row;
-        for (int it = threadIdx.x; it < n_items; it += kCopyThreads) {
+        for (int it = tid; it < n_items; it += threads) {
             const int rr = it >> vr_shift;
             const int c = it & (vec_per_row - 1);
             const uint4 x = __ldcs(s4 + it);
@@ -874,7 +875,8 @@ int grid_for(int64_t work_items, int per_block, int n_sm, int waves) {
 // SM busy to its end instead of draining after each graft.  ROT > 0: some
 // grafts are re-based (their key chunks rotate with their own cos/sin table,
 // as the single-graft kernels do; values and own-position grafts copy).
-// MANY: small pages, several jobs of a plane per unit.
+// MANY: small pages, several jobs of a plane per unit; re-based key pages are
+// left to graft_batch_rotate_kernel (ROT: there are some).
 template <int ROT, bool MANY>
 __global__ void __launch_bounds__(kCopyThreads) graft_batch_kernel(const GraftBatchParams p) {
     after_previous();
@@ -888,23 +890,26 @@ __global__ void __launch_bounds__(kCopyThreads) graft_batch_kernel(const GraftBa
         for (int64_t unit = blockIdx.x; unit < (int64_t)p.n_layers * 2 * gpp; unit += gridDim.x) {
             const int64_t lkv = unit / gpp, j0 = (unit - lkv * gpp) * q;
             const int n = (int)(q < p.n_jobs - j0 ? q : p.n_jobs - j0);
-            auto src = [&](int j) {
-                const GraftJob &job = p.jobs[j0 + j];
-                return job.src + (uint64_t)lkv * job.block_pages * page_bytes;
+            auto copy = [&](int64_t jf, int pages) {
+                copy_pages(
+                    pages, (int)(page_bytes >> 4),
+                    [&](int j) {
+                        const GraftJob &job = p.jobs[jf + j];
+                        return job.src + (uint64_t)lkv * job.block_pages * page_bytes;
+                    },
+                    [&](int j) {
+                        return p.pool + ((uint64_t)lkv * p.pool_pages + (uint64_t)p.jobs[jf + j].pid) * page_bytes;
+                    });
             };
-            auto dst = [&](int j) {
-                return p.pool + ((uint64_t)lkv * p.pool_pages + (uint64_t)p.jobs[j0 + j].pid) * page_bytes;
-            };
-            if (!p.rotated_only) copy_pages(n, (int)(page_bytes >> 4), src, dst);
-            if (ROT == 0 || (lkv & 1)) continue;
-            __syncthreads();  // the copies of re-based pages, before they are written again
-            for (int j = 0; j < n; ++j) {
-                const GraftJob job = p.jobs[j0 + j];
-                const GraftMeta &m = p.metas[job.meta];
-                if (m.trig < 0) continue;
-                const int half = p.head_dim >> 1;
-                rotate_chunk<ROT>(dst(j), src(j), (int)page_bytes, 0, (int64_t)job.page * p.page_size, p.head_dim,
-                                  p.page_size, m.n_tokens, TableTrig{p.trig + (int64_t)m.trig * 2 * half, half});
+            if constexpr (ROT == 0) {
+                copy(j0, n);
+            } else {
+                for (int first = 0, end; first < n; first = end + 1) {  // runs of pages to copy
+                    end = n;
+                    if (!(lkv & 1))
+                        for (end = first; end < n && p.metas[p.jobs[j0 + end].meta].trig < 0;) ++end;
+                    copy(j0 + first, end - first);
+                }
             }
         }
     }
@@ -930,16 +935,52 @@ __global__ void __launch_bounds__(kCopyThreads) graft_batch_kernel(const GraftBa
     if (p.write_meta) batch_metadata(p);
 }
 
+// The re-based key pages of a batch of small pages: a unit's pages side by
+// side, each by as many threads as its rows keep busy.  A kernel of its own:
+// in graft_batch_kernel the rotation took twice the registers that the copies
+// need, so one CTA fitted an SM.  8 re-based grafts of 8,192 tokens of 16 layers
+// of the tiny shape (4 KiB pages, 537 MB) take 244 us from HBM and 2.14 ms from
+// pinned host memory (own positions: 161 us, 2.13 ms); with every page copied
+// first and the keys rotated over them 484 us and 3.79 ms, 8 of 4,096 tokens
+// with 16 KiB pages 543 us and 6.91 ms against 343 us and 4.54 ms now.
+template <int ROT>
+__global__ void __launch_bounds__(kCopyThreads) graft_batch_rotate_kernel(const GraftBatchParams p) {
+    after_previous();
+    const uint64_t page_bytes = p.page_bytes;
+    const int items = (int)(page_bytes >> (ROT == 1 ? 5 : 4)) / (ROT == 1 ? kRotUnroll : 1);
+    const int threads = min((items + 31) & ~31, kCopyThreads), side = kCopyThreads / threads;
+    if ((int)threadIdx.x >= side * threads) return;
+    const int half = p.head_dim >> 1;
+    const int64_t q = p.unit_pages, gpp = (p.n_jobs + q - 1) / q;
+    for (int64_t unit = blockIdx.x; unit < (int64_t)p.n_layers * gpp; unit += gridDim.x) {
+        const int64_t l = unit / gpp, j0 = (unit - l * gpp) * q;
+        const int n = (int)(q < p.n_jobs - j0 ? q : p.n_jobs - j0);
+        for (int j = threadIdx.x / threads; j < n; j += side) {
+            const GraftJob job = p.jobs[j0 + j];
+            const GraftMeta &m = p.metas[job.meta];
+            if (m.trig < 0) continue;
+            rotate_chunk<ROT>(p.pool + ((uint64_t)l * 2 * p.pool_pages + (uint64_t)job.pid) * page_bytes,
+                              job.src + (uint64_t)l * 2 * job.block_pages * page_bytes, (int)page_bytes, 0,
+                              (int64_t)job.page * p.page_size, p.head_dim, p.page_size, m.n_tokens,
+                              TableTrig{p.trig + (int64_t)m.trig * 2 * half, half}, threadIdx.x % threads, threads);
+        }
+    }
+}
+
 cudaError_t launch_graft_batch(const GraftBatchParams &p, int n_sm, cudaStream_t s, int max_ctas, int rotate) {
     const int64_t units = (p.n_jobs + p.unit_pages - 1) / p.unit_pages * p.n_layers * 2 *
                           (int64_t)(p.page_bytes / p.chunk_bytes);
     int grid = grid_for(units, 1, n_sm, 4);
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
-    if (p.unit_pages > 1)
-        return launch_after(rotate == 0   ? graft_batch_kernel<0, true>
-                            : rotate == 1 ? graft_batch_kernel<1, true>
-                                          : graft_batch_kernel<2, true>,
-                            grid, kCopyThreads, 0, s, p);
+    if (p.unit_pages > 1) {
+        cudaError_t e = cudaSuccess;
+        if (!p.rotated_only)
+            e = launch_after(rotate == 0 ? graft_batch_kernel<0, true> : graft_batch_kernel<1, true>, grid, kCopyThreads,
+                             0, s, p);
+        if (e != cudaSuccess || rotate == 0) return e;
+        return launch_after(rotate == 1 ? graft_batch_rotate_kernel<1> : graft_batch_rotate_kernel<2>, grid,
+                            kCopyThreads, 0, s, p);
+    }
     return launch_after(rotate == 0   ? graft_batch_kernel<0, false>
                         : rotate == 1 ? graft_batch_kernel<1, false>
                                       : graft_batch_kernel<2, false>,

@@ -66,3 +66,43 @@ def test_units_of_several_pages(pages, ragged, style, residency):
         else:
             assert np.array_equal(got, single)
         kvg.kvg_sync(c.h)
+
+
+@pytest.mark.parametrize("verify", [0, 1])
+@pytest.mark.parametrize("style", [0, 1])
+@pytest.mark.parametrize("residency", [0, 1])
+def test_batch_of_own_and_rebased_pages_in_turn(verify, style, residency):
+    """Units of a batch that hold runs of own-position and of re-based pages, against a graft at a time."""
+    kvg = need_gpu()
+    w = syn.Workload("runs", 16, 2, 2, 64, 16, 10000.0, 0x91)
+    lens = [3 * 16, 18 * 16 - 5, 7, 40 * 16, 16, 29 * 16 - 1]
+    deltas = [0, 9, 0, 4097, 9, 0]
+    dims = dims_for(kvg, w, style)
+    src = kvg.Cache(dims, 40, 1, 640)
+    store = kvg.Store(dims, residency, 1 << 30)
+    bids = []
+    for i, n in enumerate(lens):
+        k, v = (syn.as_u16(x) for x in syn.kv_rows(w, n, 94 + i))
+        append(kvg, src, 0, k, v, syn.positions(0, n))
+        bids.append(kvg.kvg_deposit(store.h, src.h, 0, 0, n))
+        kvg.kvg_cache_release(src.h, 0)
+    torch.cuda.synchronize()
+    times = 6  # 558 pages in 2 x 16 planes: sixteen to a unit
+    pages = times * sum(-(-n // 16) for n in lens)
+    seqs = [i // len(lens) for i in range(times * len(lens))]
+    flags = kvg.KVG_GRAFT_VERIFY if verify else 0
+    got = []
+    for how in ("batch", "single"):
+        c = kvg.Cache(dims, pages + 3, times, pages * 16)
+        fill_canary(c)
+        kvg.kvg_cache_set_free_order(c.h, syn.permutation(pages + 3, 95))
+        if how == "batch":
+            kvg.kvg_graft_batch(store.h, bids * times, c.h, seqs, flags, deltas=deltas * times)
+        else:
+            for b, s, d in zip(bids * times, seqs, deltas * times):
+                kvg.kvg_graft(store.h, b, c.h, s, -1, d, flags)
+        torch.cuda.synchronize()
+        kvg.kvg_sync(c.h)
+        got.append((pool_u16(c, w), *tables(c)))
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
