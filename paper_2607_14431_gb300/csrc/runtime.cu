@@ -1279,7 +1279,8 @@ static kvg_status pool_deposit(kvg_store *s, kvg_cache *c, int32_t seq, int32_t 
     return KVG_OK;
 }
 
-constexpr int kChainSms = 8;  // SMs a long deposit's leaf hashes leave free
+constexpr int kChainSms = 8;       // SMs a long deposit's leaf hashes leave free
+constexpr int kPartsLeaves = 256;  // leaves of a page up to which a deposit is hashed in parts
 
 extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq, int32_t slot0, int32_t n,
                                   void *stream, uint64_t *block_id_out) {
@@ -1351,13 +1352,23 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
     // pages: while one chunk's leaves are hashed on the caller's stream, the
     // page digests of the one before follow on the store's page stream and
     // the chain over those on its digest stream (its state waits in the
-    // header's digest field between chunks).  The chain is what the whole waits
-    // for, so the leaf hashes leave it alone: one CTA (a warp per scheduler) on
-    // all but kChainSms of the SMs, which still hashes 1.2 times what the chain
-    // takes in, and the page digests and the chain have the others to themselves
-    // (beside a leaf CTA a page chunk's digests took 92 us instead of 35, and a
-    // block of the chain 0.88 instead of 0.80).  A chunk is one round of those
-    // CTAs; later ones grow, since the hashing runs ahead.  The call waits for
+    // header's digest field between chunks).  The leaf hashes leave the page
+    // digests and the chain alone: one CTA (a warp per scheduler) on all but
+    // kChainSms of the SMs, and the others to those two (beside a leaf CTA a page
+    // chunk's digests took 92 us instead of 35, and a block of the chain 0.88
+    // instead of 0.80).  A chunk is one round of those CTAs; later ones grow.
+    // Up to 64 leaves a page the chain is what the whole waits for (it takes two
+    // digests a block, the leaf CTAs hash 1.2 times that); with larger pages the
+    // leaves are, and from kPartsLeaves on the page digests, one serial chain of
+    // leaves / 2 blocks in each chunk.  Deposits of the 12B shape (48 layers) in
+    // parts, in parts with four leaf CTAs per SM, and one after the other, us:
+    //   rows x leaves a page   2,048 x 64   2,048 x 128   2,048 x 256   2,048 x 512
+    //                          1,895        1,616         1,579         2,030
+    //                          2,444        1,907         1,578         1,826
+    //                          2,593        2,022         1,775         1,735
+    // and 499 rows of 64, 128 and 256 leaves a page 583, 494 and 585 in parts,
+    // 728, 614 and 607 otherwise; 640 of 320 leaves a page 716 against 686,
+    // 4,096 of 1,024 (24 layers) 3,439 against 1,958.  The call waits for
     // the rows (it reads the position tags back, which bound later
     // relocations) but not for the digests, and everything that reads a block
     // digest (block info, export, save) synchronizes the device first.
@@ -1371,7 +1382,7 @@ extern "C" kvg_status kvg_deposit(kvg_store *s, const kvg_cache *cc, int32_t seq
     uint32_t *leaf = static_cast<uint32_t *>(s->leaf.ptr);
     const int leaf_ctas = std::max(1, s->n_sm - kChainSms);
     const int64_t wave = std::max<int64_t>(1, (int64_t)leaf_ctas * kLeafCtaThreads / m);
-    const bool parts = sha256_parts_ok() && n_pages > wave + wave / 4 &&
+    const bool parts = sha256_parts_ok() && m <= kPartsLeaves && n_pages > wave + wave / 4 &&
                        serial_blocks(pos_bytes + (uint64_t)n_pages * 32) < (1ll << 30);
     std::vector<int32_t> pos(n);
     cudaStream_t rows = st;  // the stream the position tags are read back on
