@@ -757,6 +757,7 @@ constexpr int kHostVerifyChunks = 16;  // page-range chunks of a verified host-s
 // longer than the next chunk's copy: on one stream the hashes fell behind and
 // ended 0.3 ms after the block had landed.
 constexpr int kHostHashStreams = 2;
+constexpr int kChunkSplitLeavesPerSm = 16;  // of a chunked call's chunk, up to which its hash takes two warps
 constexpr int32_t kMaxGraftsPerBatch = 4096;
 
 struct kvg_cache {
@@ -1781,10 +1782,15 @@ static kvg_status graft_impl(kvg_store *s, uint64_t block_id, kvg_cache *c, int3
                            (int64_t)c->n_pages};
             src.out_plane_stride = npb;
             src.out_j0 = (int32_t)base;
-            // in the one-warp form, which needs no shared memory: the append's and
-            // the decode's CTAs leave room for little of it on an SM
-            KVG_CUDA(launch_sha256_leaves(src, (int64_t)c->dims.n_layers * 2 * p.npb,
-                                          static_cast<uint32_t *>(c->leaf.ptr), c->n_sm, aux, false));
+            // A chunked call runs beside an append and decodes, whose CTAs leave little
+            // shared memory on an SM: its larger chunks take the one-warp form, which
+            // needs none (20 leaves per SM 1,329 us against 1,387, 40 2,113 against 2,193;
+            // 12B shape, 1,024 tokens restored beside 4,096).  Up to one two-warp CTA per
+            // SM that form's shorter chains win (7 leaves per SM 689 us against 933, 31B shape, 13
+            // to 20 991 against 1,063; two pages of the tiny shape 140 against 185).
+            const int64_t pages = (int64_t)c->dims.n_layers * 2 * p.npb;
+            const bool split_ok = !ce.events || pages * m <= (int64_t)c->n_sm * kChunkSplitLeavesPerSm;
+            KVG_CUDA(launch_sha256_leaves(src, pages, static_cast<uint32_t *>(c->leaf.ptr), c->n_sm, aux, split_ok));
         }
     }
     if (piped) {
