@@ -483,9 +483,10 @@ cudaError_t noalloc_prepare_device(int device);
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// early = false: launched when the kernel before it has ended.
 template <typename... Params, typename... Args>
-inline cudaError_t launch_after(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t s,
-                                Args &&...args) {
+inline cudaError_t launch_kernel(bool early, void (*kernel)(Params...), dim3 grid, int threads, size_t smem,
+                                 cudaStream_t s, Args &&...args) {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -495,10 +496,15 @@ inline cudaError_t launch_after(void (*kernel)(Params...), dim3 grid, int thread
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
     count_launches(1);
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+template <typename... Params, typename... Args>
+inline cudaError_t launch_after(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                                Args &&...args) {
+    return launch_kernel(true, kernel, grid, threads, smem, s, std::forward<Args>(args)...);
 }
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {

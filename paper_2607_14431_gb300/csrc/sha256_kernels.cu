@@ -1274,6 +1274,16 @@ static bool lat_order(int64_t n, int n_sm) {
     return n <= (int64_t)n_sm * per_sm;
 }
 
+// Whether a leaf launch may start while the kernel before it still holds SMs.
+// Not where it has a CTA for more than every fourth SM and at most four for
+// each: its CTAs are then placed around the other's (the page digests of the
+// call before), some SMs get one more than their share, and the chains there are
+// what the launch waits for.  Digests of 64 KiB pages back to back, us a call, 48,
+// 64, 128, 220 and 512 leaves per SM: 65, 109, 156, 240 and 386 started early, 68,
+// 68, 98, 173 and 325 not; of 4 KiB pages with 48 leaves per SM 103 and 62.  A few
+// CTAs gain the 3 us of the launch (20 leaves per SM: 63 against 66).
+static bool leaves_early(int64_t grid, int n_sm) { return grid * 4 <= n_sm || grid > (int64_t)n_sm * 4; }
+
 static int current_sm_count() {
     static int cache[64] = {};
     int dev = 0;
@@ -1295,7 +1305,8 @@ cudaError_t launch_sha256_leaves(const PageSource &src, int64_t n_pages, uint32_
     if (split_ok && !split_off() && src.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
         const bool wide = split_wide(n, n_sm);
         auto *kernel = wide ? sha256_leaves_split_kernel<true> : sha256_leaves_split_kernel<false>;
-        return launch_after(kernel, split_grid(n, wide), 64, 0, s, src, n_pages, m, leaf_words, 1u);
+        const int grid = split_grid(n, wide);
+        return launch_kernel(leaves_early(grid, n_sm), kernel, grid, 64, 0, s, src, n_pages, m, leaf_words, 1u);
     }
     int64_t grid = (n + 127) / 128;
     // One CTA per 128 leaves (no grid-stride cap by default): 4 CTAs of
@@ -1305,7 +1316,7 @@ cudaError_t launch_sha256_leaves(const PageSource &src, int64_t n_pages, uint32_
     if (ctas_per_sm > 0 && grid > (int64_t)n_sm * ctas_per_sm) grid = (int64_t)n_sm * ctas_per_sm;
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
     auto *kernel = lat_order(n, n_sm) ? sha256_leaves_kernel<true> : sha256_leaves_kernel<false>;
-    return launch_after(kernel, (int)grid, 128, 0, s, src, n_pages, m, leaf_words, 1u);
+    return launch_kernel(leaves_early(grid, n_sm), kernel, (int)grid, 128, 0, s, src, n_pages, m, leaf_words, 1u);
 }
 
 cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int n_sm, cudaStream_t s, bool ring_ok,
@@ -1316,7 +1327,8 @@ cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int 
     if (split_ok && !split_off() && p.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
         const bool wide = split_wide(n, n_sm);
         auto *kernel = wide ? graft_verify_split_kernel<true> : graft_verify_split_kernel<false>;
-        return launch_after(kernel, split_grid(n, wide), 64, 0, s, p, m, leaf_words, 1u);
+        const int grid = split_grid(n, wide);
+        return launch_kernel(leaves_early(grid, n_sm), kernel, grid, 64, 0, s, p, m, leaf_words, 1u);
     }
     int64_t grid = (n + 127) / 128;
     // One CTA per 128 leaves (no grid-stride cap by default): four CTAs of
@@ -1332,7 +1344,7 @@ cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int 
         const size_t smem = (size_t)128 * kGraftVerifyRing * 64;  // 24 KiB of ring slots per CTA
         return launch_after(graft_verify_ring_kernel, (int)grid, 128, smem, s, p, m, leaf_words, 1u);
     }
-    return launch_after(graft_verify_kernel, (int)grid, 128, 0, s, p, m, leaf_words, 1u);
+    return launch_kernel(leaves_early(grid, n_sm), graft_verify_kernel, (int)grid, 128, 0, s, p, m, leaf_words, 1u);
 }
 
 cudaError_t launch_graft_batch_verify(const GraftBatchParams &p, uint32_t *leaf_words, int n_sm, cudaStream_t s,
