@@ -369,7 +369,7 @@ cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int 
 // (hash_only: hashes alone), leaf_words[(plane * slice_jobs + job - job0) *
 // leaves_per_page + leaf]; then the page digests, compared with each block's.
 cudaError_t launch_graft_batch_verify(const GraftBatchParams &p, uint32_t *leaf_words, int n_sm, cudaStream_t s,
-                                      bool ring_ok, bool split_ok);
+                                      bool ring_ok);
 cudaError_t launch_graft_batch_pages(const GraftBatchParams &p, const uint32_t *leaf_words, DevStatus *status,
                                      uint32_t call, cudaStream_t s);
 cudaError_t launch_append(const AppendParams &p, int n_sm, cudaStream_t s);

@@ -2001,9 +2001,8 @@ extern "C" kvg_status kvg_graft_batch(kvg_store *s, const uint64_t *block_ids, k
         p.hash_only = host_src;
         for (p.job0 = 0; p.job0 < pages; p.job0 += slice) {
             p.slice_jobs = std::min(slice, pages - p.job0);
-            // the two-warp form's loads are too slow for host memory (re-based grafts hash the store)
             KVG_CUDA(launch_graft_batch_verify(p, static_cast<uint32_t *>(c->leaf.ptr), c->n_sm, st,
-                                               c->dims.kv_dtype == KVG_KV_BF16, !(host_src && rotate)));
+                                               c->dims.kv_dtype == KVG_KV_BF16));
             KVG_CUDA(launch_graft_batch_pages(p, static_cast<const uint32_t *>(c->leaf.ptr), c->status, call, st));
             p.write_meta = 0;
         }

@@ -1348,13 +1348,16 @@ cudaError_t launch_graft_verify(const GraftParams &p, uint32_t *leaf_words, int 
 }
 
 cudaError_t launch_graft_batch_verify(const GraftBatchParams &p, uint32_t *leaf_words, int n_sm, cudaStream_t s,
-                                      bool ring_ok, bool split_ok) {
+                                      bool ring_ok) {
     const int64_t m = (int64_t)((p.page_bytes + kLeafBytes - 1) / kLeafBytes);
     const int64_t n = p.slice_jobs * p.n_layers * 2 * m;
     if (n == 0) return cudaSuccess;
     const int grid = (int)((n + 127) / 128);
-    // the forms and their launch sizes are those of launch_graft_verify
-    if (split_ok && !split_off() && p.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
+    // The forms and their launch sizes are those of launch_graft_verify, the two-warp
+    // form also where re-based pages are hashed in pinned host memory: one graft of
+    // 40 tokens of 2 layers of the tiny shape 94 us (one warp 187), 4 of 200 tokens of
+    // the 12B shape, 27 leaves per SM, 244 (293).
+    if (!split_off() && p.page_bytes % kLeafBytes == 0 && n <= (int64_t)n_sm * split_leaves_per_sm()) {
         const bool wide = split_wide(n, n_sm);
         auto *kernel = p.hash_only ? (wide ? graft_batch_verify_split_kernel<false, true>
                                            : graft_batch_verify_split_kernel<false, false>)
