@@ -1,16 +1,30 @@
 """Copies that take several small pages at a time (graft, re-based graft, batch,
 deposit): page counts that fill units, leave a short last unit and a ragged
-last page, from HBM and pinned host memory, against grafts that take one page
-at a time (the batch of one-page units of a small block) and the oracle."""
+last page, and ones that take a page at a time, from HBM and pinned host
+memory, against the oracle; re-based keys within the rounding of the rotation."""
 import numpy as np
 import pytest
 import torch
 
 import kvg_synth as syn
 import oracle as orc
-from kvg_testlib import CANARY, append, dims_for, fill_canary, need_gpu, oracle_dims, pool_u16, tables
+from kvg_testlib import (CANARY, append, check_rotation_rounding, dims_for, fill_canary, need_gpu, oracle_dims, pool_u16,
+                         tables)
 
 pytestmark = pytest.mark.gpu
+
+
+def rotated(k, delta, theta, style):
+    """Key rows [..., D] (bf16 bits) moved by delta positions, in fp64 (style 0: pairs i, i + D/2; 1: 2i, 2i + 1)."""
+    x = orc.bf16_to_f64(k)
+    d = x.shape[-1]
+    angle = delta * theta ** (-2.0 * np.arange(d // 2) / d)
+    at = (slice(0, d // 2), slice(d // 2, d)) if style == 0 else (slice(0, d, 2), slice(1, d, 2))
+    a, b = x[..., at[0]], x[..., at[1]]
+    out = np.empty_like(x)
+    out[..., at[0]] = a * np.cos(angle) - b * np.sin(angle)
+    out[..., at[1]] = a * np.sin(angle) + b * np.cos(angle)
+    return out
 
 
 # 4 KiB pages in 2 x 16 planes: from 4 x 152 pages a unit has two, from 16 x 4 x 152 sixteen
@@ -32,6 +46,8 @@ def test_units_of_several_pages(pages, ragged, style, residency):
     bid = kvg.kvg_deposit(store.h, src.h, 0, 0, n)
     blk = orc.block_from_kv(od, k, v, pos)
     assert kvg.kvg_store_export(store.h, bid) == blk.serialize()
+    k64 = rotated(k, 4097, w.rope_theta, style)
+    assert np.allclose(k64[0, 0], orc.rope_rotate_rows(k[0, 0], 4097, w.rope_theta, style), rtol=0, atol=1e-11)
     # own position; re-based; a batch of both
     cp = 2 * pages + 5
     slots = 2 * pages * 16
@@ -57,10 +73,11 @@ def test_units_of_several_pages(pages, ragged, style, residency):
         keys = np.zeros(cp, bool)
         keys[moved] = True
         assert np.array_equal(got[:, 1], want[:, 1]) and np.array_equal(got[:, 0, ~keys], want[:, 0, ~keys])
-        # re-based keys: within the fp32 rotation's rounding of the fp64 one (the
-        # last bf16 bit), padding rows untouched
-        a, b = got[:, 0, keys].astype(np.int32), want[:, 0, keys].astype(np.int32)
-        assert (a != b).mean() < 1e-3
+        # re-based keys: every valid row within the fp32 rotation's rounding of the
+        # fp64 one, padding rows untouched
+        logical = [np.swapaxes(x[:, 0, moved], 2, 3).reshape(w.n_layers, pages * 16, 2, 64) for x in (got, want)]
+        check_rotation_rounding(orc, logical[0][:, :n], k64)
+        assert np.array_equal(logical[0][:, n:], logical[1][:, n:])
         if how == "graft":
             single = got
         else:
