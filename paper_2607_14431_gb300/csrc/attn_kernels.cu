@@ -643,10 +643,10 @@ __device__ __forceinline__ int64_t warp_of(int64_t t, int64_t T, int64_t W) { re
 // every warp's range holds a tile and every partial in [wa, wb] was written.
 // One layer of the 12B shape over 32,768 rows (76 partials per head): 48 us
 // with one thread per output column walking the partials and two 64-bit
-// divisions per partial; now the whole call takes 53.5 us instead of 98.6
-// (42 us of it the decode kernel), and one layer of the 31B shape over 2,111
-// rows 14.3 us instead of 30.7.
-// Where heads x rows x layers leave most SMs idle, each head's columns are
+// divisions per partial, so that the whole call took 98.6; this way it took
+// 53.5, and one layer of the 31B shape over 2,111 rows 14.3 instead of 30.7
+// (46.6 and 7.8 with what follows and dependent launches).
+// Where heads x rows x layers are fewer than the SMs, each head's columns are
 // shared by D / COLS blocks (COLS = 64): a block's groups are then 16 lanes, so
 // four times as many partials are in flight (one layer of the 12B shape over
 // 32,768 rows 49.1 -> 47.4 us, of the 31B shape over 2,111 rows 8.15 -> 7.84).
@@ -655,7 +655,6 @@ struct Merged {
     float M, L;  // maximum, sum of l_w 2^(m_w - M)
 };
 constexpr int kCombineMaxThreads = 512;
-constexpr int kNarrowBlocks = 152;  // up to this many (layer, row, head)s: a block per 64 columns
 
 template <int D, int COLS>
 __device__ __forceinline__ Merged merge_partials(const DecodeParams &p, int h, int col0, int b, int lr) {
@@ -951,9 +950,8 @@ static int combine_threads(int cols, const DecodeParams &p) {
     return threads;
 }
 
-cudaError_t launch_combine(int head_dim, int group, const DecodeParams &p, cudaStream_t s) {
-    (void)group;
-    const bool narrow = !p.state && (int64_t)p.n_q_heads * p.B * p.n_layers_run <= kNarrowBlocks;
+cudaError_t launch_combine(int head_dim, const DecodeParams &p, int n_sm, cudaStream_t s) {
+    const bool narrow = !p.state && (int64_t)p.n_q_heads * p.B * p.n_layers_run <= n_sm;
     const int cols = narrow ? 64 : head_dim;
     const dim3 grid(p.n_q_heads * (head_dim / cols), p.B, p.n_layers_run);
     const int n = combine_threads(cols, p);

@@ -433,7 +433,7 @@ cudaError_t make_pool_tensor_map(CUtensorMap *out, void *pool, int head_dim, boo
 // innermost first, byte strides of dims 1.., box extents per dim.
 cudaError_t encode_tensor_map(CUtensorMap *out, int rank, void *base, const cuuint64_t *dims,
                               const cuuint64_t *strides, const cuuint32_t *box);
-cudaError_t launch_combine(int head_dim, int group, const DecodeParams &p, cudaStream_t s);
+cudaError_t launch_combine(int head_dim, const DecodeParams &p, int n_sm, cudaStream_t s);
 bool decode_supported(int head_dim, int group, bool fp8 = false);
 int decode_tile_tokens(int head_dim, bool fp8, int page_size);
 int decode_max_warps(int head_dim, int group, bool fp8, int page_size, int n_sm);

@@ -138,7 +138,7 @@ extern "C" kvg_status kvg_decode_attention_noalloc(kvg_cache *c, int32_t layer, 
         p.out = static_cast<__nv_bfloat16 *>(out);
         cudaError_t e = launch_decode(cs.head_dim, G, fp8, p, *cs.pool_map, st);
         if (e != cudaSuccess) return reject(KVG_ERR_CUDA, std::string("decode launch: ") + cudaGetErrorString(e));
-        e = launch_combine(cs.head_dim, G, p, st);
+        e = launch_combine(cs.head_dim, p, cs.n_sm, st);
         if (e != cudaSuccess) return reject(KVG_ERR_CUDA, std::string("combine launch: ") + cudaGetErrorString(e));
     }
     return KVG_OK;

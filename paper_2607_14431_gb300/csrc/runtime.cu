@@ -2226,7 +2226,7 @@ static kvg_status decode_impl(const char *what, kvg_cache *c, int32_t layer, con
         p.state = state;
         p.state_merge = merge;
         KVG_CUDA(launch_decode(d.head_dim, G, fp8, p, c->pool_map, st));
-        KVG_CUDA(launch_combine(d.head_dim, G, p, st));
+        KVG_CUDA(launch_combine(d.head_dim, p, c->n_sm, st));
     }
     KVG_CUDA(cudaEventRecord(c->part_ev, st));
     c->part_stream = st;
