@@ -399,9 +399,11 @@ kvg_status kvg_graft_chunked(kvg_store *store, uint64_t block_id, kvg_cache *cac
  * grafted (KVG_ERR_POSITION when tags + delta leave [0, 2^31), KVG_ERR_ARG
  * for a nonzero delta on an fp8 cache).  Not for pool-resident stores
  * (KVG_ERR_ARG; use kvg_graft).  flags as for kvg_graft: KVG_GRAFT_VERIFY
- * hashes each own-position graft's pages as it copies them, and each
- * re-based graft's stored pages after the copies; the report's seq is the (last)
- * failing graft's sequence and mismatch_pages its block page indices.  The
+ * hashes each own-position graft's pages as it copies them (from a
+ * pinned-host store: once they are in the cache), and each re-based graft's
+ * pages as the store has them, before the rotating copy (pinned host: after
+ * it), which reads them again; the report's seq is the (last) failing
+ * graft's sequence and mismatch_pages its block page indices.  The
  * call stages its job table in library-owned pinned memory and waits for
  * the previous batch's table copy on this cache before reusing it; on the GPU
  * a batch on another stream than the cache's previous one runs after it (they
